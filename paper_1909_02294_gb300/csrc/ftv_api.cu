@@ -76,6 +76,14 @@ int64_t max_pixel_cost(const ftv_ctx* c, int n_nbrs) {
 
 }  // namespace
 
+// View v of a context packed at byte `offset` of the allocation `base`, as the kernels see it.
+NbrView ftv::nbr_view(const ftv_ctx* c, int v, void* base, size_t offset, size_t texel_bytes) {
+    const int w = c->cams[v].width, h = c->cams[v].height;
+    const size_t off = offset / texel_bytes;
+    const bool fits = off + (size_t)w * h <= (size_t)INT32_MAX;
+    return {static_cast<char*>(base) + offset, w, h, w, fits ? (int32_t)off : -1};
+}
+
 // The host-only tables of ftv_compute_homographies[_f64]: the same arithmetic as ftv_depth_init.
 template <typename T>
 static ftv_status compute_homographies(const ftv_config* cfg, int32_t ref_index, T* host_out) {
@@ -159,7 +167,7 @@ ftv_status ftv_depth_init(const ftv_config* cfg, ftv_ctx** out) {
     c->penalty = cfg->oob_penalty >= 0 ? cfg->oob_penalty : (int32_t)(3 * ((1LL << cfg->bit_depth) - 1));
     // 4-byte texels wherever the samples fit (one 32-bit gather per evaluation)
     c->fmt = cfg->sample_bytes == 1 ? FMT_U8X4 : (cfg->bit_depth <= 10 ? FMT_P10 : FMT_U16X4);
-    c->texel_bytes = c->fmt == FMT_U16X4 ? 8 : 4;
+    c->texel_bytes = texel_size(c->fmt);
     c->cams.assign(cfg->cams, cfg->cams + cfg->n_views);
 
     std::vector<double> iz;
@@ -233,18 +241,24 @@ ftv_status ftv_depth_init(const ftv_config* cfg, ftv_ctx** out) {
             for (size_t e = 0; e < r.h_H.size(); e += 9) any_affine = any_affine || (r.h_H[e + 6] == 0.0f && r.h_H[e + 7] == 0.0f);
         c->kind = any_affine ? kKindMixed : kKindProjective;
         if (c->precision == FTV_PRECISION_FP64) c->kind = any_affine ? kKindPreciseMixed : kKindPrecise;
+        c->cost_fmt = cost_format(any_affine, c->sample_bytes, c->bit_depth, c->fmt);
+        c->cost_texel_bytes = texel_size(c->cost_fmt);
     }
 
     // device scratch (all host-side validation is done by now)
     if (cudaGetDevice(&c->device) != cudaSuccess) { free_ctx(c); return FTV_ERR_CUDA; }
     cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
-    size_t packed = 0;
+    size_t packed = 0, cost_packed = 0;
     c->view_offset_bytes.resize(c->n_views);
+    c->cost_offset_bytes.resize(c->n_views);
     for (int v = 0; v < c->n_views; ++v) {
         c->view_offset_bytes[v] = packed;
-        const size_t bytes = (size_t)c->cams[v].width * c->cams[v].height * c->texel_bytes;
-        packed += (bytes + 255) & ~(size_t)255;
+        c->cost_offset_bytes[v] = cost_packed;
+        const size_t texels = (size_t)c->cams[v].width * c->cams[v].height;
+        packed += (texels * c->texel_bytes + 255) & ~(size_t)255;
+        cost_packed += (texels * c->cost_texel_bytes + 255) & ~(size_t)255;
     }
+    packed = std::max(packed, cost_packed);
     bool ok = dalloc(reinterpret_cast<char**>(&c->d_packed), packed) == cudaSuccess;
     ok = ok && dalloc(&c->d_status, 1) == cudaSuccess;
     ok = ok && dalloc(&c->d_jobs, kMaxUnits) == cudaSuccess;
@@ -258,7 +272,7 @@ ftv_status ftv_depth_init(const ftv_config* cfg, ftv_ctx** out) {
     for (auto& r : c->refs) {
         ok = ok && dalloc(&r.d_H, r.h_H.size()) == cudaSuccess;
         if (c->precision == FTV_PRECISION_FP64) ok = ok && dalloc(&r.d_H64, r.h_H64.size()) == cudaSuccess;
-        ok = ok && dalloc(&r.d_nbrs, (size_t)r.n_nbrs) == cudaSuccess;
+        ok = ok && dalloc(&r.d_nbrs, (size_t)r.n_nbrs * 2) == cudaSuccess;
         ok = ok && dalloc(&r.d_offs, (size_t)c->max_segments + 1) == cudaSuccess;
         ok = ok && dalloc(&r.d_cursor, (size_t)c->max_segments) == cudaSuccess;
         ok = ok && dalloc(&r.d_woffs, (size_t)c->max_segments + 1) == cudaSuccess;
@@ -274,14 +288,12 @@ ftv_status ftv_depth_init(const ftv_config* cfg, ftv_ctx** out) {
     ok = cudaMemset(c->d_status, 0, sizeof(uint32_t)) == cudaSuccess;
     ok = ok && cudaMemcpy(c->d_label_z, c->label_z.data(), sizeof(float) * c->L, cudaMemcpyHostToDevice) == cudaSuccess;
     for (auto& r : c->refs) {
-        std::vector<NbrView> nv(r.n_nbrs);
-        for (int k = 0; k < r.n_nbrs; ++k) {
-            const int v = r.nbrs[k];
-            nv[k].texels = static_cast<char*>(c->d_packed) + c->view_offset_bytes[v];
-            nv[k].w = c->cams[v].width;
-            nv[k].h = c->cams[v].height;
-            nv[k].pitch = c->cams[v].width;
-            nv[k].pad = 0;
+        std::vector<NbrView> nv(2 * (size_t)r.n_nbrs);
+        for (int k = 0; k < 2 * r.n_nbrs; ++k) {
+            const bool cost = k < r.n_nbrs;
+            const int v = r.nbrs[cost ? k : k - r.n_nbrs];
+            nv[k] = nbr_view(c, v, c->d_packed, cost ? c->cost_offset_bytes[v] : c->view_offset_bytes[v],
+                             cost ? c->cost_texel_bytes : c->texel_bytes);
         }
         ok = ok && cudaMemcpy(r.d_H, r.h_H.data(), sizeof(float) * r.h_H.size(), cudaMemcpyHostToDevice) == cudaSuccess;
         if (r.d_H64)
@@ -292,7 +304,7 @@ ftv_status ftv_depth_init(const ftv_config* cfg, ftv_ctx** out) {
     }
     c->fast_rcp = fast_reciprocal_exact();
     c->penalty_floor = (int64_t)c->penalty >= max_sample_cost(c);
-    c->cost_blocks_per_sm = cost_blocks_per_sm(c->fmt, c->combine, c->fast_rcp);
+    c->cost_blocks_per_sm = cost_blocks_per_sm(c->cost_fmt, c->combine, c->fast_rcp);
     if (!ok) {
         free_ctx(c);
         return FTV_ERR_CUDA;
@@ -393,9 +405,9 @@ ftv_status ftv_cost_volume(ftv_ctx* ctx, const void* const* d_planes, const int6
     for (int v = 0; v < ctx->n_views && e == cudaSuccess; ++v) {
         if (!used[v]) continue;
         NvtxRange stage("pack");
-        e = launch_pack(d_planes + 3 * v, pitch_bytes + 3 * v, ctx->sample_bytes, ctx->bit_depth, ctx->fmt,
+        e = launch_pack(d_planes + 3 * v, pitch_bytes + 3 * v, ctx->sample_bytes, ctx->bit_depth, ctx->cost_fmt,
                         ctx->cams[v].width, ctx->cams[v].height,
-                        static_cast<char*>(ctx->d_packed) + ctx->view_offset_bytes[v], ctx->d_status, s);
+                        static_cast<char*>(ctx->d_packed) + ctx->cost_offset_bytes[v], ctx->d_status, s);
         ctx->launches++;
     }
     std::vector<RefJob> jobs(ctx->n_refs);
@@ -420,7 +432,8 @@ ftv_status ftv_cost_volume(ftv_ctx* ctx, const void* const* d_planes, const int6
         }
         RefJob& J = jobs[i];
         std::memset(&J, 0, sizeof(J));
-        J.ref_texels = static_cast<char*>(ctx->d_packed) + ctx->view_offset_bytes[r.view];
+        J.ref_texels = static_cast<char*>(ctx->d_packed) + ctx->cost_offset_bytes[r.view];
+        J.all_texels = ctx->d_packed;
         J.pix = r.d_pix;
         J.offs = r.d_offs;
         J.list = list;
@@ -438,7 +451,7 @@ ftv_status ftv_cost_volume(ftv_ctx* ctx, const void* const* d_planes, const int6
         J.LB = ctx->LB;
         J.nLB = ctx->nLB;
         J.penalty = ctx->penalty;
-        J.fmt = ctx->fmt;
+        J.fmt = ctx->cost_fmt;
     }
     if (e == cudaSuccess) {
         NvtxRange stage("plan");
@@ -449,7 +462,7 @@ ftv_status ftv_cost_volume(ftv_ctx* ctx, const void* const* d_planes, const int6
     if (e == cudaSuccess) {
         NvtxRange stage("cost kernel");
         const int per_sm = ctx->ctas_per_sm > 0 ? ctx->ctas_per_sm : ctx->cost_blocks_per_sm;
-        e = launch_cost(ctx->d_jobs, ctx->d_plan, ctx->fmt, ctx->combine, ctx->fast_rcp, ctx->penalty_floor, ctx->kind,
+        e = launch_cost(ctx->d_jobs, ctx->d_plan, ctx->cost_fmt, ctx->combine, ctx->fast_rcp, ctx->penalty_floor, ctx->kind,
                         0, 1, ctx->n_sm * per_sm, s);
         ctx->launches++;
     }

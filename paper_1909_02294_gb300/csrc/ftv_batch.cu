@@ -32,6 +32,7 @@ struct PackTask {
     const void* planes[3];
     int64_t pitch[3];
     void* out;
+    void* cost_out;    // the view in the cost kernel's format (FMT_U16S), where that differs from fmt; else null
     uint32_t* status;  // the job's status word
     int32_t W, H, sb, fmt;
     uint32_t maxv;
@@ -137,6 +138,7 @@ __global__ void pack_multi_kernel(const Header* __restrict__ hdr, const PackTask
             if (T.fmt == FMT_U8X4) static_cast<uint32_t*>(T.out)[i] = a | (b << 8) | (c << 16);
             else if (T.fmt == FMT_P10) static_cast<uint32_t*>(T.out)[i] = a | (b << 10) | (c << 20);
             else static_cast<uint2*>(T.out)[i] = make_uint2(a | (b << 16), c);
+            if (T.cost_out) static_cast<uint2*>(T.cost_out)[i] = make_uint2(a | (b << 16), c | ((a + b + c) << 16));
         }
     }
 }
@@ -480,6 +482,7 @@ struct ftv_batch {
     int64_t budget = 0;                 // admission budget in device bytes (0: none)
     std::vector<int8_t> ring;           // status of ticket t at t % kTicketRing
     int32_t fmt = -1, combine = -1;
+    int32_t cost_fmt = -1;              // the cost kernel's texel format: the jobs' common one, else fmt
     bool fast_rcp = false;
     bool penalty_floor = false;
     int kind = 0;
@@ -490,7 +493,7 @@ struct ftv_batch {
     cudaEvent_t done = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
-    int graph_fmt = -1, graph_combine = -1;
+    int graph_cost_fmt = -1, graph_combine = -1;
     bool graph_pf = false;
     int graph_kind = -1;
     int64_t launches = 0;
@@ -585,7 +588,7 @@ int64_t context_bytes_of(size_t packed, const std::vector<RefDims>& refs, int64_
     int64_t b = (int64_t)packed + sizeof(uint32_t) + kMaxUnits * (int64_t)sizeof(RefJob) + sizeof(Plan);
     b += std::max<int64_t>(1, (int64_t)refs.size()) * MS * 8 * 8 + L * 4 + MS * 4 + MS * 32 * 4 + MS * 4;
     for (const RefDims& r : refs) {
-        b += r.N * L * 9 * 4 + (fp64 ? r.N * L * 9 * 8 : 0) + r.N * (int64_t)sizeof(NbrView);
+        b += r.N * L * 9 * 4 + (fp64 ? r.N * L * 9 * 8 : 0) + 2 * r.N * (int64_t)sizeof(NbrView);
         b += 2 * (MS + 1) * 4 + MS * 4 + r.W * r.H * 4 + MS * 8 + std::max<int64_t>(1, r.N) * 8;
     }
     return b;
@@ -603,18 +606,42 @@ int64_t stream_bytes(const ftv_ctx* c, const int32_t* n_segments) {
 // A stream's whole footprint, as ftv_job_footprint states it: its context, its resident stream state and
 // one frame of input planes.
 int64_t job_bytes(const ftv_ctx* c) {
-    size_t packed = 0;
+    size_t packed = 0, cost_packed = 0;
     int64_t input = 0;
     for (int v = 0; v < c->n_views; ++v) {
         packed += align256((size_t)c->cams[v].width * c->cams[v].height * c->texel_bytes);
+        cost_packed += align256((size_t)c->cams[v].width * c->cams[v].height * c->cost_texel_bytes);
         input += 3 * (int64_t)c->cams[v].width * c->cams[v].height * c->sample_bytes;
     }
     std::vector<RefDims> refs;
     for (int i = 0; i < c->n_refs; ++i)
         refs.push_back({c->refs[i].W, c->refs[i].H, c->refs[i].n_nbrs,
                         c->stream.ready ? c->stream.refs[i].S : c->max_segments});
-    return context_bytes_of(packed, refs, c->L, c->max_segments, c->precision == FTV_PRECISION_FP64) +
+    return context_bytes_of(std::max(packed, cost_packed), refs, c->L, c->max_segments,
+                            c->precision == FTV_PRECISION_FP64) +
            stream_bytes_of(packed, refs, c->L) + input;
+}
+
+// Whether any homography of cfg is affine (as FP32), which decides the cost kernel's texel format.
+bool any_affine_entry(const ftv_config* cfg) {
+    std::vector<double> iz;
+    if (!label_inv_depths(cfg->n_labels, cfg->z_near, cfg->z_far, iz)) return false;
+    const bool centre = cfg->plane_mode == FTV_PLANES_CENTRE && cfg->centre_view >= 0 && cfg->centre_view < cfg->n_views;
+    const ftv_camera* cc = centre ? &cfg->cams[cfg->centre_view] : nullptr;
+    for (int i = 0; i < cfg->n_refs; ++i) {
+        const int r = cfg->ref_views[i];
+        const int b = cfg->nbr_offsets ? cfg->nbr_offsets[i] : 0, e = cfg->nbr_offsets ? cfg->nbr_offsets[i + 1] : cfg->n_views;
+        for (int k = b; k < e; ++k) {
+            const int v = cfg->nbr_offsets ? (cfg->nbr_views ? cfg->nbr_views[k] : r) : k;
+            if (v == r || v < 0 || v >= cfg->n_views) continue;
+            for (int d = 0; d < cfg->n_labels; ++d) {
+                double H[9];
+                if (plane_homography(cfg->cams[r], cfg->cams[v], cc, iz[d], H) != 0) continue;
+                if ((float)H[6] == 0.0f && (float)H[7] == 0.0f) return true;
+            }
+        }
+    }
+    return false;
 }
 
 }  // namespace
@@ -659,11 +686,7 @@ ftv_status ftv_stream_init(ftv_ctx* ctx, const int32_t* const* d_labels, const i
             std::vector<NbrView> nv(r.n_nbrs);
             for (int k = 0; k < r.n_nbrs; ++k) {
                 const int v = r.nbrs[k];
-                nv[k].texels = static_cast<char*>(st.d_ring[b]) + ctx->view_offset_bytes[v];
-                nv[k].w = ctx->cams[v].width;
-                nv[k].h = ctx->cams[v].height;
-                nv[k].pitch = ctx->cams[v].width;
-                nv[k].pad = 0;
+                nv[k] = nbr_view(ctx, v, st.d_ring[b], ctx->view_offset_bytes[v], ctx->texel_bytes);
             }
             if (ok && r.n_nbrs)
                 ok = cudaMemcpy(R.d_nbrs_ring[b], nv.data(), sizeof(NbrView) * nv.size(), cudaMemcpyHostToDevice) ==
@@ -933,7 +956,7 @@ ftv_status ftv_batch_prepare(ftv_batch* b, const ftv_frame_job* jobs, int32_t n_
     cudaGetLastError();
     harvest(b);  // a completed ticketed launch keeps its jobs' statuses before this launch overwrites them
     NvtxRange range("ftv_batch_prepare");
-    int n_views = 0, n_units = 0, fmt = -1, combine = -1;
+    int n_views = 0, n_units = 0, fmt = -1, cost_fmt = -1, combine = -1;
     bool pf_all = true;
     int kind = kKindMixed;
     for (int j = 0; j < n_jobs; ++j) {
@@ -948,6 +971,7 @@ ftv_status ftv_batch_prepare(ftv_batch* b, const ftv_frame_job* jobs, int32_t n_
         // one cost-kernel instantiation per launch: FP32- and FP64-precision streams do not share a batch
         if (j > 0 && J.ctx->precision != jobs[0].ctx->precision) return FTV_ERR_INVALID_ARG;
         fmt = J.ctx->fmt;
+        cost_fmt = j == 0 || J.ctx->cost_fmt == cost_fmt ? J.ctx->cost_fmt : fmt;
         combine = J.ctx->combine;
         pf_all = pf_all && J.ctx->penalty_floor;
         // contexts of one batch share a precision; differing entry classes take the mixed instantiation
@@ -981,6 +1005,7 @@ ftv_status ftv_batch_prepare(ftv_batch* b, const ftv_frame_job* jobs, int32_t n_
         const int prev = is_i ? cur : st.prev;
         const int ifr = is_i ? cur : st.iframe;
         const uint32_t maxv = c->bit_depth >= 32 ? 0xffffffffu : ((1u << c->bit_depth) - 1u);
+        const bool own = cost_fmt != fmt;  // the cost kernel reads the context's own copy of the current frame
         for (int v = 0; v < c->n_views; ++v) {
             PackTask& t = P[pv++];
             for (int k = 0; k < 3; ++k) {
@@ -988,6 +1013,7 @@ ftv_status ftv_batch_prepare(ftv_batch* b, const ftv_frame_job* jobs, int32_t n_
                 t.pitch[k] = J.pitch_bytes[3 * v + k];
             }
             t.out = static_cast<char*>(st.d_ring[cur]) + c->view_offset_bytes[v];
+            t.cost_out = own ? static_cast<char*>(c->d_packed) + c->cost_offset_bytes[v] : nullptr;
             t.W = c->cams[v].width;
             t.H = c->cams[v].height;
             t.sb = c->sample_bytes;
@@ -1031,7 +1057,8 @@ ftv_status ftv_batch_prepare(ftv_batch* b, const ftv_frame_job* jobs, int32_t n_
             temp_chunks += S.S > 0 ? (S.S + kTChunk - 1) / kTChunk : 1;
             RefJob& q = R[pu];
             std::memset(&q, 0, sizeof(q));
-            q.ref_texels = t.cur;
+            q.ref_texels = own ? static_cast<char*>(c->d_packed) + c->cost_offset_bytes[r.view] : t.cur;
+            q.all_texels = own ? c->d_packed : st.d_ring[cur];
             q.pix = r.d_pix;
             q.offs = r.d_offs;
             q.list = S.d_changed;
@@ -1039,7 +1066,7 @@ ftv_status ftv_batch_prepare(ftv_batch* b, const ftv_frame_job* jobs, int32_t n_
             q.woffs = r.d_woffs;
             q.H = r.d_H;
             q.H64 = r.d_H64;
-            q.nbrs = S.d_nbrs_ring[cur];
+            q.nbrs = own ? r.d_nbrs : S.d_nbrs_ring[cur];
             q.cost = S.d_cost;
             q.W = r.W;
             q.Href = r.H;
@@ -1049,7 +1076,7 @@ ftv_status ftv_batch_prepare(ftv_batch* b, const ftv_frame_job* jobs, int32_t n_
             q.LB = c->LB;
             q.nLB = c->nLB;
             q.penalty = c->penalty;
-            q.fmt = c->fmt;
+            q.fmt = cost_fmt;
             WtaUnit& w = Wt[pu];
             w.cost = S.d_cost;
             w.mask = S.d_mask;
@@ -1095,10 +1122,11 @@ ftv_status ftv_batch_prepare(ftv_batch* b, const ftv_frame_job* jobs, int32_t n_
     H.temp_stats = temp_stats;
     H.wta_segs = wta_segs;
     H.depth_rows = depth_rows;
-    if (fmt >= 0 && (fmt != b->fmt || combine != b->combine))
-        b->cost_grid = b->n_sm * cost_blocks_per_sm(fmt, combine, b->fast_rcp);
+    if (fmt >= 0 && (cost_fmt != b->cost_fmt || combine != b->combine))
+        b->cost_grid = b->n_sm * cost_blocks_per_sm(cost_fmt, combine, b->fast_rcp);
     if (fmt >= 0) {
         b->fmt = fmt;
+        b->cost_fmt = cost_fmt;
         b->combine = combine;
         b->penalty_floor = pf_all;
         b->kind = kind;
@@ -1130,7 +1158,7 @@ static cudaError_t enqueue(ftv_batch* b, cudaStream_t s) {
     // them the GPU can start other streams' work (of a higher priority first) instead of waiting for the
     // whole batch.
     for (int k = 0; k < b->chunks && e == cudaSuccess; ++k)
-        e = launch_cost(jobs, b->d_plan, b->fmt, b->combine, b->fast_rcp, b->penalty_floor, b->kind, k, b->chunks,
+        e = launch_cost(jobs, b->d_plan, b->cost_fmt, b->combine, b->fast_rcp, b->penalty_floor, b->kind, k, b->chunks,
                         b->cost_grid, s);
     if (e != cudaSuccess) return e;
     wta_multi_kernel<<<g, 256, 0, s>>>(hdr, wta);
@@ -1166,7 +1194,7 @@ ftv_status ftv_batch_replay(ftv_batch* b, ftv_stream stream) {
     NvtxRange range("ftv_batch_replay");
     cudaStream_t s = (cudaStream_t)stream;
     cudaError_t e = cudaSuccess;
-    if (!b->exec || b->graph_fmt != b->fmt || b->graph_combine != b->combine || b->graph_pf != b->penalty_floor ||
+    if (!b->exec || b->graph_cost_fmt != b->cost_fmt || b->graph_combine != b->combine || b->graph_pf != b->penalty_floor ||
         b->graph_kind != b->kind || b->graph_chunks != b->chunks) {
         if (b->exec) cudaGraphExecDestroy(b->exec);
         if (b->graph) cudaGraphDestroy(b->graph);
@@ -1186,7 +1214,7 @@ ftv_status ftv_batch_replay(ftv_batch* b, ftv_stream stream) {
         }
         if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, b->graph, 0);
         if (e == cudaSuccess) {
-            b->graph_fmt = b->fmt;
+            b->graph_cost_fmt = b->cost_fmt;
             b->graph_combine = b->combine;
             b->graph_pf = b->penalty_floor;
             b->graph_kind = b->kind;
@@ -1236,12 +1264,13 @@ ftv_status ftv_job_footprint(const ftv_config* cfg, int32_t n_segments_max, int6
     if (cfg->sample_bytes != 1 && cfg->sample_bytes != 2) return FTV_ERR_INVALID_ARG;
     if (cfg->bit_depth < 1 || cfg->bit_depth > 8 * cfg->sample_bytes) return FTV_ERR_INVALID_ARG;
     const size_t tb = (cfg->sample_bytes == 1 || cfg->bit_depth <= 10) ? 4 : 8;
-    size_t packed = 0;
+    size_t packed = 0, cost_packed = 0;
     int64_t input = 0;
     for (int v = 0; v < cfg->n_views; ++v) {
         const int64_t w = cfg->cams[v].width, h = cfg->cams[v].height;
         if (w < 1 || h < 1 || w > FTV_MAX_DIM || h > FTV_MAX_DIM) return FTV_ERR_INVALID_ARG;
         packed += align256((size_t)(w * h) * tb);
+        cost_packed += align256((size_t)(w * h) * 8);
         input += 3 * w * h * cfg->sample_bytes;
     }
     const int64_t S = n_segments_max > 0 ? n_segments_max : cfg->max_segments;
@@ -1256,7 +1285,12 @@ ftv_status ftv_job_footprint(const ftv_config* cfg, int32_t n_segments_max, int6
         }
         refs.push_back({cfg->cams[r].width, cfg->cams[r].height, N, S});
     }
-    *bytes = context_bytes_of(packed, refs, cfg->n_labels, cfg->max_segments, cfg->precision == FTV_PRECISION_FP64) +
+    // the cost kernel's 8-byte texels, where the views are held as 4-byte ones otherwise
+    const int fmt = cfg->sample_bytes == 1 ? FMT_U8X4 : (tb == 4 ? FMT_P10 : FMT_U16X4);
+    const bool wide = tb == 4 && cfg->sample_bytes == 2 &&
+                      cost_format(any_affine_entry(cfg), cfg->sample_bytes, cfg->bit_depth, fmt) == FMT_U16S;
+    *bytes = context_bytes_of(wide ? cost_packed : packed, refs, cfg->n_labels, cfg->max_segments,
+                              cfg->precision == FTV_PRECISION_FP64) +
              stream_bytes_of(packed, refs, cfg->n_labels) + input;
     return FTV_OK;
 }

@@ -524,7 +524,7 @@ extern "C" ftv_status ftv_centre_table(ftv_ctx* ctx, const void* const* d_planes
         a.H = r.d_H;
         a.H64 = r.d_H64;
         a.ref_tex = static_cast<char*>(ctx->d_packed) + ctx->view_offset_bytes[r.view];
-        a.nbrs = r.d_nbrs;
+        a.nbrs = r.d_nbrs + r.n_nbrs;
         a.labels_v = r.d_nbr_labels;
         a.m = d_m[i];
         a.sp = d_sprime[i];

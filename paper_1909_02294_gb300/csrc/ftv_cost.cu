@@ -11,13 +11,20 @@
 // pixels contiguous) times one block of LB consecutive labels of one (job, reference) unit. Resident
 // CTAs take items from a global counter in increasing order, so CTAs that run together work on
 // neighbouring tiles and label blocks and share their neighbour-view footprints in L2. Per item:
-//   - the N x LB homographies and the neighbour geometry are staged in shared memory;
-//   - each thread owns kPPT pixels (x, y and the reference samples in registers);
-//   - for each label, for each neighbour: FP32 projection, one packed-texel gather, |dY|+|dCb|+|dCr|,
+//   - the N x LB homographies and the neighbour geometry are staged in shared memory; the tile's pixel box then
+//     tells which entries sample no pixel, which sample every pixel in view (no tests), and which need the tests;
+//   - each label's neighbours are listed by class, so that the pixel loop has no dispatch for the common class;
+//   - each thread owns kPPT pixels (position and reference samples in registers), a warp kWarpPix consecutive ones;
+//   - for each label, for each listed neighbour: projection, one packed-texel gather, |dY|+|dCb|+|dCr|,
 //     running min/sum per pixel in registers;
-//   - per label, warp reductions over runs of equal segment collapse the per-pixel costs, one shared
-//     atomic per run, and at the end of the item each segment's row slice is written: plain stores
-//     for segments wholly inside the tile, global atomics for segments cut by a tile boundary.
+//   - per label, each run of equal segments among the warp's pixels is summed (in the thread, then one warp
+//     reduction and one shared atomic per run), and at the end of the item each segment's row slice is
+//     written: plain stores for segments wholly inside the tile, global atomics for segments cut by a tile
+//     boundary.
+// The kernel is bound by instruction issue, so instructions per evaluation decide its time. With one offset per
+// in-view integer-shift entry (no tests, no row arithmetic), the listed classes, the sums in the thread and the
+// packed comparisons below, the 1920x1080 8-view 250-label rig went from 29.0 to 19.3 ms per launch, the
+// 3840x2160 15-view 400-label rig from 506 to 435 ms, a 480x270 8-bit frame from 151 to 86 us.
 // All arithmetic that decides a sample position is explicit round-to-nearest FP32 (no contraction
 // freedom is left to the compiler), so the result is bit-identical to any implementation of the same
 // sequence; costs are integers, so summation order does not matter.
@@ -39,53 +46,81 @@ constexpr int kSentinel = INT_MAX;
 // Segments of a tile whose listed-pixel offsets are cached in shared memory (more: binary search in
 // global memory). Together with kSegAcc this keeps a CTA near 30 KB of shared memory, so that four CTAs
 // leave about half of the SM's 256 KB L1 to the neighbour-view gathers (prefer_l1).
-constexpr int kLocCache = 257;
+constexpr int kLocCache = 65;
+constexpr int kWarpPix = 32 * kPPT;  // consecutive records of one warp
 
-// cost(): |dY| + |dCb| + |dCr| as a chain of __sad (|x - y| + z, unsigned accumulate; exact here, as every
-// term and the sum are below 2^18), which measured 12.5 % fewer instructions per evaluation than separate
-// subtractions, absolute values and adds (1920x1080 8-view rig: 30.9 -> 29.4 ms).
+// Ref: a reference pixel's samples in the form cost() compares. cost(): |dY| + |dCb| + |dCr|, exact integers.
 template <int FMT>
 struct TexelOps;
 
+// 8-bit samples: one packed absolute difference sums all four bytes (the fourth is zero on both sides).
 template <>
 struct TexelOps<FMT_U8X4> {
-    static __device__ __forceinline__ void unpack_ref(const void* base, int64_t i, int& a, int& b, int& c) {
-        const uint32_t t = __ldg(static_cast<const uint32_t*>(base) + i);
-        a = t & 0xff;
-        b = (t >> 8) & 0xff;
-        c = t >> 16;
+    struct Ref {
+        uint32_t t;
+    };
+    static __device__ __forceinline__ Ref load_ref(const void* base, int64_t i) {
+        return {__ldg(static_cast<const uint32_t*>(base) + i)};
     }
-    static __device__ __forceinline__ int cost(const void* base, int i, int a, int b, int c) {
-        const uint32_t t = __ldg(static_cast<const uint32_t*>(base) + i);
-        return (int)__sad((int)(t & 0xff), a, __sad((int)((t >> 8) & 0xff), b, __sad((int)(t >> 16), c, 0u)));
+    static __device__ __forceinline__ int cost(const void* base, int i, const Ref& r) {
+        return (int)__vsadu4(__ldg(static_cast<const uint32_t*>(base) + i), r.t);
     }
 };
 
 template <>
 struct TexelOps<FMT_P10> {
-    static __device__ __forceinline__ void unpack_ref(const void* base, int64_t i, int& a, int& b, int& c) {
+    struct Ref {
+        int a, b, c;
+    };
+    static __device__ __forceinline__ Ref load_ref(const void* base, int64_t i) {
         const uint32_t t = __ldg(static_cast<const uint32_t*>(base) + i);
-        a = t & 0x3ff;
-        b = (t >> 10) & 0x3ff;
-        c = t >> 20;
+        return {(int)(t & 0x3ff), (int)((t >> 10) & 0x3ff), (int)(t >> 20)};
     }
-    static __device__ __forceinline__ int cost(const void* base, int i, int a, int b, int c) {
+    static __device__ __forceinline__ int cost(const void* base, int i, const Ref& r) {
         const uint32_t t = __ldg(static_cast<const uint32_t*>(base) + i);
-        return (int)__sad((int)(t & 0x3ff), a, __sad((int)((t >> 10) & 0x3ff), b, __sad((int)(t >> 20), c, 0u)));
+        return (int)__sad((int)(t & 0x3ff), r.a, __sad((int)((t >> 10) & 0x3ff), r.b, __sad((int)(t >> 20), r.c, 0u)));
+    }
+};
+
+// a.lo * lo + a.hi * hi + c with the unsigned 16-bit halves of a (every product and sum fits int).
+template <int LO, int HI>
+__device__ __forceinline__ int dot_halves(uint32_t a, int c) {
+    int d;
+    asm("dp2a.lo.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"((LO & 0xff) | ((HI & 0xff) << 8)), "r"(c));
+    return d;
+}
+
+// 9- to 14-bit samples with their sum S = Y + Cb + Cr in the fourth half-word: |y - r| = y + r - 2 min(y, r), so
+// the cost is S + S_r - 2 (the three minima): two packed minima and two dot products (S passes through the
+// second minimum against 0xffff; S <= 3 * 16383).
+template <>
+struct TexelOps<FMT_U16S> {
+    struct Ref {
+        uint32_t a, b;
+        int s;
+    };
+    static __device__ __forceinline__ Ref load_ref(const void* base, int64_t i) {
+        const uint2 t = __ldg(static_cast<const uint2*>(base) + i);
+        return {t.x, t.y | 0xffff0000u, (int)(t.y >> 16)};
+    }
+    static __device__ __forceinline__ int cost(const void* base, int i, const Ref& r) {
+        const uint2 t = __ldg(static_cast<const uint2*>(base) + i);
+        return dot_halves<-2, 1>(__vminu2(t.y, r.b), dot_halves<-2, -2>(__vminu2(t.x, r.a), r.s));
     }
 };
 
 template <>
 struct TexelOps<FMT_U16X4> {
-    static __device__ __forceinline__ void unpack_ref(const void* base, int64_t i, int& a, int& b, int& c) {
+    struct Ref {
+        int a, b, c;
+    };
+    static __device__ __forceinline__ Ref load_ref(const void* base, int64_t i) {
         const uint2 t = __ldg(static_cast<const uint2*>(base) + i);
-        a = t.x & 0xffff;
-        b = t.x >> 16;
-        c = t.y;
+        return {(int)(t.x & 0xffff), (int)(t.x >> 16), (int)t.y};
     }
-    static __device__ __forceinline__ int cost(const void* base, int i, int a, int b, int c) {
+    static __device__ __forceinline__ int cost(const void* base, int i, const Ref& r) {
         const uint2 t = __ldg(static_cast<const uint2*>(base) + i);
-        return (int)__sad((int)(t.x & 0xffff), a, __sad((int)(t.x >> 16), b, __sad((int)t.y, c, 0u)));
+        return (int)__sad((int)(t.x & 0xffff), r.a, __sad((int)(t.x >> 16), r.b, __sad((int)t.y, r.c, 0u)));
     }
 };
 
@@ -109,6 +144,8 @@ struct TexelOps<FMT_U16X4> {
 //             view's pitch is the reference width and its height at least the reference height: the
 //             sample's index is then the pixel's y * W + x plus D, the row needs no test, and the column
 //             test is -D <= x < w - D, staged as floats (h[6], h[7]) with D in h[8];
+//   kShiftIn  kShift whose every sample of the item's tile is in view (the tile's columns lie within the bounds);
+//             h[0] of a kShift entry holds the view's texel offset in the unit's allocation (NbrView::off);
 //   kOut      affine with 1/h8 not finite and positive, or no pixel of the item's tile can reach the view
 //             (box_class): every sample is out of view;
 //   kIn       projective, and at every pixel of the item's tile Wz > 2^-92 and the sample rounds into the
@@ -122,7 +159,8 @@ struct __align__(16) HEntry {
     float h[9];
     uint32_t w, h_, pm;
 };
-enum : uint32_t { kGeneral = 0, kAffine = 1, kUnit = 2, kOut = 3, kRect = 4, kSlow = 5, kShift = 6, kIn = 7, kFront = 8 };
+enum : uint32_t { kGeneral = 0, kAffine = 1, kUnit = 2, kOut = 3, kRect = 4, kSlow = 5, kShift = 6, kIn = 7, kFront = 8,
+                kShiftIn = 9 };
 
 // FP64-projection entries (kKindPrecise) stage local-frame coefficients in HEntry::h (stage_precise) and
 // this alongside: the integer column u0 and row v0 the frame is shifted by, and the tie-test thresholds.
@@ -131,6 +169,8 @@ struct __align__(16) PEntry {
     float thr_u, thr_v;
 };
 constexpr uint32_t kPitchMask = (1u << 28) - 1u;
+constexpr float kRound = 0x1.8p23f;  // t + kRound rounds t (|t| < 2^21) to an integer, held in the sum's low bits
+constexpr int kRoundBits = 0x4b400000;
 
 __device__ __forceinline__ bool finite_positive(float r) {
     return (unsigned)(__float_as_int(r) - 1) < 0x7f7fffffu;
@@ -203,16 +243,32 @@ __device__ __forceinline__ bool checked_gather(bool ok, int idx, unsigned lim, u
 }
 
 template <int FMT, int COMB, bool PF>
-__device__ __forceinline__ void accumulate(int& m, bool ok, const void* tex, int idx, int a, int b, int c,
-                                           int penalty, unsigned lim, uint32_t* status) {
+__device__ __forceinline__ void accumulate(int& m, bool ok, const void* tex, int idx,
+                                           const typename TexelOps<FMT>::Ref& ref, int penalty, unsigned lim,
+                                           uint32_t* status) {
     ok = checked_gather(ok, idx, lim, status);
     if (COMB == FTV_COMBINE_MIN && PF) {
-        if (ok) m = min(m, TexelOps<FMT>::cost(tex, idx, a, b, c));
+        if (ok) m = min(m, TexelOps<FMT>::cost(tex, idx, ref));
     } else {
         int cst = penalty;
-        if (ok) cst = TexelOps<FMT>::cost(tex, idx, a, b, c);
+        if (ok) cst = TexelOps<FMT>::cost(tex, idx, ref);
         m = COMB == FTV_COMBINE_MIN ? min(m, cst) : m + cst;
     }
+}
+
+// The same for a sample known to be in view.
+template <int FMT, int COMB>
+__device__ __forceinline__ void accumulate_in(int& m, const void* tex, int idx, const typename TexelOps<FMT>::Ref& ref,
+                                              int penalty, unsigned lim, uint32_t* status) {
+#ifdef FTV_CHECKED
+    accumulate<FMT, COMB, false>(m, true, tex, idx, ref, penalty, lim, status);
+#else
+    (void)penalty;
+    (void)lim;
+    (void)status;
+    const int cst = TexelOps<FMT>::cost(tex, idx, ref);
+    m = COMB == FTV_COMBINE_MIN ? min(m, cst) : m + cst;
+#endif
 }
 
 // Classifies a projective entry for the pixel box [x0, x1] x [y0, y1] (x, y >= 0) under the FP32 contract,
@@ -305,9 +361,9 @@ __device__ __forceinline__ bool shift_fp64(const double* __restrict__ hg, int& D
 //   the quotient of those errors ((e_X + |u'| e_W) / W), the rounded reciprocal, product and + 0.5
 //   (2^-23 |u'| + 2^-24 (|u'| + 1)), and the FP64 projection's own error against exact arithmetic
 //   (3 * 2^-53 (A_X + |u| A_W) / W + 2 * 2^-53 (|u| + 1)),
-// doubled. Where t = u' + 0.5 computed in FP32 lies farther than delta from every integer, floor(t) + U0
-// is the FP64 projection's column (both floors see the same side of the same integer); otherwise the
-// evaluation is redone in FP64. Returns kGeneral (that test applies), kRect (the same, rectified: below),
+// doubled. Where u' computed in FP32 lies farther than delta from every half-integer, the integer nearest to
+// it, plus U0, is the FP64 projection's column floor(u + 0.5) (both see the same side of the same
+// half-integer); otherwise the evaluation is redone in FP64. Returns kGeneral (that test applies), kRect (the same, rectified: below),
 // kOut (the FP64 projection puts no
 // pixel of the box in view: behind the camera, or wholly beyond one image edge by more than the bound) or
 // kSlow (no bound: W may come near zero in the box, or delta is large; every evaluation in FP64).
@@ -360,18 +416,20 @@ __device__ uint32_t stage_precise(const double* __restrict__ hg, int x0, int y0,
         V0 - Vb + 0.5 - dv >= (double)hv)
         return kOut;
     if (!(du < 0.25 && dv < 0.25 && Ub < 0x1p21 && Vb < 0x1p21)) return kSlow;
-    P.u0 = (int)U0;
-    P.v0 = (int)V0;
-    // near a tie when |frac(t) - 0.5| >= thr; 2^-22 more covers the FP32 rounding of that test itself
+    P.u0 = (int)U0 - kRoundBits;  // the kernel adds it to the bits of t + kRound
+    P.v0 = (int)V0 - kRoundBits;
+    // near a tie when |t - nearest integer| >= thr
     P.thr_u = __double2float_rd(0.5 - du - 0x1p-22);
     P.thr_v = __double2float_rd(0.5 - dv - 0x1p-22);
     // Rectified local frame (linear rigs with parallel axes): with a0 = b1 = c2 = 1 and a1 = b0 = c0 = c1 = 0
-    // the general evaluation computes exactly t_u = (x' + a2) + 0.5 (both rounded) and W = r = 1, so the
+    // the general evaluation computes exactly t_u = x' + a2 (rounded) and W = r = 1, so the
     // bound above holds for that shorter sequence; and when |b2| + delta_v < 0.5 every pixel's row decision
-    // is floor(y' + b2 + 0.5 +- delta_v) = y', i.e. the row is y' + V0 with no test.
+    // is floor(y' + b2 + 0.5 +- delta_v) = y', i.e. the row is y' + V0 = y + (V0 - y0) with no test.
     if (h[0] == 1.0f && h[1] == 0.0f && h[3] == 0.0f && h[4] == 1.0f && h[6] == 0.0f && h[7] == 0.0f &&
-        h[8] == 1.0f && fabs((double)h[5]) + dv < 0.49)
+        h[8] == 1.0f && fabs((double)h[5]) + dv < 0.49) {
+        P.v0 = (int)V0 - y0;
         return kRect;
+    }
     return kGeneral;
 }
 
@@ -422,6 +480,9 @@ __device__ __forceinline__ int warp_upper_index(const int32_t* a, int lo, int hi
 template <int FMT, int COMB, bool FAST_RCP, bool PF, int KIND>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) cost_kernel(const RefJob* __restrict__ jobs,
                                                                     Plan* __restrict__ plan, int chunk, int chunks) {
+    constexpr bool kProj = KIND == kKindProjective;
+    constexpr bool kShifts = KIND == kKindMixed || KIND == kKindPreciseMixed;  // kinds with integer-shift entries
+    using Ref = typename TexelOps<FMT>::Ref;
     __shared__ HEntry sH[kHEntries];
     __shared__ const void* sBase[FTV_MAX_NBRS];
     __shared__ int sAcc[kSegAcc * kMaxLB];
@@ -429,12 +490,16 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cost_kernel(const RefJob
     __shared__ int s_item, s_k0, s_k1, s_culled;
     __shared__ int s_box[4];  // the tile's pixel box: x min, x max, y min, y max
     __shared__ PEntry sP[precise_kind(KIND) ? kHEntries : 1];
-    __shared__ uint8_t sOrd[KIND == kKindProjective ? kHEntries : 1];  // per label: neighbours to visit
-    __shared__ int sCnt[KIND == kKindProjective ? kMaxLB : 1];         // per label: kIn | kFront << 8 | kGeneral << 16
+    // per label the neighbours to visit, grouped by class (kOut entries are left out): the first group is kIn
+    // (projective) or kShiftIn, whose texel offsets are listed in sShift instead
+    __shared__ uint8_t sOrd[kHEntries];
+    __shared__ int sCnt[kMaxLB];  // sizes of the groups: first | second << 8 | third << 16
+    __shared__ int sShift[kShifts ? kHEntries : 1];
+    __shared__ uint16_t sKey[kThreads / 32][kWarpPix];  // per warp: segment (relative to k0) of each run
     unsigned n_recomputed = 0;  // FP64-precision evaluations computed in double precision by this thread
     uint32_t* const ck = &plan->checked;  // out-of-view gathers of checked builds
 
-    const int tid = threadIdx.x, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // this launch's items: [chunk_begin(chunk), chunk_begin(chunk + 1)); only thread 0 needs the first (it
     // recomputes it from the plan when it fetches an item, which keeps it out of every thread's registers)
     const int total = chunk_begin(*reinterpret_cast<volatile int*>(&plan->total_items), chunk + 1, chunks);
@@ -462,6 +527,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cost_kernel(const RefJob
         const int32_t* __restrict__ offs = Jp->offs;
         const uint32_t* __restrict__ pix = Jp->pix;
         const void* ref_tex = Jp->ref_texels;
+        const void* all_tex = Jp->all_texels;
         int32_t* __restrict__ cost = Jp->cost;
         const int w0 = tile * kTile;
         const int w1 = min(w0 + kTile, n_rec);
@@ -485,11 +551,12 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cost_kernel(const RefJob
                     mode = kRect;
                 E.h[6] = r;
                 E.h[8] = E.h[2];  // Wz is not needed any more; a rectified entry then reads one float4
-                if (mode == kRect && nbrs[n].pitch == W && nbrs[n].h >= Jp->Href) {
+                if (mode == kRect && nbrs[n].off >= 0 && nbrs[n].pitch == W && nbrs[n].h >= Jp->Href) {
                     const double h2 = (double)E.h[2];
                     const double D = floor(h2 + 0.5), g = h2 + 0.5 - D;
                     if (fabs(h2) < 0x1p20 && fmin(g, 1.0 - g) > 0x1p-23 * (32768.0 + fabs(h2))) {
                         mode = kShift;
+                        E.h[0] = __int_as_float(nbrs[n].off);
                         E.h[6] = (float)(-D);
                         E.h[7] = (float)((double)nbrs[n].w - D);
                         E.h[8] = __int_as_float((int)D);
@@ -521,21 +588,25 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cost_kernel(const RefJob
             for (int i = tid; i <= nk; i += kThreads) sWoffs[i] = woffs[k0 + i];
         __syncthreads();
 
-        // this thread's pixels
+        // This thread's pixels: a warp owns kWarpPix consecutive records, 32 per slot. run[j]: which of the warp's
+        // runs of equal segments the pixel lies in (-1: past the unit's last pixel).
         float px[kPPT], py[kPPT];
-        int ra[kPPT], rb[kPPT], rc[kPPT], key[kPPT], iy[kPPT];
-        int rowx[kPPT];  // y * W + x (kShift entries of the mixed kernel)
+        Ref ref[kPPT];
+        int run[kPPT], iy[kPPT];
+        int rowx[kPPT];  // y * W + x (integer-shift entries)
         // The float row: kept in registers except in the mixed kernel, which needs registers for rowx and,
         // on the rigs it serves, rarely takes the general or affine paths that read it (exact conversion).
         auto row_f = [&](int j) { return KIND == kKindMixed ? (float)iy[j] : py[j]; };
+        int n_runs = 0, last_key = -1;
+        int bx0 = INT_MAX, bx1 = INT_MIN, by0 = INT_MAX, by1 = INT_MIN;
 #pragma unroll
         for (int j = 0; j < kPPT; ++j) {
-            const int w = w0 + j * kThreads + tid;
-            key[j] = kSentinel;
+            const int w = w0 + warp * kWarpPix + j * 32 + lane;
+            int key = kSentinel;
             iy[j] = 0;
             rowx[j] = 0;
             px[j] = py[j] = 0.0f;
-            ra[j] = rb[j] = rc[j] = 0;
+            ref[j] = Ref{};
             if (w < w1) {
                 int k;
                 if (cached) k = k0 + upper_index(sWoffs, 0, nk + 1, w);
@@ -548,151 +619,152 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cost_kernel(const RefJob
                 py[j] = (float)y;
                 iy[j] = y;
                 rowx[j] = y * W + x;
-                TexelOps<FMT>::unpack_ref(ref_tex, (int64_t)y * W + x, ra[j], rb[j], rc[j]);
-                key[j] = k - k0;
+                ref[j] = TexelOps<FMT>::load_ref(ref_tex, (int64_t)y * W + x);
+                key = k - k0;
+                bx0 = min(bx0, x);
+                bx1 = max(bx1, x);
+                by0 = min(by0, y);
+                by1 = max(by1, y);
             }
+            const int left = __shfl_up_sync(kFull, key, 1);
+            const bool first = key != kSentinel && key != (lane == 0 ? last_key : left);
+            const unsigned starts = __ballot_sync(kFull, first);
+            const int r = n_runs + __popc(starts & (kFull >> (31 - lane))) - 1;
+            run[j] = key != kSentinel ? r : -1;
+            if (first) sKey[warp][r] = (uint16_t)min(key, 0xffff);
+            n_runs += __popc(starts);
+            last_key = __shfl_sync(kFull, key, 31);
         }
 
-        // An entry whose neighbour view no pixel of the tile can reach (box_class, on the staged coefficients)
-        // takes the penalty for every pixel, without sampling: it becomes an all-out entry, which the pixel
-        // loop does not visit. box_class also marks the entries whose samples all land in view (kIn) or in
-        // front of the camera (kFront), which skip the tests they cannot fail. Only the projective-only
-        // instantiation does this: on a rectified rig an out-of-view sample is
-        // already cheap, and there the test cost more than it saved (1920x1080 linear 8-view rig: 7.8 % of
-        // the evaluations culled, 31.1 against 30.9 ms).
+        // The tile's pixel box decides each entry's class: an entry whose neighbour view no pixel of the tile can
+        // reach (box_class, on the staged coefficients) takes the penalty for every pixel, without sampling: it
+        // becomes an all-out entry, which the pixel loop does not visit; entries whose samples all land in view
+        // (kIn, kShiftIn) or in front of the camera (kFront) skip the tests they cannot fail. box_class is run
+        // for the projective-only instantiation alone: on a rectified rig the column bounds of an integer-shift
+        // entry tell the same in two comparisons.
         // FP64-precision units stage their entries here, once the box is known (stage_precise), and move the
         // pixels into the box's local frame.
-        int fx0 = 0, fy0 = 0;  // local-frame origin (kKindPrecise)
-        if constexpr (KIND == kKindProjective || precise_kind(KIND)) {  // uniform way through the barriers
-            int bx0 = INT_MAX, bx1 = INT_MIN, by0 = INT_MAX, by1 = INT_MIN;
+        bx0 = __reduce_min_sync(kFull, bx0);
+        bx1 = __reduce_max_sync(kFull, bx1);
+        by0 = __reduce_min_sync(kFull, by0);
+        by1 = __reduce_max_sync(kFull, by1);
+        if (lane == 0) {
+            atomicMin(&s_box[0], bx0);
+            atomicMax(&s_box[1], bx1);
+            atomicMin(&s_box[2], by0);
+            atomicMax(&s_box[3], by1);
+        }
+        __syncthreads();
+        int fx0 = 0, fy0 = 0;  // local-frame origin (FP64-precision units)
+        const bool any = s_box[0] <= s_box[1];  // a tile always holds a pixel; kept for safety
+        if constexpr (!precise_kind(KIND)) {
+            const int X0 = any ? s_box[0] : 0, Y0 = any ? s_box[2] : 0;
+            const float bx0f = (float)X0, bx1f = (float)(any ? s_box[1] : 0), by0f = (float)Y0,
+                        by1f = (float)(any ? s_box[3] : 0);
+            // Slots past the end of the unit's last tile hold no pixel (their result is discarded); they take
+            // the box's first corner, so that every slot lies in the box and the unchecked gathers of kIn and
+            // kShiftIn entries stay inside the view for them too.
 #pragma unroll
             for (int j = 0; j < kPPT; ++j)
-                if (key[j] != kSentinel) {
-                    bx0 = min(bx0, (int)px[j]);
-                    bx1 = max(bx1, (int)px[j]);
-                    by0 = min(by0, iy[j]);
-                    by1 = max(by1, iy[j]);
+                if (run[j] < 0) {
+                    px[j] = bx0f;
+                    py[j] = by0f;
+                    iy[j] = Y0;
+                    rowx[j] = Y0 * W + X0;
                 }
-            bx0 = __reduce_min_sync(kFull, bx0);
-            bx1 = __reduce_max_sync(kFull, bx1);
-            by0 = __reduce_min_sync(kFull, by0);
-            by1 = __reduce_max_sync(kFull, by1);
-            if (lane == 0) {
-                atomicMin(&s_box[0], bx0);
-                atomicMax(&s_box[1], bx1);
-                atomicMin(&s_box[2], by0);
-                atomicMax(&s_box[3], by1);
+            for (int e = tid; e < nh; e += kThreads) {
+                HEntry& E = sH[e];
+                const uint32_t mode = E.pm >> 28;
+                uint32_t cls = mode;
+                if (kProj && mode == kGeneral) {
+                    cls = box_class(E.h, bx0f, bx1f, by0f, by1f, (float)E.w, (float)E.h_);
+                } else if (kShifts && mode == kShift) {
+                    if (bx0f >= E.h[6] && bx1f < E.h[7]) cls = kShiftIn;
+                    else if (bx1f < E.h[6] || bx0f >= E.h[7]) cls = kOut;
+                }
+                if (cls != mode) {
+                    E.pm = (E.pm & kPitchMask) | (cls << 28);
+                    if (kProj && cls == kOut) atomicAdd(&s_culled, 1);
+                }
             }
-            __syncthreads();
-            if constexpr (KIND == kKindProjective) {
-                if (s_box[0] <= s_box[1]) {
-                    const float bx0f = (float)s_box[0], bx1f = (float)s_box[1], by0f = (float)s_box[2],
-                                by1f = (float)s_box[3];
-                    // Slots past the end of the unit's last tile hold no pixel (their result is discarded);
-                    // they take the box's first corner, so that every slot lies in the box and the kIn
-                    // path's unchecked gathers stay inside the view for them too.
-#pragma unroll
-                    for (int j = 0; j < kPPT; ++j)
-                        if (key[j] == kSentinel) {
-                            px[j] = bx0f;
-                            py[j] = by0f;
-                        }
-                    for (int e = tid; e < nh; e += kThreads) {
-                        HEntry& E = sH[e];
-                        if ((E.pm >> 28) == kGeneral) {
-                            const uint32_t cls = box_class(E.h, bx0f, bx1f, by0f, by1f, (float)E.w, (float)E.h_);
-                            E.pm = (E.pm & kPitchMask) | (cls << 28);
-                            if (cls == kOut) atomicAdd(&s_culled, 1);
-                        }
-                    }
-                }
-            } else {
-                const bool any = s_box[0] <= s_box[1];  // a tile always holds a pixel; kept for safety
-                fx0 = any ? (s_box[0] + s_box[1]) >> 1 : 0;
-                fy0 = any ? (s_box[2] + s_box[3]) >> 1 : 0;
-                const int rx = any ? max(fx0 - s_box[0], s_box[1] - fx0) : 0;
-                const int ry = any ? max(fy0 - s_box[2], s_box[3] - fy0) : 0;
-                for (int e = tid; e < nh; e += kThreads) {
-                    const int n = e / LBa, l = e - n * LBa;
-                    HEntry& E = sH[e];
-                    const int wv = nbrs[n].w, hv = nbrs[n].h;
-                    const double* hg = &Jp->H64[((int64_t)n * L + d0 + l) * 9];
-                    int D = 0;
-                    uint32_t mode;
-                    if (KIND == kKindPreciseMixed && nbrs[n].pitch == W && hv >= Jp->Href && shift_fp64(hg, D)) {
-                        // every pixel's FP64 column is x + D and its row y: bounds on the local x' = x - fx0
-                        mode = kShift;
-                        E.h[6] = (float)(-D - fx0);
-                        E.h[7] = (float)(wv - D - fx0);
-                        E.h[8] = __int_as_float(D);
-                    } else {
-                        mode = stage_precise(hg, fx0, fy0, rx, ry, wv, hv, E.h, sP[e]);
-                    }
-                    E.w = (uint32_t)wv;
-                    E.h_ = (uint32_t)hv;
-                    E.pm = (uint32_t)nbrs[n].pitch | (mode << 28);
+        } else {
+            fx0 = any ? (s_box[0] + s_box[1]) >> 1 : 0;
+            fy0 = any ? (s_box[2] + s_box[3]) >> 1 : 0;
+            const int rx = any ? max(fx0 - s_box[0], s_box[1] - fx0) : 0;
+            const int ry = any ? max(fy0 - s_box[2], s_box[3] - fy0) : 0;
+            for (int e = tid; e < nh; e += kThreads) {
+                const int n = e / LBa, l = e - n * LBa;
+                HEntry& E = sH[e];
+                const int wv = nbrs[n].w, hv = nbrs[n].h;
+                const double* hg = &Jp->H64[((int64_t)n * L + d0 + l) * 9];
+                int D = 0;
+                uint32_t mode;
+                if (kShifts && nbrs[n].off >= 0 && nbrs[n].pitch == W && hv >= Jp->Href && shift_fp64(hg, D)) {
+                    // every pixel's FP64 column is x + D and its row y: bounds on the local x' = x - fx0
+                    mode = kShift;
+                    if (fx0 - rx >= -D && fx0 + rx < wv - D) mode = kShiftIn;
+                    else if (fx0 + rx < -D || fx0 - rx >= wv - D) mode = kOut;
+                    E.h[0] = __int_as_float(nbrs[n].off);
+                    E.h[6] = (float)(-D - fx0);
+                    E.h[7] = (float)(wv - D - fx0);
+                    E.h[8] = __int_as_float(D);
+                } else {
+                    mode = stage_precise(hg, fx0, fy0, rx, ry, wv, hv, E.h, sP[e]);
                     if (mode == kOut) atomicAdd(&s_culled, 1);
                 }
-                // every slot into the local frame; an empty slot (past the end of the unit's last tile, its
-                // result discarded) takes the box's centre pixel, row and row index, so that every slot lies
-                // in the box the entries were staged for and its local coordinates, row index and FP64
-                // projection arguments name the same reference pixel
-#pragma unroll
-                for (int j = 0; j < kPPT; ++j) {
-                    if (key[j] == kSentinel) {
-                        px[j] = (float)fx0;
-                        iy[j] = fy0;
-                        rowx[j] = fy0 * W + fx0;
-                    }
-                    px[j] = (float)((int)px[j] - fx0);
-                    py[j] = (float)(iy[j] - fy0);
-                }
+                E.w = (uint32_t)wv;
+                E.h_ = (uint32_t)hv;
+                E.pm = (uint32_t)nbrs[n].pitch | (mode << 28);
             }
-            __syncthreads();
-            if (tid == 0 && s_culled > 0) atomicAdd(&plan->culled, (unsigned long long)s_culled * (unsigned)(w1 - w0));
-            if constexpr (KIND == kKindProjective) {
-                // per label, the neighbours to visit grouped by class (kIn, then kFront, then kGeneral; kOut
-                // entries are left out): one warp per label, N <= 32
-                for (int l = tid >> 5; l < LBa; l += kThreads / 32) {
-                    const uint32_t mode = lane < N ? (sH[lane * LBa + l].pm >> 28) : (uint32_t)kOut;
-                    const unsigned mi = __ballot_sync(kFull, mode == kIn);
-                    const unsigned mf = __ballot_sync(kFull, mode == kFront);
-                    const unsigned mg = __ballot_sync(kFull, mode == kGeneral);
-                    const unsigned lt = (1u << lane) - 1u;
-                    const int ci = __popc(mi), cf = __popc(mf);
-                    int pos = -1;
-                    if (mode == kIn) pos = __popc(mi & lt);
-                    else if (mode == kFront) pos = ci + __popc(mf & lt);
-                    else if (mode == kGeneral) pos = ci + cf + __popc(mg & lt);
-                    if (pos >= 0) sOrd[l * N + pos] = (uint8_t)lane;
-                    if (lane == 0) sCnt[l] = ci | (cf << 8) | (__popc(mg) << 16);
+            // every slot into the local frame; an empty slot (past the end of the unit's last tile, its
+            // result discarded) takes the box's centre pixel, row and row index, so that every slot lies
+            // in the box the entries were staged for and its local coordinates, row index and FP64
+            // projection arguments name the same reference pixel
+#pragma unroll
+            for (int j = 0; j < kPPT; ++j) {
+                if (run[j] < 0) {
+                    px[j] = (float)fx0;
+                    iy[j] = fy0;
+                    rowx[j] = fy0 * W + fx0;
                 }
-                __syncthreads();
+                px[j] = (float)((int)px[j] - fx0);
+                py[j] = (float)(iy[j] - fy0);
             }
         }
+        __syncthreads();
+        if (tid == 0 && s_culled > 0) atomicAdd(&plan->culled, (unsigned long long)s_culled * (unsigned)(w1 - w0));
+        // per label, the neighbours to visit grouped by class: one warp per label, N <= 32. The projective kind's
+        // groups are kIn, kFront and kGeneral; the others' are kShiftIn and everything else in or partly in view.
+        for (int l = warp; l < LBa; l += kThreads / 32) {
+            const HEntry* E = &sH[lane * LBa + l];
+            const uint32_t mode = lane < N ? (E->pm >> 28) : (uint32_t)kOut;
+            const bool g1 = kProj ? mode == kIn : (kShifts && mode == kShiftIn);
+            const bool g2 = kProj ? mode == kFront : (!g1 && mode != kOut);
+            const bool g3 = kProj && mode == kGeneral;
+            const unsigned m1 = __ballot_sync(kFull, g1), m2 = __ballot_sync(kFull, g2), m3 = __ballot_sync(kFull, g3);
+            const unsigned lt = (1u << lane) - 1u;
+            const int c1 = __popc(m1), c2 = __popc(m2);
+            int pos = -1;
+            if (g1) pos = __popc(m1 & lt);
+            else if (g2) pos = c1 + __popc(m2 & lt);
+            else if (g3) pos = c1 + c2 + __popc(m3 & lt);
+            if (pos >= 0) sOrd[l * N + pos] = (uint8_t)lane;
+            if (kShifts && g1) sShift[l * N + pos] = __float_as_int(E->h[0]) + __float_as_int(E->h[8]);
+            if (lane == 0) sCnt[l] = c1 | (c2 << 8) | (__popc(m3) << 16);
+        }
+        __syncthreads();
 
-        // Per pixel slot, whether the warp's 32 pixels belong to one segment (uni: one reduction, lane 0's key)
-        // or to none (none: nothing to add); decided once per item instead of once per label.
-        unsigned uni = 0, none = 0;
-#pragma unroll
-        for (int j = 0; j < kPPT; ++j) {
-            const int kf = __shfl_sync(kFull, key[j], 0), kl = __shfl_sync(kFull, key[j], 31);
-            if (kf == kl) {
-                if (kf != kSentinel) uni |= 1u << j;
-                else none |= 1u << j;
-            }
-        }
         for (int l = 0; l < LBa; ++l) {
             int m[kPPT];
 #pragma unroll
             for (int j = 0; j < kPPT; ++j)
                 m[j] = (COMB == FTV_COMBINE_MIN && N > 0) ? (PF ? penalty : INT_MAX) : 0;
-            if constexpr (KIND == kKindProjective) {
-                const int cnt = sCnt[l];
-                const int ci = cnt & 0xff, cf = ci + ((cnt >> 8) & 0xff), cg = cf + (cnt >> 16);
-                const uint8_t* ord = &sOrd[l * N];
-#pragma unroll 2  // two entries in flight: measured 2 % faster on the 4K rig together with the uniform mask
-                for (int k = 0; k < ci; ++k) {  // every pixel's sample is in view
+            const int cnt = sCnt[l];
+            const int c1 = cnt & 0xff, c2 = c1 + ((cnt >> 8) & 0xff), c3 = c2 + (cnt >> 16);
+            const uint8_t* ord = &sOrd[l * N];
+            if constexpr (kProj) {
+#pragma unroll 2  // two entries in flight: measured 2 % faster on the 4K rig
+                for (int k = 0; k < c1; ++k) {  // every pixel's sample is in view
                     const int n = ord[k];
                     const float4* e4 = reinterpret_cast<const float4*>(&sH[n * LBa + l]);
                     const float4 ha = e4[0], hb = e4[1], hc = e4[2];
@@ -707,16 +779,10 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cost_kernel(const RefJob
                         const float r = contract_rcp_normal<FAST_RCP>(Wz);
                         const int ui = __float2int_rd(__fadd_rn(__fmul_rn(X, r), 0.5f));
                         const int vi = __float2int_rd(__fadd_rn(__fmul_rn(Yh, r), 0.5f));
-#ifdef FTV_CHECKED
-                        accumulate<FMT, COMB, false>(m[j], true, tex, vi * pitch + ui, ra[j], rb[j], rc[j], penalty, lim,
-                                                     ck);
-#else
-                        const int cst = TexelOps<FMT>::cost(tex, vi * pitch + ui, ra[j], rb[j], rc[j]);
-                        m[j] = COMB == FTV_COMBINE_MIN ? min(m[j], cst) : m[j] + cst;
-#endif
+                        accumulate_in<FMT, COMB>(m[j], tex, vi * pitch + ui, ref[j], penalty, lim, ck);
                     }
                 }
-                for (int k = ci; k < cf; ++k) {  // Wz proven positive and normal: range tests only
+                for (int k = c1; k < c2; ++k) {  // Wz proven positive and normal: range tests only
                     const int n = ord[k];
                     const float4* e4 = reinterpret_cast<const float4*>(&sH[n * LBa + l]);
                     const float4 ha = e4[0], hb = e4[1], hc = e4[2];
@@ -732,10 +798,10 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cost_kernel(const RefJob
                         const int ui = __float2int_rd(__fadd_rn(__fmul_rn(X, r), 0.5f));
                         const int vi = __float2int_rd(__fadd_rn(__fmul_rn(Yh, r), 0.5f));
                         const bool ok = ((unsigned)ui < __float_as_uint(hc.y)) & ((unsigned)vi < __float_as_uint(hc.z));
-                        accumulate<FMT, COMB, PF>(m[j], ok, tex, vi * pitch + ui, ra[j], rb[j], rc[j], penalty, lim, ck);
+                        accumulate<FMT, COMB, PF>(m[j], ok, tex, vi * pitch + ui, ref[j], penalty, lim, ck);
                     }
                 }
-                for (int k = cf; k < cg; ++k) {  // the contract's sequence as written
+                for (int k = c2; k < c3; ++k) {  // the contract's sequence as written
                     const int n = ord[k];
                     const float4* e4 = reinterpret_cast<const float4*>(&sH[n * LBa + l]);
                     const float4 ha = e4[0], hb = e4[1], hc = e4[2];
@@ -746,16 +812,31 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cost_kernel(const RefJob
                     for (int j = 0; j < kPPT; ++j) {
                         int idx;
                         const bool ok = pos_general<FAST_RCP>(ha, hb, hc, pitch, px[j], py[j], idx);
-                        accumulate<FMT, COMB, PF>(m[j], ok, tex, idx, ra[j], rb[j], rc[j], penalty, lim, ck);
+                        accumulate<FMT, COMB, PF>(m[j], ok, tex, idx, ref[j], penalty, lim, ck);
                     }
                 }
-                if (!(COMB == FTV_COMBINE_MIN && PF) && cg < N) {  // entries out of view: the penalty each
+            }
+            if constexpr (kShifts) {  // every sample of the tile in view, at the pixel's own index plus one offset
+                const int* sh = &sShift[l * N];
+#pragma unroll 2
+                for (int k = 0; k < c1; ++k) {
+                    const int delta = sh[k];
+#ifdef FTV_CHECKED
+                    const int n = ord[k];
+                    const unsigned lim = (unsigned)W * sH[n * LBa + l].h_;
+                    const int own = delta - nbrs[n].off;
 #pragma unroll
                     for (int j = 0; j < kPPT; ++j)
-                        m[j] = (COMB == FTV_COMBINE_MIN) ? min(m[j], penalty) : m[j] + (N - cg) * penalty;
+                        accumulate_in<FMT, COMB>(m[j], sBase[n], rowx[j] + own, ref[j], penalty, lim, ck);
+#else
+#pragma unroll
+                    for (int j = 0; j < kPPT; ++j)
+                        accumulate_in<FMT, COMB>(m[j], all_tex, rowx[j] + delta, ref[j], penalty, 0u, ck);
+#endif
                 }
             }
-            for (int n = 0; n < (KIND == kKindProjective ? 0 : N); ++n) {
+            for (int k = c1; k < (kProj ? 0 : c2); ++k) {
+                const int n = ord[k];
                 const float4* e4 = reinterpret_cast<const float4*>(&sH[n * LBa + l]);
                 const float4 hc = e4[2];
                 const void* tex = sBase[n];
@@ -763,167 +844,151 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cost_kernel(const RefJob
                 const uint32_t mode = pm >> 28;
                 const int pitch = (int)(pm & kPitchMask);
                 const unsigned lim = (unsigned)pitch * __float_as_uint(hc.z);  // texels of the view
-                // a projective-only launch (no entry with h6 = h7 = 0) keeps the general path alone; a
-                // rectified-only instantiation measured slower than this mixed loop, so there is none
                 if (precise_kind(KIND)) {
                     const double* h64 = &Jp->H64[((int64_t)n * L + d0 + l) * 9];
                     const int wv = __float_as_int(hc.y), hv = __float_as_int(hc.z);
-                    if (mode == kOut) {
-                        if (!(COMB == FTV_COMBINE_MIN && PF)) {
-#pragma unroll
-                            for (int j = 0; j < kPPT; ++j)
-                                m[j] = (COMB == FTV_COMBINE_MIN) ? min(m[j], penalty) : m[j] + penalty;
-                        }
-                    } else if (mode == kSlow) {
+                    if (mode == kSlow) {
 #pragma unroll
                         for (int j = 0; j < kPPT; ++j) {
                             const long long q = project_fp64_packed(h64, (int)px[j] + fx0, iy[j], wv, hv);
-                            n_recomputed += key[j] != kSentinel;
+                            n_recomputed += run[j] >= 0;
                             const int idx = (int)(q >> 32) * pitch + (int)(unsigned)q;
-                            accumulate<FMT, COMB, PF>(m[j], q >= 0, tex, idx, ra[j], rb[j], rc[j], penalty, lim, ck);
+                            accumulate<FMT, COMB, PF>(m[j], q >= 0, tex, idx, ref[j], penalty, lim, ck);
                         }
-                    } else if (KIND == kKindPreciseMixed && mode == kShift) {
+                    } else if (kShifts && mode == kShift) {
                         const float4 hb = e4[1];  // (h4, h5, lower and upper bound of x')
                         const int D = __float_as_int(hc.x);
 #pragma unroll
                         for (int j = 0; j < kPPT; ++j) {
                             const bool ok = (px[j] >= hb.z) & (px[j] < hb.w);
-                            accumulate<FMT, COMB, PF>(m[j], ok, tex, rowx[j] + D, ra[j], rb[j], rc[j], penalty, lim, ck);
-                        }
-                    } else if (KIND == kKindPreciseMixed && mode == kRect) {
-                        const float a2 = e4[0].z;
-                        const float4 pe = reinterpret_cast<const float4*>(sP)[n * LBa + l];
-                        const int u0 = __float_as_int(pe.x), dv0 = __float_as_int(pe.y) - fy0;
-#pragma unroll
-                        for (int j = 0; j < kPPT; ++j) {
-                            const float tu = __fadd_rn(__fadd_rn(px[j], a2), 0.5f);
-                            const float fu = floorf(tu);
-                            int ui = __float2int_rz(fu) + u0, vi = iy[j] + dv0;
-                            bool ok;
-                            if (fabsf(__fsub_rn(__fsub_rn(tu, fu), 0.5f)) >= pe.z) {
-                                const long long q = project_fp64_packed(h64, (int)px[j] + fx0, iy[j], wv, hv);
-                                ok = q >= 0;
-                                ui = (int)(unsigned)q;
-                                vi = (int)(q >> 32);
-                                n_recomputed += key[j] != kSentinel;
-                            } else {
-                                ok = ((unsigned)ui < (unsigned)wv) & ((unsigned)vi < (unsigned)hv);
-                            }
-                            accumulate<FMT, COMB, PF>(m[j], ok, tex, vi * pitch + ui, ra[j], rb[j], rc[j], penalty, lim, ck);
+                            accumulate<FMT, COMB, PF>(m[j], ok, tex, rowx[j] + D, ref[j], penalty, lim, ck);
                         }
                     } else {
-                        const float4 ha = e4[0], hb = e4[1];
+                        // The column and row nearest u' = X'/W (as FP32) by the rounding of u' + kRound, whose low
+                        // bits hold the integer; t - nearest is exact, and when it lies within the staged threshold
+                        // of 0 the FP64 projection rounds the same way. The others (rare) are redone in FP64 below.
                         const float4 pe = reinterpret_cast<const float4*>(sP)[n * LBa + l];
                         const int u0 = __float_as_int(pe.x), v0 = __float_as_int(pe.y);
+                        unsigned redo = 0;
+                        if (kShifts && mode == kRect) {
+                            const float a2 = e4[0].z;
 #pragma unroll
-                        for (int j = 0; j < kPPT; ++j) {
-                            const float X = __fmaf_rn(ha.x, px[j], __fmaf_rn(ha.y, py[j], ha.z));
-                            const float Yh = __fmaf_rn(ha.w, px[j], __fmaf_rn(hb.x, py[j], hb.y));
-                            const float Wz = __fmaf_rn(hb.z, px[j], __fmaf_rn(hb.w, py[j], hc.x));
-                            const float r = contract_rcp<FAST_RCP>(Wz);
-                            const float tu = __fadd_rn(__fmul_rn(X, r), 0.5f);
-                            const float tv = __fadd_rn(__fmul_rn(Yh, r), 0.5f);
-                            const float fu = floorf(tu), fv = floorf(tv);
-                            const bool near = fabsf(__fsub_rn(__fsub_rn(tu, fu), 0.5f)) >= pe.z ||
-                                              fabsf(__fsub_rn(__fsub_rn(tv, fv), 0.5f)) >= pe.w;
-                            int ui = __float2int_rz(fu) + u0, vi = __float2int_rz(fv) + v0;
-                            bool ok;
-                            if (near) {
-                                const long long q = project_fp64_packed(h64, (int)px[j] + fx0, iy[j], wv, hv);
-                                ok = q >= 0;
-                                ui = (int)(unsigned)q;
-                                vi = (int)(q >> 32);
-                                n_recomputed += key[j] != kSentinel;
-                            } else {
-                                ok = ((unsigned)ui < (unsigned)wv) & ((unsigned)vi < (unsigned)hv);
+                            for (int j = 0; j < kPPT; ++j) {
+                                const float tu = __fadd_rn(px[j], a2), ru = __fadd_rn(tu, kRound);
+                                const int ui = __float_as_int(ru) + u0, vi = iy[j] + v0;
+                                if (fabsf(__fsub_rn(tu, __fsub_rn(ru, kRound))) >= pe.z) {
+                                    redo |= 1u << j;
+                                } else {
+                                    const bool ok = ((unsigned)ui < (unsigned)wv) & ((unsigned)vi < (unsigned)hv);
+                                    accumulate<FMT, COMB, PF>(m[j], ok, tex, vi * pitch + ui, ref[j], penalty, lim, ck);
+                                }
                             }
-                            accumulate<FMT, COMB, PF>(m[j], ok, tex, vi * pitch + ui, ra[j], rb[j], rc[j], penalty, lim, ck);
+                        } else {
+                            const float4 ha = e4[0], hb = e4[1];
+#pragma unroll
+                            for (int j = 0; j < kPPT; ++j) {
+                                const float X = __fmaf_rn(ha.x, px[j], __fmaf_rn(ha.y, py[j], ha.z));
+                                const float Yh = __fmaf_rn(ha.w, px[j], __fmaf_rn(hb.x, py[j], hb.y));
+                                const float Wz = __fmaf_rn(hb.z, px[j], __fmaf_rn(hb.w, py[j], hc.x));
+                                const float r = contract_rcp_normal<FAST_RCP>(Wz);
+                                const float tu = __fmul_rn(X, r), tv = __fmul_rn(Yh, r);
+                                const float ru = __fadd_rn(tu, kRound), rv = __fadd_rn(tv, kRound);
+                                const int ui = __float_as_int(ru) + u0, vi = __float_as_int(rv) + v0;
+                                if (fabsf(__fsub_rn(tu, __fsub_rn(ru, kRound))) >= pe.z ||
+                                    fabsf(__fsub_rn(tv, __fsub_rn(rv, kRound))) >= pe.w) {
+                                    redo |= 1u << j;
+                                } else {
+                                    const bool ok = ((unsigned)ui < (unsigned)wv) & ((unsigned)vi < (unsigned)hv);
+                                    accumulate<FMT, COMB, PF>(m[j], ok, tex, vi * pitch + ui, ref[j], penalty, lim, ck);
+                                }
+                            }
+                        }
+                        if (redo) {
+#pragma unroll
+                            for (int j = 0; j < kPPT; ++j)
+                                if (redo >> j & 1u) {
+                                    const long long q = project_fp64_packed(h64, (int)px[j] + fx0, iy[j], wv, hv);
+                                    const int idx = (int)(q >> 32) * pitch + (int)(unsigned)q;
+                                    accumulate<FMT, COMB, PF>(m[j], q >= 0, tex, idx, ref[j], penalty, lim, ck);
+                                    n_recomputed += run[j] >= 0;
+                                }
                         }
                     }
-                } else if (KIND == kKindMixed && mode == kShift) {
+                } else if (mode == kShift) {
                     const float4 hb = e4[1];  // (h4, h5, -D, w - D)
                     const int D = __float_as_int(hc.x);
 #pragma unroll
                     for (int j = 0; j < kPPT; ++j) {
                         const bool ok = (px[j] >= hb.z) & (px[j] < hb.w);
-                        accumulate<FMT, COMB, false>(m[j], ok, tex, rowx[j] + D, ra[j], rb[j], rc[j], penalty, lim, ck);
+                        accumulate<FMT, COMB, false>(m[j], ok, tex, rowx[j] + D, ref[j], penalty, lim, ck);
                     }
-                } else if (KIND == kKindMixed && mode == kRect) {
+                } else if (mode == kRect) {
 #pragma unroll
                     for (int j = 0; j < kPPT; ++j) {
                         int idx;
                         const bool ok = pos_rect(hc.x, __float_as_uint(hc.y), __float_as_uint(hc.z), pitch, px[j], iy[j],
                                                  idx);
-                        accumulate<FMT, COMB, false>(m[j], ok, tex, idx, ra[j], rb[j], rc[j], penalty, lim, ck);
+                        accumulate<FMT, COMB, false>(m[j], ok, tex, idx, ref[j], penalty, lim, ck);
                     }
-                } else if (KIND == kKindMixed && mode == kGeneral) {
+                } else if (mode == kGeneral) {
                     const float4 ha = e4[0], hb = e4[1];
 #pragma unroll
                     for (int j = 0; j < kPPT; ++j) {
                         int idx;
                         const bool ok = pos_general<FAST_RCP>(ha, hb, hc, pitch, px[j], row_f(j), idx);
-                        accumulate<FMT, COMB, PF>(m[j], ok, tex, idx, ra[j], rb[j], rc[j], penalty, lim, ck);
+                        accumulate<FMT, COMB, PF>(m[j], ok, tex, idx, ref[j], penalty, lim, ck);
                     }
-                } else if (KIND == kKindMixed && mode == kUnit) {
+                } else if (mode == kUnit) {
                     const float4 ha = e4[0], hb = e4[1];
 #pragma unroll
                     for (int j = 0; j < kPPT; ++j) {
                         int idx;
                         const bool ok = pos_affine<true>(ha, hb, hc, 1.0f, pitch, px[j], row_f(j), idx);
-                        accumulate<FMT, COMB, false>(m[j], ok, tex, idx, ra[j], rb[j], rc[j], penalty, lim, ck);
+                        accumulate<FMT, COMB, false>(m[j], ok, tex, idx, ref[j], penalty, lim, ck);
                     }
-                } else if (KIND == kKindMixed && mode == kAffine) {
+                } else {  // kAffine
                     const float4 ha = e4[0], hb = e4[1];
 #pragma unroll
                     for (int j = 0; j < kPPT; ++j) {
                         int idx;
                         const bool ok = pos_affine<false>(ha, hb, hc, hb.z, pitch, px[j], row_f(j), idx);
-                        accumulate<FMT, COMB, false>(m[j], ok, tex, idx, ra[j], rb[j], rc[j], penalty, lim, ck);
+                        accumulate<FMT, COMB, false>(m[j], ok, tex, idx, ref[j], penalty, lim, ck);
                     }
-                } else if (KIND == kKindMixed && !(COMB == FTV_COMBINE_MIN && PF)) {
-#pragma unroll
-                    for (int j = 0; j < kPPT; ++j) m[j] = (COMB == FTV_COMBINE_MIN) ? min(m[j], penalty) : m[j] + penalty;
                 }
             }
-            // segmented warp reduction: keys are nondecreasing along the lanes
+            const int seen = kProj ? c3 : c2;
+            if (!(COMB == FTV_COMBINE_MIN && PF) && seen < N) {  // entries out of view: the penalty each
 #pragma unroll
-            for (int j = 0; j < kPPT; ++j) {
-                const int v = key[j] != kSentinel ? m[j] : 0;
-                const int kfirst = key[j];  // lane 0's key is the warp's when uni
-                if ((uni | none) >> j & 1u) {
-                    if (uni >> j & 1u) {
-                        const int sum = __reduce_add_sync(kFull, v);
-                        if (lane == 0) {
-                            if (kfirst < kSegAcc) atomicAdd(&sAcc[kfirst * kMaxLB + l], sum);
-                            else {
-                                const int s = list ? list[k0 + kfirst] : k0 + kfirst;
-                                atomicAdd(&cost[(int64_t)s * L + d0 + l], sum);
-                            }
-                        }
-                    }
-                } else {
-                    unsigned rem = kFull;
-                    while (rem) {
-                        const int leader = __ffs(rem) - 1;
-                        const int kk = __shfl_sync(kFull, key[j], leader);
-                        const unsigned grp = __ballot_sync(kFull, key[j] == kk);
-                        const int sum = __reduce_add_sync(kFull, key[j] == kk ? v : 0);
-                        if (lane == leader && kk != kSentinel) {
-                            if (kk < kSegAcc) atomicAdd(&sAcc[kk * kMaxLB + l], sum);
-                            else {
-                                const int s = list ? list[k0 + kk] : k0 + kk;
-                                atomicAdd(&cost[(int64_t)s * L + d0 + l], sum);
-                            }
-                        }
-                        rem &= ~grp;
+                for (int j = 0; j < kPPT; ++j)
+                    m[j] = (COMB == FTV_COMBINE_MIN) ? min(m[j], penalty) : m[j] + (N - seen) * penalty;
+            }
+            // Each run's sum over the warp's pixels: a thread adds its own slots first, so that a label costs one
+            // warp reduction per run (a 128-pixel stretch meets two or three segments) instead of one per slot.
+            if (nk < 0xffff) {
+                for (int r = 0; r < n_runs; ++r) {
+                    int v = 0;
+#pragma unroll
+                    for (int j = 0; j < kPPT; ++j) v += run[j] == r ? m[j] : 0;
+                    const int sum = __reduce_add_sync(kFull, v);
+                    if (lane == 0) {
+                        const int k = sKey[warp][r];
+                        if (k < kSegAcc) atomicAdd(&sAcc[k * kMaxLB + l], sum);
+                        else atomicAdd(&cost[(int64_t)(list ? list[k0 + k] : k0 + k) * L + d0 + l], sum);
                     }
                 }
+            } else {  // a tile spanning 2^16 empty segments: their keys do not fit sKey; each pixel on its own
+#pragma unroll
+                for (int j = 0; j < kPPT; ++j)
+                    if (run[j] >= 0) {
+                        const int k = upper_index(woffs, k0, k1 + 1, w0 + warp * kWarpPix + j * 32 + lane);
+                        atomicAdd(&cost[(int64_t)(list ? list[k] : k) * L + d0 + l], m[j]);
+                    }
             }
         }
         __syncthreads();
 
-        // write the row slices of this tile's segments
-        const int nacc = min(nk, kSegAcc);
+        // write the row slices of this tile's segments (all but the last case above)
+        const int nacc = nk < 0xffff ? min(nk, kSegAcc) : 0;
         for (int i = tid; i < nacc * LBa; i += kThreads) {
             const int loc = i / LBa, l = i - loc * LBa;
             const int k = k0 + loc;
@@ -947,7 +1012,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cost_kernel(const RefJob
 template <int FMT, int COMB, bool FAST>
 int blocks_per_sm_for() {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, cost_kernel<FMT, COMB, FAST, COMB == FTV_COMBINE_MIN, kKindMixed>,
+    constexpr int kind = FMT == FMT_U16S ? kKindProjective : kKindMixed;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, cost_kernel<FMT, COMB, FAST, COMB == FTV_COMBINE_MIN, kind>,
                                                       kThreads, 0) != cudaSuccess)
         return 1;
     return n > 0 ? n : 1;
@@ -1001,6 +1067,8 @@ int cost_blocks_per_sm(int fmt, int combine, bool fast) {
 #define FTV_OCC(F, C) (fast ? blocks_per_sm_for<F, C, true>() : blocks_per_sm_for<F, C, false>())
     if (fmt == FMT_U8X4) return combine == FTV_COMBINE_MIN ? FTV_OCC(FMT_U8X4, FTV_COMBINE_MIN)
                                                            : FTV_OCC(FMT_U8X4, FTV_COMBINE_SUM);
+    if (fmt == FMT_U16S) return combine == FTV_COMBINE_MIN ? FTV_OCC(FMT_U16S, FTV_COMBINE_MIN)
+                                                           : FTV_OCC(FMT_U16S, FTV_COMBINE_SUM);
     if (fmt == FMT_P10) return combine == FTV_COMBINE_MIN ? FTV_OCC(FMT_P10, FTV_COMBINE_MIN)
                                                           : FTV_OCC(FMT_P10, FTV_COMBINE_SUM);
     return combine == FTV_COMBINE_MIN ? FTV_OCC(FMT_U16X4, FTV_COMBINE_MIN) : FTV_OCC(FMT_U16X4, FTV_COMBINE_SUM);
@@ -1033,32 +1101,48 @@ void launch_one(const RefJob* jobs, Plan* p, int ck, int nck, int grid, cudaStre
     cost_kernel<FMT, COMB, FAST, PF, KIND><<<grid, kThreads, 0, s>>>(jobs, p, ck, nck);
 }
 
-template <int FMT, int COMB, bool FAST, bool PF>
-void launch_kind(const RefJob* jobs, Plan* p, int kind, int ck, int nck, int grid, cudaStream_t s) {
-    if (kind == kKindPrecise) launch_one<FMT, COMB, FAST, PF, kKindPrecise>(jobs, p, ck, nck, grid, s);
-    else if (kind == kKindPreciseMixed) launch_one<FMT, COMB, FAST, PF, kKindPreciseMixed>(jobs, p, ck, nck, grid, s);
-    else if (kind == kKindProjective) launch_one<FMT, COMB, FAST, PF, kKindProjective>(jobs, p, ck, nck, grid, s);
-    else launch_one<FMT, COMB, FAST, PF, kKindMixed>(jobs, p, ck, nck, grid, s);
+// Kinds an instantiation exists for: FMT_U16S units are all projective; FMT_P10 ones have affine entries, or share
+// a batch with units that do (cost_format()).
+constexpr bool kind_of_format(int fmt, int kind) {
+    return fmt == FMT_U16S ? kind == kKindProjective || kind == kKindPrecise
+                           : fmt != FMT_P10 || kind == kKindMixed || kind == kKindPreciseMixed;
 }
 
-template <int FMT, int COMB>
-void launch_fast_pf(const RefJob* jobs, Plan* p, bool fast, bool pf, int kind, int ck, int nck, int grid,
-                    cudaStream_t s) {
-    const bool use_pf = COMB == FTV_COMBINE_MIN && pf;
-    if (fast) {
-        if (use_pf) launch_kind<FMT, COMB, true, true>(jobs, p, kind, ck, nck, grid, s);
-        else launch_kind<FMT, COMB, true, false>(jobs, p, kind, ck, nck, grid, s);
+template <int FMT, int COMB, bool FAST, bool PF, int KIND>
+cudaError_t launch_if(const RefJob* jobs, Plan* p, int ck, int nck, int grid, cudaStream_t s) {
+    if constexpr (kind_of_format(FMT, KIND)) {
+        launch_one<FMT, COMB, FAST, PF, KIND>(jobs, p, ck, nck, grid, s);
+        return cudaSuccess;
     } else {
-        if (use_pf) launch_kind<FMT, COMB, false, true>(jobs, p, kind, ck, nck, grid, s);
-        else launch_kind<FMT, COMB, false, false>(jobs, p, kind, ck, nck, grid, s);
+        return cudaErrorInvalidValue;
     }
 }
 
+template <int FMT, int COMB, bool FAST, bool PF>
+cudaError_t launch_kind(const RefJob* jobs, Plan* p, int kind, int ck, int nck, int grid, cudaStream_t s) {
+    if (kind == kKindPrecise) return launch_if<FMT, COMB, FAST, PF, kKindPrecise>(jobs, p, ck, nck, grid, s);
+    if (kind == kKindPreciseMixed) return launch_if<FMT, COMB, FAST, PF, kKindPreciseMixed>(jobs, p, ck, nck, grid, s);
+    if (kind == kKindProjective) return launch_if<FMT, COMB, FAST, PF, kKindProjective>(jobs, p, ck, nck, grid, s);
+    return launch_if<FMT, COMB, FAST, PF, kKindMixed>(jobs, p, ck, nck, grid, s);
+}
+
+template <int FMT, int COMB>
+cudaError_t launch_fast_pf(const RefJob* jobs, Plan* p, bool fast, bool pf, int kind, int ck, int nck, int grid,
+                    cudaStream_t s) {
+    const bool use_pf = COMB == FTV_COMBINE_MIN && pf;
+    if (fast) {
+        if (use_pf) return launch_kind<FMT, COMB, true, true>(jobs, p, kind, ck, nck, grid, s);
+        return launch_kind<FMT, COMB, true, false>(jobs, p, kind, ck, nck, grid, s);
+    }
+    if (use_pf) return launch_kind<FMT, COMB, false, true>(jobs, p, kind, ck, nck, grid, s);
+    return launch_kind<FMT, COMB, false, false>(jobs, p, kind, ck, nck, grid, s);
+}
+
 template <int FMT>
-void launch_comb(const RefJob* jobs, Plan* p, int combine, bool fast, bool pf, int kind, int ck, int nck, int grid,
+cudaError_t launch_comb(const RefJob* jobs, Plan* p, int combine, bool fast, bool pf, int kind, int ck, int nck, int grid,
                  cudaStream_t s) {
-    if (combine == FTV_COMBINE_MIN) launch_fast_pf<FMT, FTV_COMBINE_MIN>(jobs, p, fast, pf, kind, ck, nck, grid, s);
-    else launch_fast_pf<FMT, FTV_COMBINE_SUM>(jobs, p, fast, pf, kind, ck, nck, grid, s);
+    if (combine == FTV_COMBINE_MIN) return launch_fast_pf<FMT, FTV_COMBINE_MIN>(jobs, p, fast, pf, kind, ck, nck, grid, s);
+    return launch_fast_pf<FMT, FTV_COMBINE_SUM>(jobs, p, fast, pf, kind, ck, nck, grid, s);
 }
 
 }  // namespace
@@ -1067,9 +1151,12 @@ cudaError_t launch_cost(const RefJob* jobs, const Plan* plan, int fmt, int combi
                         int chunk, int chunks, int grid, cudaStream_t s) {
     if (chunks < 1 || chunks > kMaxChunks || chunk < 0 || chunk >= chunks) return cudaErrorInvalidValue;
     Plan* p = const_cast<Plan*>(plan);
-    if (fmt == FMT_U8X4) launch_comb<FMT_U8X4>(jobs, p, combine, fast, pf, kind, chunk, chunks, grid, s);
-    else if (fmt == FMT_P10) launch_comb<FMT_P10>(jobs, p, combine, fast, pf, kind, chunk, chunks, grid, s);
-    else launch_comb<FMT_U16X4>(jobs, p, combine, fast, pf, kind, chunk, chunks, grid, s);
+    cudaError_t e;
+    if (fmt == FMT_U8X4) e = launch_comb<FMT_U8X4>(jobs, p, combine, fast, pf, kind, chunk, chunks, grid, s);
+    else if (fmt == FMT_U16S) e = launch_comb<FMT_U16S>(jobs, p, combine, fast, pf, kind, chunk, chunks, grid, s);
+    else if (fmt == FMT_P10) e = launch_comb<FMT_P10>(jobs, p, combine, fast, pf, kind, chunk, chunks, grid, s);
+    else e = launch_comb<FMT_U16X4>(jobs, p, combine, fast, pf, kind, chunk, chunks, grid, s);
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 

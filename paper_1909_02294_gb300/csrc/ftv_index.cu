@@ -47,6 +47,8 @@ __global__ void pack_kernel(const void* Yp, const void* Up, const void* Vp, int6
         static_cast<uint32_t*>(out)[i] = a | (b << 8) | (c << 16);
     } else if (FMT == FMT_P10) {
         static_cast<uint32_t*>(out)[i] = a | (b << 10) | (c << 20);
+    } else if (FMT == FMT_U16S) {
+        static_cast<uint2*>(out)[i] = make_uint2(a | (b << 16), c | ((a + b + c) << 16));
     } else {
         static_cast<uint2*>(out)[i] = make_uint2(a | (b << 16), c);
     }
@@ -257,6 +259,9 @@ cudaError_t launch_pack(const void* const* planes, const int64_t* pitch, int sam
     } else if (fmt == FMT_P10) {
         pack_kernel<2, FMT_P10><<<grid, block, 0, s>>>(planes[0], planes[1], planes[2], pitch[0], pitch[1],
                                                       pitch[2], W, maxv, out, status);
+    } else if (fmt == FMT_U16S) {
+        pack_kernel<2, FMT_U16S><<<grid, block, 0, s>>>(planes[0], planes[1], planes[2], pitch[0], pitch[1],
+                                                       pitch[2], W, maxv, out, status);
     } else {
         pack_kernel<2, FMT_U16X4><<<grid, block, 0, s>>>(planes[0], planes[1], planes[2], pitch[0], pitch[1],
                                                         pitch[2], W, maxv, out, status);
@@ -291,9 +296,9 @@ cudaError_t launch_plan_device(RefJob* d_jobs, const int32_t* n_jobs, Plan* plan
 }
 
 cudaError_t launch_plan(const RefJob* host_jobs, int n_jobs, RefJob* d_jobs, Plan* plan, cudaStream_t s) {
-    if (n_jobs < 0 || n_jobs > kMaxUnits) return cudaErrorInvalidValue;
+    if (n_jobs < 0 || n_jobs > FTV_MAX_VIEWS) return cudaErrorInvalidValue;  // one unit per reference
     if (n_jobs <= 16) return launch_plan_cap<16>(host_jobs, n_jobs, d_jobs, plan, s);
-    return launch_plan_cap<kMaxUnits>(host_jobs, n_jobs, d_jobs, plan, s);
+    return launch_plan_cap<FTV_MAX_VIEWS>(host_jobs, n_jobs, d_jobs, plan, s);
 }
 
 cudaError_t launch_zero_rows(int32_t* cost, int L, int S, const int32_t* list, const int32_t* n_listed,

@@ -27,6 +27,7 @@ enum TexelFormat : int32_t {
     FMT_U8X4 = 0,   // uint32: Y | Cb << 8 | Cr << 16          (8-bit samples)
     FMT_P10 = 1,    // uint32: Y | Cb << 10 | Cr << 20         (16-bit samples of at most 10 bits)
     FMT_U16X4 = 2,  // uint2 : (Y | Cb << 16, Cr)              (16-bit samples of 11 to 16 bits)
+    FMT_U16S = 3,   // uint2 : (Y | Cb << 16, Cr | (Y + Cb + Cr) << 16)  (16-bit samples of at most 14 bits)
 };
 
 // Device status bits (OR-ed by kernels, read and cleared by ftv_check).
@@ -55,12 +56,14 @@ constexpr int kSegAcc = 16;         // per-tile segment accumulators in shared m
 // Geometry of a neighbour view as the cost kernel sees it.
 struct NbrView {
     const void* texels;  // packed view, row pitch `pitch` texels
-    int32_t w, h, pitch, pad;
+    int32_t w, h, pitch;
+    int32_t off;  // texels from the start of the allocation that holds all the unit's views; -1: beyond int32
 };
 
 // One (job, reference) unit of the persistent cost kernel. Plan fields are written on the device.
 struct RefJob {
     const void* ref_texels;    // packed reference view (row pitch = W texels)
+    const void* all_texels;    // start of the allocation that holds every view (NbrView::off)
     const uint32_t* pix;       // segment index records: (y << 16) | x, grouped by segment
     const int32_t* offs;       // segment index offsets [S + 1]
     const int32_t* list;       // listed segments or nullptr (all)
@@ -96,7 +99,7 @@ struct RefState {
     std::vector<int32_t> nbrs;
     float* d_H = nullptr;      // [N][L][9]
     double* d_H64 = nullptr;   // [N][L][9] unrounded table (FP64-precision contexts only)
-    NbrView* d_nbrs = nullptr; // [N]
+    NbrView* d_nbrs = nullptr; // [2][N]: views packed in cost_fmt, then in fmt (both in the context's d_packed)
     int32_t* d_offs = nullptr;   // [max_segments + 1]
     int32_t* d_cursor = nullptr; // [max_segments]
     int32_t* d_woffs = nullptr;  // [max_segments + 1]
@@ -155,8 +158,11 @@ struct ftv_ctx {
     std::vector<float> label_z;
     // device scratch
     void* d_packed = nullptr;                 // all views, packed texels
-    std::vector<size_t> view_offset_bytes;    // byte offset of each packed view
+    std::vector<size_t> view_offset_bytes;    // byte offset of each packed view (fmt)
     size_t texel_bytes = 4;
+    int32_t cost_fmt = 0;                     // texel format of the cost kernel's views in d_packed
+    std::vector<size_t> cost_offset_bytes;    // byte offset of each view packed in cost_fmt
+    size_t cost_texel_bytes = 4;
     uint32_t* d_status = nullptr;
     ftv::RefJob* d_jobs = nullptr;            // [n_refs]
     ftv::Plan* d_plan = nullptr;
@@ -174,6 +180,17 @@ struct ftv_ctx {
 };
 
 namespace ftv {
+
+// ftv_api.cu
+NbrView nbr_view(const ftv_ctx* c, int v, void* base, size_t offset, size_t texel_bytes);
+// Texel format of the cost kernel's views. Projective rigs take FMT_U16S where the samples allow it: its cost is
+// four instructions instead of seven, and the projection leaves the L1 room for 8-byte texels (3840x2160 15-view
+// rig: 435 against 479 ms per volume with FMT_P10). Rigs with affine entries keep 4-byte texels: there the gathers
+// are most of the work (1920x1080 8-view rig: 20.0 against 21.2 ms).
+inline int cost_format(bool any_affine, int sample_bytes, int bit_depth, int fmt) {
+    return !any_affine && sample_bytes == 2 && bit_depth <= 14 ? FMT_U16S : fmt;
+}
+inline size_t texel_size(int fmt) { return fmt == FMT_U16X4 || fmt == FMT_U16S ? 8 : 4; }
 
 // Stream state (ftv_batch.cu)
 void free_stream_state(ftv_ctx* c);
