@@ -204,10 +204,8 @@ extern "C" ftv_status ftv_adjacency(ftv_ctx* ctx, int32_t ref_index, const void*
     if (prev != ctx->device) cudaSetDevice(ctx->device);
     NvtxRange range("ftv_adjacency");
     cudaStream_t s = (cudaStream_t)stream;
-    const int64_t one = std::max<int64_t>(ctx->penalty, 3LL * ((1LL << ctx->bit_depth) - 1));
-    const int64_t mpc = ctx->combine == FTV_COMBINE_MIN ? one : one * std::max(1, r.n_nbrs);
-    cudaError_t e = launch_segment_index(d_labels, r.W, r.H, n_segments, mpc, r.d_offs, r.d_cursor, r.d_pix,
-                                         ctx->d_status, s, &ctx->launches);
+    const IndexRef ref = index_ref(ctx, ref_index, d_labels, n_segments);
+    cudaError_t e = launch_segment_index(&ref, 1, ctx->d_status, s, &ctx->launches);
     r.S_indexed = n_segments;
     if (e == cudaSuccess && n_segments > 0) {
         AdjArgs a{};

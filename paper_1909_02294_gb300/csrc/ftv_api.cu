@@ -47,7 +47,8 @@ void free_ctx(ftv_ctx* c) {
         cudaFree(r.d_H64);
         cudaFree(r.d_nbrs);
         cudaFree(r.d_offs);
-        cudaFree(r.d_cursor);
+        cudaFree(r.d_recs);
+        cudaFree(r.d_tiles);
         cudaFree(r.d_woffs);
         cudaFree(r.d_pix);
         cudaFree(r.d_centre);
@@ -55,6 +56,7 @@ void free_ctx(ftv_ctx* c) {
     }
     cudaFree(c->d_packed);
     cudaFree(c->d_status);
+    cudaFree(c->d_cursors);
     cudaFree(c->d_jobs);
     cudaFree(c->d_plan);
     cudaFree(c->d_tstats);
@@ -75,6 +77,12 @@ int64_t max_pixel_cost(const ftv_ctx* c, int n_nbrs) {
 }
 
 }  // namespace
+
+// Reference `ref` of a context with a label map, as launch_segment_index takes it.
+IndexRef ftv::index_ref(const ftv_ctx* c, int ref, const int32_t* labels, int n_segments) {
+    const RefState& r = c->refs[ref];
+    return {labels, r.d_offs, r.d_cursor, r.d_pix, max_pixel_cost(c, r.n_nbrs), r.W, r.H, n_segments, c->max_segments};
+}
 
 // View v of a context packed at byte `offset` of the allocation `base`, as the kernels see it.
 NbrView ftv::nbr_view(const ftv_ctx* c, int v, void* base, size_t offset, size_t texel_bytes) {
@@ -262,7 +270,8 @@ ftv_status ftv_depth_init(const ftv_config* cfg, ftv_ctx** out) {
     bool ok = dalloc(reinterpret_cast<char**>(&c->d_packed), packed) == cudaSuccess;
     ok = ok && dalloc(&c->d_status, 1) == cudaSuccess;
     ok = ok && dalloc(&c->d_jobs, kMaxUnits) == cudaSuccess;
-    ok = ok && dalloc(&c->d_plan, 1) == cudaSuccess;
+    ok = ok && dalloc(&c->d_plan, 1) == cudaSuccess && cudaMemset(c->d_plan, 0, sizeof(Plan)) == cudaSuccess;
+    ok = ok && dalloc(&c->d_cursors, (size_t)c->n_refs * c->max_segments) == cudaSuccess;
     ok = ok && dalloc(&c->d_tstats, (size_t)std::max(1, c->n_refs) * c->max_segments * 8) == cudaSuccess;
     c->tstats_zero.assign(c->n_refs, 0);
     ok = ok && dalloc(&c->d_label_z, (size_t)c->L) == cudaSuccess;
@@ -274,7 +283,9 @@ ftv_status ftv_depth_init(const ftv_config* cfg, ftv_ctx** out) {
         if (c->precision == FTV_PRECISION_FP64) ok = ok && dalloc(&r.d_H64, r.h_H64.size()) == cudaSuccess;
         ok = ok && dalloc(&r.d_nbrs, (size_t)r.n_nbrs * 2) == cudaSuccess;
         ok = ok && dalloc(&r.d_offs, (size_t)c->max_segments + 1) == cudaSuccess;
-        ok = ok && dalloc(&r.d_cursor, (size_t)c->max_segments) == cudaSuccess;
+        r.d_cursor = c->d_cursors ? c->d_cursors + (&r - c->refs.data()) * (size_t)c->max_segments : nullptr;
+        ok = ok && dalloc(&r.d_recs, (size_t)tiles_of((int64_t)r.W * r.H) * kTile) == cudaSuccess;
+        ok = ok && dalloc(&r.d_tiles, (size_t)tiles_of((int64_t)r.W * r.H)) == cudaSuccess;
         ok = ok && dalloc(&r.d_woffs, (size_t)c->max_segments + 1) == cudaSuccess;
         ok = ok && dalloc(&r.d_pix, (size_t)r.W * r.H) == cudaSuccess;
         ok = ok && dalloc(&r.d_centre, (size_t)c->max_segments) == cudaSuccess;
@@ -363,9 +374,8 @@ ftv_status ftv_segment_index(ftv_ctx* ctx, int32_t ref_index, const int32_t* d_l
     if (n_segments < 0 || n_segments > ctx->max_segments) return FTV_ERR_INVALID_ARG;
     DeviceGuard g(ctx->device);
     RefState& r = ctx->refs[ref_index];
-    const cudaError_t e = launch_segment_index(d_labels, r.W, r.H, n_segments, max_pixel_cost(ctx, r.n_nbrs), r.d_offs,
-                                               r.d_cursor, r.d_pix, ctx->d_status, (cudaStream_t)stream,
-                                               &ctx->launches);
+    const IndexRef ref = index_ref(ctx, ref_index, d_labels, n_segments);
+    const cudaError_t e = launch_segment_index(&ref, 1, ctx->d_status, (cudaStream_t)stream, &ctx->launches);
     if (e != cudaSuccess) return FTV_ERR_CUDA;
     r.S_indexed = n_segments;
     return FTV_OK;
@@ -402,34 +412,36 @@ ftv_status ftv_cost_volume(ftv_ctx* ctx, const void* const* d_planes, const int6
     DeviceGuard g(ctx->device);
     NvtxRange range("ftv_cost_volume");
     cudaError_t e = cudaSuccess;
-    for (int v = 0; v < ctx->n_views && e == cudaSuccess; ++v) {
-        if (!used[v]) continue;
+    {
         NvtxRange stage("pack");
-        e = launch_pack(d_planes + 3 * v, pitch_bytes + 3 * v, ctx->sample_bytes, ctx->bit_depth, ctx->cost_fmt,
-                        ctx->cams[v].width, ctx->cams[v].height,
-                        static_cast<char*>(ctx->d_packed) + ctx->cost_offset_bytes[v], ctx->d_status, s);
-        ctx->launches++;
+        PackView views[FTV_MAX_VIEWS];
+        int n = 0;
+        for (int v = 0; v < ctx->n_views; ++v)
+            if (used[v])
+                views[n++] = {{d_planes[3 * v], d_planes[3 * v + 1], d_planes[3 * v + 2]},
+                              {pitch_bytes[3 * v], pitch_bytes[3 * v + 1], pitch_bytes[3 * v + 2]},
+                              static_cast<char*>(ctx->d_packed) + ctx->cost_offset_bytes[v], ctx->cams[v].width,
+                              ctx->cams[v].height, 0};
+        e = launch_pack(views, n, ctx->sample_bytes, ctx->bit_depth, ctx->cost_fmt, ctx->d_status, s, &ctx->launches);
+    }
+    if (e == cudaSuccess) {
+        NvtxRange stage("segment index");
+        IndexRef fresh[FTV_MAX_VIEWS];
+        int n = 0;
+        for (int i = 0; i < ctx->n_refs; ++i)
+            if (d_labels && d_labels[i]) {
+                fresh[n++] = index_ref(ctx, i, d_labels[i], n_segments[i]);
+                ctx->refs[i].S_indexed = n_segments[i];
+            }
+        e = launch_segment_index(fresh, n, ctx->d_status, s, &ctx->launches);
     }
     std::vector<RefJob> jobs(ctx->n_refs);
-    for (int i = 0; i < ctx->n_refs && e == cudaSuccess; ++i) {
-        RefState& r = ctx->refs[i];
-        if (d_labels && d_labels[i]) {
-            NvtxRange stage("segment index");
-            e = launch_segment_index(d_labels[i], r.W, r.H, n_segments[i], max_pixel_cost(ctx, r.n_nbrs), r.d_offs,
-                                     r.d_cursor, r.d_pix, ctx->d_status, s, &ctx->launches);
-            r.S_indexed = n_segments[i];
-        }
+    int64_t tiles = 0;
+    for (int i = 0; i < ctx->n_refs; ++i) {
+        const RefState& r = ctx->refs[i];
         const int S = r.S_indexed;
         const int32_t* list = d_seg_list ? d_seg_list[i] : nullptr;
         const int32_t* nl = list ? d_n_listed[i] : nullptr;
-        if (e == cudaSuccess) {
-            if (list) {
-                e = launch_zero_rows(d_cost[i], ctx->L, S, list, nl, s);
-                ctx->launches++;
-            } else {
-                e = cudaMemsetAsync(d_cost[i], 0, sizeof(int32_t) * (size_t)S * ctx->L, s);
-            }
-        }
         RefJob& J = jobs[i];
         std::memset(&J, 0, sizeof(J));
         J.ref_texels = static_cast<char*>(ctx->d_packed) + ctx->cost_offset_bytes[r.view];
@@ -439,6 +451,10 @@ ftv_status ftv_cost_volume(ftv_ctx* ctx, const void* const* d_planes, const int6
         J.list = list;
         J.n_listed = nl;
         J.woffs = r.d_woffs;
+        J.recs = r.d_recs;
+        J.tiles = r.d_tiles;
+        J.first = r.d_cursor;
+        tiles += tiles_of((int64_t)r.W * r.H);
         J.H = r.d_H;
         J.H64 = r.d_H64;
         J.nbrs = r.d_nbrs;
@@ -453,17 +469,19 @@ ftv_status ftv_cost_volume(ftv_ctx* ctx, const void* const* d_planes, const int6
         J.penalty = ctx->penalty;
         J.fmt = ctx->cost_fmt;
     }
+    const int grid = ctx->n_sm * (ctx->ctas_per_sm > 0 ? ctx->ctas_per_sm : ctx->cost_blocks_per_sm);
     if (e == cudaSuccess) {
         NvtxRange stage("plan");
-        e = launch_plan(jobs.data(), ctx->n_refs, ctx->d_jobs, ctx->d_plan, s);
-        ctx->launches++;
+        e = launch_plan(jobs.data(), ctx->n_refs, grid, ctx->d_jobs, ctx->d_plan, s);
+        if (e == cudaSuccess)
+            e = launch_tiles(ctx->d_jobs, ctx->d_plan, (int)std::min<int64_t>(tiles, ctx->n_sm * 8), s);
+        ctx->launches += 2;
     }
     if (e == cudaSuccess && ctx->profiling) e = cudaEventRecord(ctx->ev_start, s);
     if (e == cudaSuccess) {
         NvtxRange stage("cost kernel");
-        const int per_sm = ctx->ctas_per_sm > 0 ? ctx->ctas_per_sm : ctx->cost_blocks_per_sm;
         e = launch_cost(ctx->d_jobs, ctx->d_plan, ctx->cost_fmt, ctx->combine, ctx->fast_rcp, ctx->penalty_floor, ctx->kind,
-                        0, 1, ctx->n_sm * per_sm, s);
+                        0, 1, grid, s);
         ctx->launches++;
     }
     if (e == cudaSuccess && ctx->profiling) {

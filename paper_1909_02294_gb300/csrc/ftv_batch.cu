@@ -370,20 +370,6 @@ __global__ void __launch_bounds__(kTChunk) temporal_compact_multi_kernel(const H
     }
 }
 
-// Zero the cost rows of each unit's changed segments (blockIdx.y = unit).
-__global__ void zero_changed_rows_kernel(const Header* __restrict__ hdr, const RefJob* __restrict__ jobs) {
-    for (int u = blockIdx.y; u < hdr->n_units; u += gridDim.y) {
-        const RefJob& J = jobs[u];
-        const int n = min(max(*J.n_listed, 0), J.S);
-        const int64_t total = (int64_t)n * J.L;
-        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-            const int k = (int)(i / J.L), d = (int)(i - (int64_t)k * J.L);
-            const int s = J.list[k];
-            if ((unsigned)s < (unsigned)J.S) J.cost[(int64_t)s * J.L + d] = 0;
-        }
-    }
-}
-
 // ------------------------------------------------------------------------------------------ WTA etc.
 
 // One warp per segment over all units: argmin for changed segments (smallest label on ties), adoption
@@ -590,6 +576,7 @@ int64_t context_bytes_of(size_t packed, const std::vector<RefDims>& refs, int64_
     for (const RefDims& r : refs) {
         b += r.N * L * 9 * 4 + (fp64 ? r.N * L * 9 * 8 : 0) + 2 * r.N * (int64_t)sizeof(NbrView);
         b += 2 * (MS + 1) * 4 + MS * 4 + r.W * r.H * 4 + MS * 8 + std::max<int64_t>(1, r.N) * 8;
+        b += tiles_of(r.W * r.H) * (int64_t)(kTile * sizeof(int2) + sizeof(int4));
     }
     return b;
 }
@@ -704,17 +691,14 @@ ftv_status ftv_stream_init(ftv_ctx* ctx, const int32_t* const* d_labels, const i
         if (prev_dev >= 0 && prev_dev != ctx->device) cudaSetDevice(prev_dev);
         return FTV_ERR_OUT_OF_MEMORY;
     }
-    cudaError_t e = cudaSuccess;
-    for (int i = 0; i < ctx->n_refs && e == cudaSuccess; ++i) {
-        // the stream's label map is static: its segment index is built once here (with the same int32
-        // overflow check as ftv_segment_index) and reused by every frame
-        RefState& r = ctx->refs[i];
-        const int64_t one = std::max<int64_t>(ctx->penalty, 3LL * ((1LL << ctx->bit_depth) - 1));
-        const int64_t mpc = ctx->combine == FTV_COMBINE_MIN ? one : one * std::max(1, r.n_nbrs);
-        e = launch_segment_index(st.refs[i].d_labels, r.W, r.H, n_segments[i], mpc, r.d_offs, r.d_cursor, r.d_pix,
-                                 st.d_status, s, &ctx->launches);
-        r.S_indexed = n_segments[i];
+    // the stream's label maps are static: their segment indexes are built once here (with the same int32
+    // overflow check as ftv_segment_index) and reused by every frame
+    IndexRef refs[FTV_MAX_VIEWS];
+    for (int i = 0; i < ctx->n_refs; ++i) {
+        refs[i] = index_ref(ctx, i, st.refs[i].d_labels, n_segments[i]);
+        ctx->refs[i].S_indexed = n_segments[i];
     }
+    const cudaError_t e = launch_segment_index(refs, ctx->n_refs, st.d_status, s, &ctx->launches);
     if (prev_dev >= 0 && prev_dev != ctx->device) cudaSetDevice(prev_dev);
     if (e != cudaSuccess) return FTV_ERR_CUDA;
     st.ready = true;
@@ -909,6 +893,7 @@ ftv_status ftv_batch_create(int32_t max_jobs, int32_t max_units, int32_t max_vie
     bool ok = cudaMalloc(reinterpret_cast<void**>(&b->d_desc), b->lay.total) == cudaSuccess;
     ok = ok && cudaMallocHost(reinterpret_cast<void**>(&b->h_stage), b->lay.total) == cudaSuccess;
     ok = ok && cudaMalloc(reinterpret_cast<void**>(&b->d_plan), sizeof(Plan)) == cudaSuccess;
+    ok = ok && cudaMemset(b->d_plan, 0, sizeof(Plan)) == cudaSuccess;
     ok = ok && cudaMalloc(reinterpret_cast<void**>(&b->d_job_status), sizeof(uint32_t) * max_jobs) == cudaSuccess;
     ok = ok && cudaMemset(b->d_job_status, 0, sizeof(uint32_t) * max_jobs) == cudaSuccess;
     ok = ok && cudaMallocHost(reinterpret_cast<void**>(&b->h_job_status), sizeof(uint32_t) * max_jobs) == cudaSuccess;
@@ -1064,6 +1049,9 @@ ftv_status ftv_batch_prepare(ftv_batch* b, const ftv_frame_job* jobs, int32_t n_
             q.list = S.d_changed;
             q.n_listed = S.d_n_changed;
             q.woffs = r.d_woffs;
+            q.recs = r.d_recs;
+            q.tiles = r.d_tiles;
+            q.first = r.d_cursor;
             q.H = r.d_H;
             q.H64 = r.d_H64;
             q.nbrs = own ? r.d_nbrs : S.d_nbrs_ring[cur];
@@ -1151,8 +1139,8 @@ static cudaError_t enqueue(ftv_batch* b, cudaStream_t s) {
     temporal_accumulate_multi_kernel<<<b->n_sm * b->temp_per_sm, 256, 0, s>>>(hdr, temp);
     temporal_decide_multi_kernel<<<g, kTChunk, 0, s>>>(hdr, temp);
     temporal_compact_multi_kernel<<<g, kTChunk, 0, s>>>(hdr, temp);
-    zero_changed_rows_kernel<<<dim3(64, std::min(b->max_units, 65535)), 256, 0, s>>>(hdr, jobs);
-    e = launch_plan_device(jobs, &hdr->n_units, b->d_plan, s);
+    e = launch_plan_device(jobs, &hdr->n_units, b->max_units, b->cost_grid, b->d_plan, s);
+    if (e == cudaSuccess) e = launch_tiles(jobs, b->d_plan, b->n_sm * 8, s);
     if (e != cudaSuccess) return e;
     // The cost items run in `chunks` persistent launches over consecutive item ranges: between two of
     // them the GPU can start other streams' work (of a higher priority first) instead of waiting for the

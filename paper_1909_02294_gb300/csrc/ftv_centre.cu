@@ -495,21 +495,24 @@ extern "C" ftv_status ftv_centre_table(ftv_ctx* ctx, const void* const* d_planes
     NvtxRange range("ftv_centre_table");
     cudaStream_t s = (cudaStream_t)stream;
     cudaError_t e = cudaSuccess;
-    for (int v = 0; v < ctx->n_views && e == cudaSuccess; ++v) {
-        e = launch_pack(d_planes + 3 * v, pitch_bytes + 3 * v, ctx->sample_bytes, ctx->bit_depth, ctx->fmt,
-                        ctx->cams[v].width, ctx->cams[v].height,
-                        static_cast<char*>(ctx->d_packed) + ctx->view_offset_bytes[v], ctx->d_status, s);
-        ctx->launches++;
+    PackView views[FTV_MAX_VIEWS];
+    for (int v = 0; v < ctx->n_views; ++v)
+        views[v] = {{d_planes[3 * v], d_planes[3 * v + 1], d_planes[3 * v + 2]},
+                    {pitch_bytes[3 * v], pitch_bytes[3 * v + 1], pitch_bytes[3 * v + 2]},
+                    static_cast<char*>(ctx->d_packed) + ctx->view_offset_bytes[v], ctx->cams[v].width,
+                    ctx->cams[v].height, 0};
+    e = launch_pack(views, ctx->n_views, ctx->sample_bytes, ctx->bit_depth, ctx->fmt, ctx->d_status, s, &ctx->launches);
+    if (e == cudaSuccess) {
+        IndexRef refs[FTV_MAX_VIEWS];
+        for (int i = 0; i < ctx->n_refs; ++i) {
+            refs[i] = index_ref(ctx, i, d_labels_views[ctx->refs[i].view], n_segments[i]);
+            ctx->refs[i].S_indexed = n_segments[i];
+        }
+        e = launch_segment_index(refs, ctx->n_refs, ctx->d_status, s, &ctx->launches);
     }
     for (int i = 0; i < ctx->n_refs && e == cudaSuccess; ++i) {
         RefState& r = ctx->refs[i];
         const int S = n_segments[i];
-        // same int32 bound as ftv_cost_volume, since the index is cached for later volume calls
-        const int64_t one = std::max<int64_t>(ctx->penalty, 3LL * ((1LL << ctx->bit_depth) - 1));
-        const int64_t mpc = ctx->combine == FTV_COMBINE_MIN ? one : one * std::max(1, r.n_nbrs);
-        e = launch_segment_index(d_labels_views[r.view], r.W, r.H, S, mpc, r.d_offs, r.d_cursor, r.d_pix, ctx->d_status,
-                                 s, &ctx->launches);
-        r.S_indexed = S;
         if (e != cudaSuccess) break;
         centroid_kernel<<<std::max(1, std::min(65535, (S + 7) / 8)), 256, 0, s>>>(r.d_offs, r.d_pix, S, r.d_centre);
         ctx->launches++;

@@ -68,23 +68,29 @@ struct RefJob {
     const int32_t* offs;       // segment index offsets [S + 1]
     const int32_t* list;       // listed segments or nullptr (all)
     const int32_t* n_listed;   // device length of `list` (nullptr with list == nullptr)
+    int32_t* first;            // scratch [S]: a segment's first entry in a list that is not strictly increasing
     int32_t* woffs;            // scratch [S + 1]: prefix of listed segment sizes (written by plan)
+    int2* recs;                // scratch [ceil(W * Href / kTile) * kTile]: per listed pixel (y << 16 | x, index of its segment in
+                               // the list), ordered within each tile (written by the tile kernel)
+    int4* tiles;               // scratch [ceil(W * Href / kTile)]: first and last listed segment, x min | x max << 16, y likewise
     const float* H;            // [N][L][9]
     const double* H64;         // [N][L][9] unrounded table (FP64-precision units; else nullptr)
     const NbrView* nbrs;       // [N]
     int32_t* cost;             // [S][L]
-    int32_t W, S, N, L, LB, nLB, penalty, fmt;
+    int32_t W, S, N, L, LB, nLB, penalty, fmt;  // LB: in, the largest label block; out, the one used
     int32_t Href;              // reference height
     // plan outputs
     int32_t n_work;            // listed segments
     int32_t n_rec;             // listed pixels
-    int32_t n_items;           // tiles * nLB
     int32_t item_base;         // first item of this unit in the launch
+    int32_t tile_base;         // first tile of this unit in the launch
 };
 
 constexpr int kMaxChunks = 16;  // a launch's items may be split over this many cost-kernel launches
 struct Plan {
     int32_t total_items;
+    int32_t total_tiles;
+    int32_t ticket;            // blocks of the plan kernel that have finished (zero between launches)
     int32_t n_jobs;            // units in the launch
     unsigned long long culled; // evaluations decided without sampling: the tile is out of that view
     unsigned long long recomputed;  // FP64-precision evaluations computed in double precision
@@ -101,7 +107,9 @@ struct RefState {
     double* d_H64 = nullptr;   // [N][L][9] unrounded table (FP64-precision contexts only)
     NbrView* d_nbrs = nullptr; // [2][N]: views packed in cost_fmt, then in fmt (both in the context's d_packed)
     int32_t* d_offs = nullptr;   // [max_segments + 1]
-    int32_t* d_cursor = nullptr; // [max_segments]
+    int32_t* d_cursor = nullptr; // [max_segments], in the context's d_cursors
+    int2* d_recs = nullptr;      // [tiles * kTile] tile records
+    int4* d_tiles = nullptr;     // [tiles]
     int32_t* d_woffs = nullptr;  // [max_segments + 1]
     uint32_t* d_pix = nullptr;   // [W * H]
     int32_t S_indexed = -1;      // segment count of the cached index (-1: none)
@@ -164,6 +172,7 @@ struct ftv_ctx {
     std::vector<size_t> cost_offset_bytes;    // byte offset of each view packed in cost_fmt
     size_t cost_texel_bytes = 4;
     uint32_t* d_status = nullptr;
+    int32_t* d_cursors = nullptr;             // [n_refs][max_segments] segment index counters
     ftv::RefJob* d_jobs = nullptr;            // [n_refs]
     ftv::Plan* d_plan = nullptr;
     int64_t* d_tstats = nullptr;              // per reference: temporal sums, 8 planes of max_segments (adjacency scratch)
@@ -182,6 +191,8 @@ struct ftv_ctx {
 namespace ftv {
 
 // ftv_api.cu
+struct IndexRef;
+IndexRef index_ref(const ftv_ctx* c, int ref, const int32_t* labels, int n_segments);
 NbrView nbr_view(const ftv_ctx* c, int v, void* base, size_t offset, size_t texel_bytes);
 // Texel format of the cost kernel's views. Projective rigs take FMT_U16S where the samples allow it: its cost is
 // four instructions instead of seven, and the projection leaves the L1 room for 8-byte texels (3840x2160 15-view
@@ -199,19 +210,36 @@ void free_stream_state(ftv_ctx* c);
 bool label_inv_depths(int L, double z_near, double z_far, std::vector<double>& iz);
 int plane_homography(const ftv_camera& cr, const ftv_camera& cv, const ftv_camera* cc, double iz, double H[9]);
 
-// Launchers (ftv_index.cu)
-cudaError_t launch_pack(const void* const* planes, const int64_t* pitch, int sample_bytes, int bit_depth, int fmt,
-                        int W, int H, void* out, uint32_t* status, cudaStream_t s);
-cudaError_t launch_segment_index(const int32_t* labels, int W, int H, int S, int64_t max_pix_cost, int32_t* offs,
-                                 int32_t* cursor, uint32_t* pix, uint32_t* status, cudaStream_t s, int64_t* launches);
-// Descriptors travel as kernel parameters (graph-capturable, no host staging buffer to race on).
+// Launchers (ftv_index.cu). Descriptors travel as kernel parameters (graph-capturable, no host staging buffer to
+// race on); a launch takes up to FTV_MAX_VIEWS views or references.
+struct PackView {
+    const void* planes[3];
+    int64_t pitch[3];
+    void* out;
+    int32_t W, H;
+    int32_t vec;  // set by launch_pack: four pixels per load and store
+};
+cudaError_t launch_pack(const PackView* views, int n, int sample_bytes, int bit_depth, int fmt, uint32_t* status,
+                        cudaStream_t s, int64_t* launches);
+struct IndexRef {
+    const int32_t* labels;  // [H][W]
+    int32_t* offs;          // [S + 1]
+    int32_t* cursor;        // [S] scratch
+    uint32_t* pix;          // [H * W]
+    int64_t max_pix_cost;
+    int32_t W, H, S;
+    int32_t stride;         // words from this reference's cursor to the next one's in the same allocation
+};
+cudaError_t launch_segment_index(const IndexRef* refs, int n, uint32_t* status, cudaStream_t s, int64_t* launches);
 constexpr int kMaxUnits = 240;  // (job, reference) units per launch
-cudaError_t launch_plan(const RefJob* host_jobs, int n_jobs, RefJob* d_jobs, Plan* plan, cudaStream_t s);
+// slots: CTAs of the cost kernel's launch, for the choice of the label blocks.
+cudaError_t launch_plan(const RefJob* host_jobs, int n_jobs, int slots, RefJob* d_jobs, Plan* plan, cudaStream_t s);
 // Same plan for descriptors already in device memory (completed in place); the unit count is read from
 // *n_jobs on the device, so one captured launch serves any batch composition.
-cudaError_t launch_plan_device(RefJob* d_jobs, const int32_t* n_jobs, Plan* plan, cudaStream_t s);
-cudaError_t launch_zero_rows(int32_t* cost, int L, int S, const int32_t* list, const int32_t* n_listed,
-                             cudaStream_t s);
+cudaError_t launch_plan_device(RefJob* d_jobs, const int32_t* n_jobs, int max_jobs, int slots, Plan* plan, cudaStream_t s);
+// Tile records of every planned unit, and its listed cost rows cleared.
+cudaError_t launch_tiles(const RefJob* jobs, const Plan* plan, int grid, cudaStream_t s);
+inline int64_t tiles_of(int64_t pixels) { return (pixels + kTile - 1) / kTile; }
 
 // Cost kernel (ftv_cost.cu)
 int cost_blocks_per_sm(int fmt, int combine, bool fast_rcp);
