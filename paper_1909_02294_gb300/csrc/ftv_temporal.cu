@@ -30,90 +30,111 @@ __device__ __forceinline__ void add64(int64_t* dst, int v) {
     atomicAdd(reinterpret_cast<unsigned long long*>(dst), (unsigned long long)(long long)v);
 }
 
-// Per-segment sums over a tile of kAccCols x kAccGroups kAccRows pixels per CTA of 256 threads: each thread
-// walks one column of kAccRows pixels and sums the vertical runs of equal labels in registers (a segment's
-// pixels are contiguous, so a column meets few runs). A finished run is added to the CTA's bins in shared
-// memory, indexed by label - (the tile's least label); labels beyond kBins of it go to global memory
-// directly. At the end each non-empty bin is added to the segment's 64-bit sums, once per tile. All sums are
-// exact integers, so the order of the additions does not change the result. Tile bins are 32-bit: a tile
-// has at most 2048 pixels of differences below 2^16.
-constexpr int kAccCols = 128;   // pixels per tile row, one thread each
-constexpr int kAccRows = 8;     // rows per thread
-constexpr int kAccGroups = 2;   // row groups per CTA
-constexpr int kAccThreads = kAccCols * kAccGroups;
+// Per-segment sums over a tile of kAccCols x kAccRowsTile pixels per CTA: each thread walks a strip of four adjacent
+// columns down kAccRows rows. A row of the strip meets at most two segments almost always (segments are many pixels
+// wide): the pixels that share the first one's label form part A, the others part B, and each part's sum over the
+// strip's row is a pair of dot products of the packed samples with the part's 0/1 weights per plane. Parts of equal
+// label in successive rows are summed in registers; a finished run is added to the CTA's bins in shared memory,
+// indexed by label - (the tile's least label); labels beyond kBins of it go to global memory directly. A row whose
+// B pixels differ in label adds them one by one. At the end each non-empty bin is added to the segment's 64-bit sums,
+// once per tile. All sums are exact integers, so the order of the additions does not change the result. Tile bins are
+// 32-bit: a tile has 1024 pixels of differences below 2^16.
+// Single columns took 61 instructions per pixel and 127 us for eight 1920x1080 references; the strips take 72, of which
+// the bytes need 54. Two rows per thread and six CTAs per SM: the loads of a strip are all in flight at once, so that
+// more rows cost warps (four rows 107 us; four CTAs 80, eight 76).
+constexpr int kAccCols = 128;      // pixels per tile row
+constexpr int kStrips = kAccCols / 4;
+constexpr int kAccRows = 2;        // rows per thread
+constexpr int kAccRowsTile = 8;    // rows per tile
+constexpr int kAccThreads = kStrips * (kAccRowsTile / kAccRows);
 constexpr int kBins = 512;
-static_assert(kAccThreads == 256, "one CTA of 256 threads per tile");
+static_assert(kAccThreads == 128, "one CTA of 128 threads per tile");
 
 // The references of one launch (kernel parameters, read in place).
 struct TemporalRefs {
     TemporalRef r[kMaxTemporalRefs];
 };
 
-template <int SB, int NCH, bool HAS_I>
-__global__ void __launch_bounds__(kAccThreads) temporal_accumulate_kernel(const __grid_constant__ TemporalRefs p,
+// Four adjacent samples of a row, packed in 16-bit lanes; n of them lie in the view (the rest repeat the last).
+template <int SB, bool VEC>
+__device__ __forceinline__ uint2 load_strip(const char* p, int n) {
+    if constexpr (VEC && SB == 2) {
+        return __ldg(reinterpret_cast<const uint2*>(p));
+    } else if constexpr (VEC) {
+        const uint32_t t = __ldg(reinterpret_cast<const uint32_t*>(p));
+        return make_uint2(__byte_perm(t, 0, 0x4140), __byte_perm(t, 0, 0x4342));
+    } else {
+        uint32_t v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = (uint32_t)load_sample<SB>(p + (int64_t)min(k, n - 1) * SB);
+        return make_uint2(v[0] | (v[1] << 16), v[2] | (v[3] << 16));
+    }
+}
+
+// c + the sum of the four samples times the weights (bytes 0/1 of the pixels, or their negatives).
+__device__ __forceinline__ int strip_dot(const uint2& v, uint32_t weights, int c) {
+    int d;
+    asm("dp2a.lo.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(v.x), "r"(weights), "r"(c));
+    asm("dp2a.hi.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(v.y), "r"(weights), "r"(d));
+    return d;
+}
+
+template <int SB, int NCH, bool HAS_I, bool VEC>
+__global__ void __launch_bounds__(kAccThreads, 6) temporal_accumulate_kernel(const __grid_constant__ TemporalRefs p,
                                                                           uint32_t* status) {
     constexpr int Q = 1 + NCH * (HAS_I ? 2 : 1);  // per segment: n, dP[NCH], dI[NCH]
-    constexpr int TR = kAccGroups * kAccRows;     // tile rows
     __shared__ __align__(16) int bins[Q][kBins];
     __shared__ int s_base, s_top;
     const TemporalRef& f = p.r[blockIdx.z];  // blockIdx.z: the reference
     const int W = f.W, H = f.H, S = f.S;
-    if ((int)blockIdx.x * kAccCols >= W || (int)blockIdx.y * TR >= H) return;  // past this view
+    if ((int)blockIdx.x * kAccCols >= W || (int)blockIdx.y * kAccRowsTile >= H) return;  // past this view
     int64_t* __restrict__ stats = f.stats;
     const int tid = threadIdx.x;
-    const int x = blockIdx.x * kAccCols + tid % kAccCols;
-    const int y0 = blockIdx.y * TR + (tid / kAccCols) * kAccRows;
-    // Every load of the column is issued before any is used: positions past the view's edge are clamped into
-    // it (the block starts inside the view), so the loads need no branch, and those pixels are then dropped
-    // through their label. Each plane's row pointer steps down the column (no per-row multiplication) and
-    // stays on the last row of the view once it is reached.
-    const int xc = min(x, W - 1), yc0 = min(y0, H - 1);
-    const int32_t* pl = f.labels + (int64_t)yc0 * W + xc;
-    const char* pa[NCH];
-    const char* pb[NCH];
-    const char* pe[HAS_I ? NCH : 1];
-#pragma unroll
-    for (int c = 0; c < NCH; ++c) {
-        pa[c] = static_cast<const char*>(f.cur[c]) + (int64_t)yc0 * f.pc[c] + (int64_t)xc * SB;
-        pb[c] = static_cast<const char*>(f.prev[c]) + (int64_t)yc0 * f.pp[c] + (int64_t)xc * SB;
-        if (HAS_I) pe[c] = static_cast<const char*>(f.ifr[c]) + (int64_t)yc0 * f.pi[c] + (int64_t)xc * SB;
-    }
-    int lab[kAccRows];
-    int a[kAccRows][NCH], b[kAccRows][NCH], e[kAccRows][HAS_I ? NCH : 1];
+    const int x = blockIdx.x * kAccCols + tid % kStrips * 4;
+    const int y0 = blockIdx.y * kAccRowsTile + (tid / kStrips) * kAccRows;
+    // Positions past the view's edge are clamped into it, so the loads need no branch, and those pixels are then
+    // dropped through their label.
+    // A vector load's strip is clamped as a whole: W is then a multiple of four.
+    const int xc = VEC ? min(x, W - 4) : min(x, W - 1), nx = min(4, W - xc), yc0 = min(y0, H - 1);
+    int lab[kAccRows][4];
+    uint2 a[kAccRows][NCH], b[kAccRows][NCH], e[kAccRows][HAS_I ? NCH : 1];
 #pragma unroll
     for (int r = 0; r < kAccRows; ++r) {
-        lab[r] = __ldg(pl);
+        const int64_t y = min(yc0 + r, H - 1);
+        const int32_t* pl = f.labels + y * W + xc;
+        if (VEC) {
+            const int4 t = __ldg(reinterpret_cast<const int4*>(pl));
+            lab[r][0] = t.x;
+            lab[r][1] = t.y;
+            lab[r][2] = t.z;
+            lab[r][3] = t.w;
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) lab[r][k] = __ldg(pl + min(k, nx - 1));
+        }
 #pragma unroll
         for (int c = 0; c < NCH; ++c) {
-            a[r][c] = load_sample<SB>(pa[c]);
-            b[r][c] = load_sample<SB>(pb[c]);
-            if (HAS_I) e[r][c] = load_sample<SB>(pe[c]);
-        }
-        if (r + 1 < kAccRows && y0 + r + 1 < H) {  // next row, unless it lies past the view
-            pl += W;
-#pragma unroll
-            for (int c = 0; c < NCH; ++c) {
-                pa[c] += f.pc[c];
-                pb[c] += f.pp[c];
-                if (HAS_I) pe[c] += f.pi[c];
-            }
+            a[r][c] = load_strip<SB, VEC>(static_cast<const char*>(f.cur[c]) + y * f.pc[c] + (int64_t)xc * SB, nx);
+            b[r][c] = load_strip<SB, VEC>(static_cast<const char*>(f.prev[c]) + y * f.pp[c] + (int64_t)xc * SB, nx);
+            if (HAS_I) e[r][c] = load_strip<SB, VEC>(static_cast<const char*>(f.ifr[c]) + y * f.pi[c] + (int64_t)xc * SB, nx);
         }
     }
     int lmin = INT_MAX, lmax = -1;
     bool bad = false;
 #pragma unroll
-    for (int r = 0; r < kAccRows; ++r) {
-        const bool in = x < W && y0 + r < H;
-        if (in && (unsigned)lab[r] < (unsigned)S) {
-            lmin = min(lmin, lab[r]);
-            lmax = max(lmax, lab[r]);
-        } else {
-            bad = bad || in;
-            lab[r] = -1;
+    for (int r = 0; r < kAccRows; ++r)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const bool in = x + k < W && y0 + r < H;
+            if (in && (unsigned)lab[r][k] < (unsigned)S) {
+                lmin = min(lmin, lab[r][k]);
+                lmax = max(lmax, lab[r][k]);
+            } else {
+                bad = bad || in;
+                lab[r][k] = -1;
+            }
         }
-    }
     if (bad) atomicOr(status, ST_BAD_LABEL);
-    for (int i = tid; i < Q * kBins / 4; i += kAccThreads) reinterpret_cast<int4*>(&bins[0][0])[i] = make_int4(0, 0, 0, 0);
     if (tid == 0) {
         s_base = INT_MAX;
         s_top = -1;
@@ -126,53 +147,92 @@ __global__ void __launch_bounds__(kAccThreads) temporal_accumulate_kernel(const 
         atomicMax(&s_top, lmax);
     }
     __syncthreads();
-    const int base = s_base;
+    // the bins in use: the tile's labels from base to s_top (those beyond kBins go to global memory)
+    const int base = s_base, used = min(kBins, s_top - base + 1);
+    for (int i = tid; i < used; i += kAccThreads)
+#pragma unroll
+        for (int q = 0; q < Q; ++q) bins[q][i] = 0;
+    __syncthreads();
 
     // word q of segment s: stats[q * ms + s] (q = 0: n, 1 + c: dP[c], 4 + c: dI[c])
     const int64_t ms = f.ms;
     {
-        int cur = -1;
-        int acc[Q];
+        auto flush = [&](int l, int (&acc)[Q]) {
+            if (l >= 0) {
+                const unsigned bi = (unsigned)(l - base);
+                if (bi < (unsigned)kBins) {
 #pragma unroll
-        for (int q = 0; q < Q; ++q) acc[q] = 0;
-        auto flush = [&]() {
-            const unsigned bi = (unsigned)(cur - base);
-            if (bi < (unsigned)kBins) {
+                    for (int q = 0; q < Q; ++q)
+                        if (q == 0 || acc[q] != 0) atomicAdd(&bins[q][bi], acc[q]);
+                } else {
+                    add64(&stats[l], acc[0]);
 #pragma unroll
-                for (int q = 0; q < Q; ++q)
-                    if (q == 0 || acc[q] != 0) atomicAdd(&bins[q][bi], acc[q]);
-            } else {
-                add64(&stats[cur], acc[0]);
-#pragma unroll
-                for (int c = 0; c < NCH; ++c) {
-                    add64(&stats[(1 + c) * ms + cur], acc[1 + c]);
-                    if (HAS_I) add64(&stats[(4 + c) * ms + cur], acc[1 + NCH + c]);
+                    for (int c = 0; c < NCH; ++c) {
+                        add64(&stats[(1 + c) * ms + l], acc[1 + c]);
+                        if (HAS_I) add64(&stats[(4 + c) * ms + l], acc[1 + NCH + c]);
+                    }
                 }
+            }
+#pragma unroll
+            for (int q = 0; q < Q; ++q) acc[q] = 0;
+        };
+        // adds the pixels of row r with the given 0/1 byte weights to a run of label l
+        auto add = [&](int r, uint32_t w, int (&acc)[Q]) {
+            const uint32_t neg = w * 255u;  // the weights' negatives
+            acc[0] += __popc(w);
+#pragma unroll
+            for (int c = 0; c < NCH; ++c) {
+                const int cur = strip_dot(a[r][c], w, 0);
+                acc[1 + c] = strip_dot(b[r][c], neg, acc[1 + c] + cur);
+                if (HAS_I) acc[1 + NCH + c] = strip_dot(e[r][c], neg, acc[1 + NCH + c] + cur);
             }
         };
+        int la = -1, lb = -1, accA[Q], accB[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) accA[q] = accB[q] = 0;
 #pragma unroll
         for (int r = 0; r < kAccRows; ++r) {
-            const int l = lab[r];
-            if (l != cur) {
-                if (cur >= 0) flush();
-                cur = l;
+            // part A: the label of the first pixel; part B: that of the last one not in A
+            const int l0 = lab[r][0];
+            uint32_t wa = 0, wb = 0;
+            int l1 = -1;
 #pragma unroll
-                for (int q = 0; q < Q; ++q) acc[q] = 0;
+            for (int k = 0; k < 4; ++k) {
+                if (lab[r][k] == l0) wa |= 1u << (8 * k);
+                else l1 = lab[r][k];
             }
-            if (l >= 0) {
-                acc[0] += 1;
 #pragma unroll
-                for (int c = 0; c < NCH; ++c) {
-                    acc[1 + c] += a[r][c] - b[r][c];
-                    if (HAS_I) acc[1 + NCH + c] += a[r][c] - e[r][c];
+            for (int k = 0; k < 4; ++k)
+                if (lab[r][k] == l1) wb |= 1u << (8 * k);
+            if (l0 < 0) wa = 0;
+            if (l1 < 0 || l1 == l0) wb = 0;
+            if (l0 != la) {
+                flush(la, accA);
+                la = l0;
+            }
+            add(r, wa, accA);
+            if (wb) {
+                if (l1 != lb) {
+                    flush(lb, accB);
+                    lb = l1;
                 }
+                add(r, wb, accB);
             }
+            // a third label (narrow segments): pixel by pixel
+#pragma unroll
+            for (int k = 1; k < 4; ++k)
+                if (lab[r][k] >= 0 && !((wa | wb) >> (8 * k) & 1u)) {
+                    int one[Q];
+#pragma unroll
+                    for (int q = 0; q < Q; ++q) one[q] = 0;
+                    add(r, 1u << (8 * k), one);
+                    flush(lab[r][k], one);
+                }
         }
-        if (cur >= 0) flush();
+        flush(la, accA);
+        flush(lb, accB);
     }
     __syncthreads();
-    // the bins in use: the tile's labels from base to s_top (those beyond kBins went to global memory)
-    const int used = min(kBins, s_top - base + 1);
     for (int i = tid; i < used; i += kAccThreads) {
         const int n = bins[0][i];
         if (n == 0) continue;
@@ -348,24 +408,35 @@ cudaError_t launch_temporal_refs(const TemporalRef* refs, int n, int sample_byte
     if (n > kMaxTemporalRefs) return cudaErrorInvalidValue;
     TemporalRefs p{};
     int tx = 0, ty = 0, chunks = 1;
-    bool any_s = false;
+    bool any_s = false, vec = true;
     for (int k = 0; k < n; ++k) {
         p.r[k] = refs[k];
         tx = std::max(tx, (refs[k].W + kAccCols - 1) / kAccCols);
-        ty = std::max(ty, (refs[k].H + kAccGroups * kAccRows - 1) / (kAccGroups * kAccRows));
+        ty = std::max(ty, (refs[k].H + kAccRowsTile - 1) / kAccRowsTile);
+        // four samples (labels) per load where every row of every plane starts on such a boundary
+        uintptr_t at = (reinterpret_cast<uintptr_t>(refs[k].labels) & 15) | (uintptr_t)(refs[k].W & 3);
+        for (int c = 0; c < (mode == FTV_TM_ALL_YUV ? 3 : 1); ++c) {
+            uintptr_t u = reinterpret_cast<uintptr_t>(refs[k].cur[c]) | reinterpret_cast<uintptr_t>(refs[k].prev[c]) |
+                          (uintptr_t)refs[k].pc[c] | (uintptr_t)refs[k].pp[c];
+            if (has_i) u |= reinterpret_cast<uintptr_t>(refs[k].ifr[c]) | (uintptr_t)refs[k].pi[c];
+            at |= u & (uintptr_t)(4 * sample_bytes - 1);
+        }
+        vec = vec && at == 0;
         chunks = std::max(chunks, (refs[k].S + kChunk - 1) / kChunk);
         any_s = any_s || refs[k].S > 0;
     }
     const int nch = mode == FTV_TM_ALL_YUV ? 3 : 1;
     if (tx > 0 && ty > 0) {
         const dim3 block(kAccThreads), grid(tx, ty, n);
-#define FTV_T(SB, NCH, HI) temporal_accumulate_kernel<SB, NCH, HI><<<grid, block, 0, s>>>(p, status)
+#define FTV_T(SB, NCH, HI) \
+    if (vec) temporal_accumulate_kernel<SB, NCH, HI, true><<<grid, block, 0, s>>>(p, status); \
+    else temporal_accumulate_kernel<SB, NCH, HI, false><<<grid, block, 0, s>>>(p, status)
         if (sample_bytes == 1) {
-            if (nch == 1) { if (has_i) FTV_T(1, 1, true); else FTV_T(1, 1, false); }
-            else { if (has_i) FTV_T(1, 3, true); else FTV_T(1, 3, false); }
+            if (nch == 1) { if (has_i) { FTV_T(1, 1, true); } else { FTV_T(1, 1, false); } }
+            else { if (has_i) { FTV_T(1, 3, true); } else { FTV_T(1, 3, false); } }
         } else {
-            if (nch == 1) { if (has_i) FTV_T(2, 1, true); else FTV_T(2, 1, false); }
-            else { if (has_i) FTV_T(2, 3, true); else FTV_T(2, 3, false); }
+            if (nch == 1) { if (has_i) { FTV_T(2, 1, true); } else { FTV_T(2, 1, false); } }
+            else { if (has_i) { FTV_T(2, 3, true); } else { FTV_T(2, 3, false); } }
         }
 #undef FTV_T
         *launches += 1;
