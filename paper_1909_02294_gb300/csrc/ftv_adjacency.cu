@@ -25,6 +25,8 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kHash = 64;        // per-warp neighbour hash slots
 constexpr int kMaxDeg = 32;      // neighbours t > s kept per segment (more sets ST_OVERFLOW)
 constexpr int kWarps = 8;
+constexpr int kFlight = 1;       // pixels per lane in flight
+constexpr int kEdgeLanes = 4;    // threads per segment writing its edges
 
 __device__ __forceinline__ int plane_sample(const void* p, int64_t pitch, int sb, int x, int y) {
     const char* row = static_cast<const char*>(p) + (int64_t)y * pitch;
@@ -44,14 +46,13 @@ struct AdjArgs {
     uint32_t* status;
 };
 
+template <int ND, int SB>
 __global__ void __launch_bounds__(kWarps * 32) neighbours_kernel(AdjArgs a) {
     __shared__ int table[kWarps][kHash];
     __shared__ int list[kWarps][kHash];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     int* tab = table[wib];
     int* lst = list[wib];
-    static const int dxs[8] = {1, -1, 0, 0, 1, 1, -1, -1}, dys[8] = {0, 0, 1, -1, 1, -1, 1, -1};
-    const int ndir = a.conn == 8 ? 8 : 4;
     for (int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < a.S; s += (gridDim.x * blockDim.x) >> 5) {
         tab[lane] = -1;
         tab[lane + 32] = -1;
@@ -59,25 +60,49 @@ __global__ void __launch_bounds__(kWarps * 32) neighbours_kernel(AdjArgs a) {
         const int b = a.offs[s], e = a.offs[s + 1];
         long long sy = 0, su = 0, sv = 0;
         bool full = false;
-        for (int i = b + lane; i < e; i += 32) {
-            const uint32_t xy = a.pix[i];
-            const int x = xy & 0xffff, y = xy >> 16;
-            sy += plane_sample(a.plane[0], a.pitch[0], a.sb, x, y);
-            su += plane_sample(a.plane[1], a.pitch[1], a.sb, x, y);
-            sv += plane_sample(a.plane[2], a.pitch[2], a.sb, x, y);
-            for (int k = 0; k < ndir; ++k) {
-                const int qx = x + dxs[k], qy = y + dys[k];
-                if (qx < 0 || qx >= a.W || qy < 0 || qy >= a.H) continue;
-                const int t = a.labels[(int64_t)qy * a.W + qx];
-                if (t <= s || t >= a.S) continue;
-                int h = (int)((unsigned)t * 2654435761u >> 26);  // top 6 bits: 0..63
-                int probes = 0;
-                for (; probes < kHash; ++probes) {
-                    const int old = atomicCAS(&tab[h], -1, t);
-                    if (old == -1 || old == t) break;
-                    h = (h + 1) & (kHash - 1);
+        for (int i0 = b; i0 < e; i0 += 32 * kFlight) {
+            // kFlight pixels per lane: their records, then their samples and neighbours' labels, each stage's loads
+            // in flight together
+            uint32_t xy[kFlight];
+#pragma unroll
+            for (int u = 0; u < kFlight; ++u) {
+                const int i = i0 + 32 * u + lane;
+                xy[u] = i < e ? __ldg(&a.pix[i]) : 0xffffffffu;
+            }
+            int t[kFlight][ND], v[kFlight][3];
+#pragma unroll
+            for (int u = 0; u < kFlight; ++u) {
+                const bool in = xy[u] != 0xffffffffu;
+                const int x = xy[u] & 0xffff, y = xy[u] >> 16;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) v[u][c] = in ? plane_sample(a.plane[c], a.pitch[c], SB, x, y) : 0;
+#pragma unroll
+                for (int k = 0; k < ND; ++k) {
+                    const int dx = k == 0 || k == 4 || k == 5 ? 1 : (k == 1 || k >= 6 ? -1 : 0);
+                    const int dy = k == 2 || k == 4 || k == 6 ? 1 : (k == 3 || k == 5 || k == 7 ? -1 : 0);
+                    const int qx = x + dx, qy = y + dy;
+                    t[u][k] = in && qx >= 0 && qx < a.W && qy >= 0 && qy < a.H
+                                  ? __ldg(&a.labels[(int64_t)qy * a.W + qx]) : s;
                 }
-                if (probes == kHash) full = true;
+            }
+#pragma unroll
+            for (int u = 0; u < kFlight; ++u) {
+                sy += v[u][0];
+                su += v[u][1];
+                sv += v[u][2];
+#pragma unroll
+                for (int k = 0; k < ND; ++k) {
+                    const int q = t[u][k];
+                    if (q <= s || q >= a.S) continue;
+                    int h = (int)((unsigned)q * 2654435761u >> 26);  // top 6 bits: 0..63
+                    int probes = 0;
+                    for (; probes < kHash; ++probes) {
+                        const int old = atomicCAS(&tab[h], -1, q);
+                        if (old == -1 || old == q) break;
+                        h = (h + 1) & (kHash - 1);
+                    }
+                    if (probes == kHash) full = true;
+                }
             }
         }
         for (int o = 16; o > 0; o >>= 1) {
@@ -114,54 +139,15 @@ __global__ void __launch_bounds__(kWarps * 32) neighbours_kernel(AdjArgs a) {
     }
 }
 
-__device__ int block_scan_adj(int v, int* total) {
-    __shared__ int warp_sums[32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = v;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += t;
-    }
-    if (lane == 31) warp_sums[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        int x = lane < (int)(blockDim.x >> 5) ? warp_sums[lane] : 0;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(kFull, x, o);
-            if (lane >= o) x += t;
-        }
-        warp_sums[lane] = x;
-    }
-    __syncthreads();
-    const int base = warp > 0 ? warp_sums[warp - 1] : 0;
-    *total = warp_sums[(blockDim.x >> 5) - 1];
-    __syncthreads();
-    return base + incl - v;
-}
-
-// One block of 1024 threads: edge offsets from the per-segment counts, and the edge count.
-__global__ void edge_offsets_kernel(const int32_t* __restrict__ deg, int S, int32_t* __restrict__ offs,
-                                    int32_t* n_edges) {
-    const int per = (S + blockDim.x - 1) / blockDim.x;
-    const int b = threadIdx.x * per, e = min(S, b + per);
-    int sum = 0;
-    for (int s = b; s < e; ++s) sum += deg[s];
-    int total;
-    int run = block_scan_adj(sum, &total);
-    for (int s = b; s < e; ++s) {
-        offs[s] = run;
-        run += deg[s];
-    }
-    if (threadIdx.x == 0) *n_edges = total;
-}
-
 __global__ void edges_kernel(const int32_t* __restrict__ deg, const int32_t* __restrict__ slots,
                              const int32_t* __restrict__ offs, const int64_t* __restrict__ stats, int S, int cap,
                              double beta0, double min_diff, int32_t* __restrict__ es, int32_t* __restrict__ et,
                              float* __restrict__ beta) {
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < S; s += gridDim.x * blockDim.x) {
+    // kEdgeLanes threads per segment: a segment has few edges, and one thread's would wait on one another
+    for (int64_t i = blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)S * kEdgeLanes; i += gridDim.x * blockDim.x) {
+        const int s = (int)(i / kEdgeLanes), n = deg[s];
         const int64_t* A = stats + (int64_t)s * 4;
-        for (int j = 0; j < deg[s]; ++j) {
+        for (int j = (int)(i % kEdgeLanes); j < n; j += kEdgeLanes) {
             const int e = offs[s] + j;
             if (e >= cap) break;
             const int t = slots[(int64_t)s * kMaxDeg + j];
@@ -229,13 +215,19 @@ extern "C" ftv_status ftv_adjacency(ftv_ctx* ctx, int32_t ref_index, const void*
         a.slots = ctx->d_adj_slots;
         a.status = ctx->d_status;
         const int blocks = std::max(1, std::min(65535, (n_segments + kWarps - 1) / kWarps));
-        neighbours_kernel<<<blocks, kWarps * 32, 0, s>>>(a);
-        edge_offsets_kernel<<<1, 1024, 0, s>>>(ctx->d_adj_deg, n_segments, ctx->d_adj_offs, d_n_edges);
-        edges_kernel<<<std::max(1, std::min(65535, (n_segments + 255) / 256)), 256, 0, s>>>(
+        if (connectivity == 4) {
+            if (a.sb == 1) neighbours_kernel<4, 1><<<blocks, kWarps * 32, 0, s>>>(a);
+            else neighbours_kernel<4, 2><<<blocks, kWarps * 32, 0, s>>>(a);
+        } else {
+            if (a.sb == 1) neighbours_kernel<8, 1><<<blocks, kWarps * 32, 0, s>>>(a);
+            else neighbours_kernel<8, 2><<<blocks, kWarps * 32, 0, s>>>(a);
+        }
+        e = launch_prefix(ctx->d_adj_deg, n_segments, ctx->d_adj_offs, d_n_edges, s);
+        edges_kernel<<<std::max(1, std::min(65535, (int)(((int64_t)n_segments * kEdgeLanes + 255) / 256))), 256, 0, s>>>(
             ctx->d_adj_deg, ctx->d_adj_slots, ctx->d_adj_offs, scratch, n_segments, capacity, beta0, min_diff,
             d_edge_s, d_edge_t, d_beta);
         ctx->launches += 3;
-        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaGetLastError();
     } else if (e == cudaSuccess) {
         e = cudaMemsetAsync(d_n_edges, 0, sizeof(int32_t), s);
     }

@@ -49,14 +49,14 @@ void free_ctx(ftv_ctx* c) {
         cudaFree(r.d_offs);
         cudaFree(r.d_recs);
         cudaFree(r.d_tiles);
-        cudaFree(r.d_woffs);
+        cudaFree(r.d_cursor);
         cudaFree(r.d_pix);
         cudaFree(r.d_centre);
         cudaFree(r.d_nbr_labels);
     }
     cudaFree(c->d_packed);
     cudaFree(c->d_status);
-    cudaFree(c->d_cursors);
+    cudaFree(c->d_woffs_all);
     cudaFree(c->d_jobs);
     cudaFree(c->d_plan);
     cudaFree(c->d_tstats);
@@ -81,7 +81,8 @@ int64_t max_pixel_cost(const ftv_ctx* c, int n_nbrs) {
 // Reference `ref` of a context with a label map, as launch_segment_index takes it.
 IndexRef ftv::index_ref(const ftv_ctx* c, int ref, const int32_t* labels, int n_segments) {
     const RefState& r = c->refs[ref];
-    return {labels, r.d_offs, r.d_cursor, r.d_pix, max_pixel_cost(c, r.n_nbrs), r.W, r.H, n_segments, c->max_segments};
+    return {labels, r.d_offs, r.d_woffs, r.d_cursor, r.d_pix, max_pixel_cost(c, r.n_nbrs), r.W, r.H, n_segments,
+            c->max_segments + 1, 0};
 }
 
 // View v of a context packed at byte `offset` of the allocation `base`, as the kernels see it.
@@ -271,7 +272,7 @@ ftv_status ftv_depth_init(const ftv_config* cfg, ftv_ctx** out) {
     ok = ok && dalloc(&c->d_status, 1) == cudaSuccess;
     ok = ok && dalloc(&c->d_jobs, kMaxUnits) == cudaSuccess;
     ok = ok && dalloc(&c->d_plan, 1) == cudaSuccess && cudaMemset(c->d_plan, 0, sizeof(Plan)) == cudaSuccess;
-    ok = ok && dalloc(&c->d_cursors, (size_t)c->n_refs * c->max_segments) == cudaSuccess;
+    ok = ok && dalloc(&c->d_woffs_all, (size_t)c->n_refs * ((size_t)c->max_segments + 1)) == cudaSuccess;
     ok = ok && dalloc(&c->d_tstats, (size_t)std::max(1, c->n_refs) * c->max_segments * 8) == cudaSuccess;
     c->tstats_zero.assign(c->n_refs, 0);
     ok = ok && dalloc(&c->d_label_z, (size_t)c->L) == cudaSuccess;
@@ -283,10 +284,10 @@ ftv_status ftv_depth_init(const ftv_config* cfg, ftv_ctx** out) {
         if (c->precision == FTV_PRECISION_FP64) ok = ok && dalloc(&r.d_H64, r.h_H64.size()) == cudaSuccess;
         ok = ok && dalloc(&r.d_nbrs, (size_t)r.n_nbrs * 2) == cudaSuccess;
         ok = ok && dalloc(&r.d_offs, (size_t)c->max_segments + 1) == cudaSuccess;
-        r.d_cursor = c->d_cursors ? c->d_cursors + (&r - c->refs.data()) * (size_t)c->max_segments : nullptr;
+        ok = ok && dalloc(&r.d_cursor, (size_t)c->max_segments) == cudaSuccess;
         ok = ok && dalloc(&r.d_recs, (size_t)tiles_of((int64_t)r.W * r.H) * kTile) == cudaSuccess;
         ok = ok && dalloc(&r.d_tiles, (size_t)tiles_of((int64_t)r.W * r.H)) == cudaSuccess;
-        ok = ok && dalloc(&r.d_woffs, (size_t)c->max_segments + 1) == cudaSuccess;
+        r.d_woffs = c->d_woffs_all ? c->d_woffs_all + (&r - c->refs.data()) * ((size_t)c->max_segments + 1) : nullptr;
         ok = ok && dalloc(&r.d_pix, (size_t)r.W * r.H) == cudaSuccess;
         ok = ok && dalloc(&r.d_centre, (size_t)c->max_segments) == cudaSuccess;
         ok = ok && dalloc(&r.d_nbr_labels, (size_t)std::max(1, r.n_nbrs)) == cudaSuccess;

@@ -108,24 +108,44 @@ struct IndexArgs {
     IndexRef r[CAP];
 };
 
-// Per-segment pixel counts (blockIdx.z: the reference). Lanes of a warp that hold the same label (a run along
-// the row) add their count with one atomic.
-template <int CAP>
-__global__ void histogram_kernel(const __grid_constant__ IndexArgs<CAP> args, uint32_t* status) {
-    const IndexRef& R = args.r[blockIdx.z];
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y;
-    if (y >= R.H) return;
-    const bool in = x < R.W;
-    const int l = in ? __ldg(&R.labels[(int64_t)y * R.W + x]) : -1;
-    const bool ok = in && (unsigned)l < (unsigned)R.S;
-    if (in && !ok) atomicOr(status, ST_BAD_LABEL);
-    const unsigned active = __ballot_sync(kFull, ok);
-    if (ok) {
-        const unsigned peers = __match_any_sync(active, l);
-        const int lane = threadIdx.x & 31;
-        if (lane == __ffs(peers) - 1) atomicAdd(&R.cursor[l], __popc(peers));
+// Four adjacent labels of a row (-1 past its end), in one load where the map allows.
+__device__ __forceinline__ void load_labels(const IndexRef& R, int x, int y, int* l) {
+    const int32_t* p = R.labels + (int64_t)y * R.W + x;
+    if (R.vec && x + 4 <= R.W) {
+        const int4 t = __ldg(reinterpret_cast<const int4*>(p));
+        l[0] = t.x;
+        l[1] = t.y;
+        l[2] = t.z;
+        l[3] = t.w;
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) l[k] = x + k < R.W ? __ldg(p + k) : -1;
     }
+}
+
+// Per-segment pixel counts (blockIdx.z: the reference). A thread counts the runs among its four adjacent pixels; a run
+// that continues into the next thread's pixels is carried on by an addition of its own (a segment's row is two or
+// three runs then, each one atomic; matching equal labels over the warp's pixels cost more than it saved).
+template <int CAP>
+__global__ void __launch_bounds__(128) histogram_kernel(const __grid_constant__ IndexArgs<CAP> args, uint32_t* status) {
+    const IndexRef& R = args.r[blockIdx.z];
+    const int x = (blockIdx.x * blockDim.x + threadIdx.x) * 4, y = blockIdx.y;
+    if (y >= R.H || x >= R.W) return;
+    int l[4];
+    load_labels(R, x, y, l);
+    bool bad = false;
+    int n = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const bool ok = (unsigned)l[k] < (unsigned)R.S;
+        bad = bad || (!ok && x + k < R.W);
+        n = ok ? n + 1 : 0;
+        if (ok && (k == 3 || l[k + 1 < 4 ? k + 1 : k] != l[k])) {
+            atomicAdd(&R.counts[l[k]], n);
+            n = 0;
+        }
+    }
+    if (bad) atomicOr(status, ST_BAD_LABEL);
 }
 
 // Block-wide exclusive scan of one int per thread (blockDim.x == 1024). Returns the exclusive prefix;
@@ -156,54 +176,96 @@ __device__ int block_exclusive_scan(int v, int* total) {
     return base + incl - v;
 }
 
-// Counts (in `cursor`) -> offsets[S + 1]; cursor[s] = offsets[s] for the scatter. One block of 1024 per
-// reference, which scans chunks of 1024 counts with the next chunk's load in flight (coalesced; one thread per
-// contiguous stretch read the same counts in 25 us for 20736 segments, this takes about 10).
-// Also checks that no segment is large enough for its int32 cost sum to overflow.
+// Exclusive prefix of n counts by blocks of 1024, each of kScanChunk counts (eight consecutive ones per thread, read and
+// written coalesced through shared memory): block b adds up the counts of the blocks before it (independent loads),
+// then scans its own. out, and out2 where it is given, receive the prefix, *total (by the last block) the sum.
+// One block walking the counts took 25 us for 20736 segments one stretch per thread, 9 us chunk by chunk; this 5.
+constexpr int kScanPer = 8, kScanChunk = 1024 * kScanPer;
+__device__ void scan_counts(const int32_t* __restrict__ in, int n, int32_t* out, int32_t* out2, int32_t* total, int* mx) {
+    __shared__ int sm[kScanChunk + kScanChunk / 32];
+    __shared__ int s_before;
+    auto at = [](int i) { return i + (i >> 5); };  // padded against bank conflicts
+    const int b = blockIdx.x * kScanChunk;
+    if (b >= n && b > 0) return;  // uniform: past this reference's counts
+    if (threadIdx.x == 0) s_before = 0;
+#pragma unroll
+    for (int k = 0; k < kScanPer; ++k) {
+        const int i = k * 1024 + threadIdx.x;
+        sm[at(i)] = b + i < n ? in[b + i] : 0;
+    }
+    int before = 0;
+#pragma unroll 8
+    for (int i = threadIdx.x; i < b; i += 1024) before += in[i];
+    before = __reduce_add_sync(kFull, before);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0 && before) atomicAdd(&s_before, before);
+    int c[kScanPer], sum = 0;
+#pragma unroll
+    for (int k = 0; k < kScanPer; ++k) {
+        c[k] = sm[at(threadIdx.x * kScanPer + k)];
+        sum += c[k];
+        *mx = max(*mx, c[k]);
+    }
+    int all;
+    int p = block_exclusive_scan(sum, &all) + s_before;  // its barriers order the additions to s_before
+#pragma unroll
+    for (int k = 0; k < kScanPer; ++k) {
+        sm[at(threadIdx.x * kScanPer + k)] = p;
+        p += c[k];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kScanPer; ++k) {
+        const int i = k * 1024 + threadIdx.x;
+        if (b + i < n) {
+            out[b + i] = sm[at(i)];
+            if (out2) out2[b + i] = sm[at(i)];
+        }
+    }
+    if (b + kScanChunk >= n && threadIdx.x == 0) *total = s_before + all;
+}
+
+// Counts -> offsets[S + 1]; cursor[s] = offsets[s] for the scatter. Also checks that no segment is large enough for its
+// int32 cost sum to overflow.
 template <int CAP>
 __global__ void __launch_bounds__(1024) offsets_kernel(const __grid_constant__ IndexArgs<CAP> args, uint32_t* status) {
-    const IndexRef& R = args.r[blockIdx.x];
-    const int S = R.S;
-    int run = 0, mx = 0;
-    int next = (int)threadIdx.x < S ? R.cursor[threadIdx.x] : 0;
-    for (int b = 0; b < S; b += 1024) {
-        const int s = b + threadIdx.x, c = next;
-        next = s + 1024 < S ? R.cursor[s + 1024] : 0;
-        int total;
-        const int at = run + block_exclusive_scan(c, &total);
-        if (s < S) {
-            R.offs[s] = at;
-            R.cursor[s] = at;
-        }
-        mx = max(mx, c);
-        run += total;
-    }
-    if (threadIdx.x == 0) R.offs[S] = run;
+    const IndexRef& R = args.r[blockIdx.y];
+    int mx = 0;
+    scan_counts(R.counts, R.S, R.offs, R.cursor, R.offs + R.S, &mx);
     mx = __reduce_max_sync(kFull, mx);
     if ((threadIdx.x & 31) == 0 && (int64_t)mx * R.max_pix_cost > (int64_t)INT32_MAX) atomicOr(status, ST_OVERFLOW);
 }
 
-// Scatter (y << 16 | x) records into their segment's range. A warp's run of equal labels takes one
-// atomic and keeps its left-to-right order.
+__global__ void __launch_bounds__(1024) prefix_kernel(const int32_t* counts, int n, int32_t* offs, int32_t* total) {
+    int mx = 0;
+    scan_counts(counts, n, offs, nullptr, total, &mx);
+}
+
+// Scatter (y << 16 | x) records into their segment's range. A warp's run of equal labels takes one atomic and keeps
+// its left-to-right order (the cost kernel's gathers follow this order: one atomic per run of a thread's four pixels
+// made it 3 % slower on the 1920x1080 rig). kScatterRows rows per warp, their atomics in flight together.
+constexpr int kScatterRows = 4;
 template <int CAP>
-__global__ void scatter_kernel(const __grid_constant__ IndexArgs<CAP> args) {
+__global__ void __launch_bounds__(256) scatter_kernel(const __grid_constant__ IndexArgs<CAP> args) {
     const IndexRef& R = args.r[blockIdx.z];
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y;
-    if (y >= R.H) return;
-    const bool in = x < R.W;
-    const int l = in ? __ldg(&R.labels[(int64_t)y * R.W + x]) : -1;
-    const bool ok = in && (unsigned)l < (unsigned)R.S;
-    const unsigned active = __ballot_sync(kFull, ok);
-    if (ok) {
-        const unsigned peers = __match_any_sync(active, l);
-        const int lane = threadIdx.x & 31;
-        const int leader = __ffs(peers) - 1;
-        int base = 0;
-        if (lane == leader) base = atomicAdd(&R.cursor[l], __popc(peers));
-        base = __shfl_sync(peers, base, leader);
-        const int rank = __popc(peers & ((1u << lane) - 1u));
-        R.pix[base + rank] = ((uint32_t)y << 16) | (uint32_t)x;
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, y0 = blockIdx.y * kScatterRows;
+    if (y0 >= R.H) return;
+    const int lane = threadIdx.x & 31;
+    int l[kScatterRows], at[kScatterRows];
+    unsigned peers[kScatterRows];
+#pragma unroll
+    for (int r = 0; r < kScatterRows; ++r) l[r] = x < R.W && y0 + r < R.H ? __ldg(&R.labels[(int64_t)(y0 + r) * R.W + x]) : -1;
+#pragma unroll
+    for (int r = 0; r < kScatterRows; ++r) {
+        if ((unsigned)l[r] >= (unsigned)R.S) l[r] = -1;
+        peers[r] = __match_any_sync(kFull, l[r]);
+        at[r] = 0;
+        if (l[r] >= 0 && lane == __ffs(peers[r]) - 1) at[r] = atomicAdd(&R.cursor[l[r]], __popc(peers[r]));
+    }
+#pragma unroll
+    for (int r = 0; r < kScatterRows; ++r) {
+        const int base = __shfl_sync(kFull, at[r], __ffs(peers[r]) - 1);
+        if (l[r] >= 0) R.pix[base + __popc(peers[r] & ((1u << lane) - 1u))] = ((uint32_t)(y0 + r) << 16) | (uint32_t)x;
     }
 }
 
@@ -497,24 +559,26 @@ cudaError_t launch_segment_index(const IndexRef* refs, int n, uint32_t* status, 
     if (n <= 0) return cudaSuccess;
     if (n > kCap) return cudaErrorInvalidValue;
     IndexArgs<kCap> args;
-    int W = 1, H = 1;
+    int W = 1, H = 1, S = 1;
     for (int k = 0; k < n; ++k) {
         args.r[k] = refs[k];
+        args.r[k].vec = (reinterpret_cast<uintptr_t>(refs[k].labels) & 15) == 0 && refs[k].W % 4 == 0;
         W = std::max(W, refs[k].W);
         H = std::max(H, refs[k].H);
-        // the references' counters lie one after the other: one clear for a run of them
-        if (k == 0 || refs[k].cursor != refs[k - 1].cursor + refs[k - 1].stride) {
+        S = std::max(S, refs[k].S);
+        // the references' counts lie one after the other: one clear for a run of them
+        if (k == 0 || refs[k].counts != refs[k - 1].counts + refs[k - 1].stride) {
             size_t words = refs[k].S > 0 ? refs[k].S : 1;
-            for (int j = k + 1; j < n && refs[j].cursor == refs[j - 1].cursor + refs[j - 1].stride; ++j)
-                words = (size_t)(refs[j].cursor - refs[k].cursor) + refs[j].S;
-            const cudaError_t e = cudaMemsetAsync(refs[k].cursor, 0, sizeof(int32_t) * words, s);
+            for (int j = k + 1; j < n && refs[j].counts == refs[j - 1].counts + refs[j - 1].stride; ++j)
+                words = (size_t)(refs[j].counts - refs[k].counts) + refs[j].S;
+            const cudaError_t e = cudaMemsetAsync(refs[k].counts, 0, sizeof(int32_t) * words, s);
             if (e != cudaSuccess) return e;
         }
     }
-    const dim3 block(256), grid((W + 255) / 256, H, n);
+    const dim3 block(128), grid((W + 511) / 512, H, n);
     histogram_kernel<kCap><<<grid, block, 0, s>>>(args, status);
-    offsets_kernel<kCap><<<n, 1024, 0, s>>>(args, status);
-    scatter_kernel<kCap><<<grid, block, 0, s>>>(args);
+    offsets_kernel<kCap><<<dim3((S + kScanChunk - 1) / kScanChunk, n), 1024, 0, s>>>(args, status);
+    scatter_kernel<kCap><<<dim3((W + 255) / 256, (H + kScatterRows - 1) / kScatterRows, n), 256, 0, s>>>(args);
     *launches += 3;
     return cudaGetLastError();
 }
@@ -539,6 +603,11 @@ cudaError_t launch_plan(const RefJob* host_jobs, int n_jobs, int slots, RefJob* 
     if (n_jobs < 0 || n_jobs > FTV_MAX_VIEWS) return cudaErrorInvalidValue;  // one unit per reference
     if (n_jobs <= 16) return launch_plan_cap<16>(host_jobs, n_jobs, slots, d_jobs, plan, s);
     return launch_plan_cap<FTV_MAX_VIEWS>(host_jobs, n_jobs, slots, d_jobs, plan, s);
+}
+
+cudaError_t launch_prefix(const int32_t* counts, int n, int32_t* offs, int32_t* total, cudaStream_t s) {
+    prefix_kernel<<<std::max(1, (n + kScanChunk - 1) / kScanChunk), 1024, 0, s>>>(counts, n, offs, total);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_tiles(const RefJob* jobs, const Plan* plan, int grid, cudaStream_t s) {

@@ -107,10 +107,10 @@ struct RefState {
     double* d_H64 = nullptr;   // [N][L][9] unrounded table (FP64-precision contexts only)
     NbrView* d_nbrs = nullptr; // [2][N]: views packed in cost_fmt, then in fmt (both in the context's d_packed)
     int32_t* d_offs = nullptr;   // [max_segments + 1]
-    int32_t* d_cursor = nullptr; // [max_segments], in the context's d_cursors
+    int32_t* d_cursor = nullptr; // [max_segments]
     int2* d_recs = nullptr;      // [tiles * kTile] tile records
     int4* d_tiles = nullptr;     // [tiles]
-    int32_t* d_woffs = nullptr;  // [max_segments + 1]
+    int32_t* d_woffs = nullptr;  // [max_segments + 1], in the context's d_woffs_all; also the index's counts
     uint32_t* d_pix = nullptr;   // [W * H]
     int32_t S_indexed = -1;      // segment count of the cached index (-1: none)
     int2* d_centre = nullptr;    // [max_segments] segment centres (centre table)
@@ -172,7 +172,7 @@ struct ftv_ctx {
     std::vector<size_t> cost_offset_bytes;    // byte offset of each view packed in cost_fmt
     size_t cost_texel_bytes = 4;
     uint32_t* d_status = nullptr;
-    int32_t* d_cursors = nullptr;             // [n_refs][max_segments] segment index counters
+    int32_t* d_woffs_all = nullptr;           // [n_refs][max_segments + 1]
     ftv::RefJob* d_jobs = nullptr;            // [n_refs]
     ftv::Plan* d_plan = nullptr;
     int64_t* d_tstats = nullptr;              // per reference: temporal sums, 8 planes of max_segments (adjacency scratch)
@@ -224,11 +224,13 @@ cudaError_t launch_pack(const PackView* views, int n, int sample_bytes, int bit_
 struct IndexRef {
     const int32_t* labels;  // [H][W]
     int32_t* offs;          // [S + 1]
-    int32_t* cursor;        // [S] scratch
+    int32_t* counts;        // [S] scratch: pixels per segment
+    int32_t* cursor;        // [S] scratch: next record of each segment
     uint32_t* pix;          // [H * W]
     int64_t max_pix_cost;
     int32_t W, H, S;
-    int32_t stride;         // words from this reference's cursor to the next one's in the same allocation
+    int32_t stride;         // words from this reference's counts to the next one's in the same allocation
+    int32_t vec;            // set by launch_segment_index: four labels per load
 };
 cudaError_t launch_segment_index(const IndexRef* refs, int n, uint32_t* status, cudaStream_t s, int64_t* launches);
 constexpr int kMaxUnits = 240;  // (job, reference) units per launch
@@ -237,6 +239,8 @@ cudaError_t launch_plan(const RefJob* host_jobs, int n_jobs, int slots, RefJob* 
 // Same plan for descriptors already in device memory (completed in place); the unit count is read from
 // *n_jobs on the device, so one captured launch serves any batch composition.
 cudaError_t launch_plan_device(RefJob* d_jobs, const int32_t* n_jobs, int max_jobs, int slots, Plan* plan, cudaStream_t s);
+// Exclusive prefix of n counts and their total.
+cudaError_t launch_prefix(const int32_t* counts, int n, int32_t* offs, int32_t* total, cudaStream_t s);
 // Tile records of every planned unit, and its listed cost rows cleared.
 cudaError_t launch_tiles(const RefJob* jobs, const Plan* plan, int grid, cudaStream_t s);
 inline int64_t tiles_of(int64_t pixels) { return (pixels + kTile - 1) / kTile; }
