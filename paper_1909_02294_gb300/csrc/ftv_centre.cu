@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(kCentreThreads, 4) centre_table3_kernel(Centre
 }
 
 // One 3x3 window pair's sum for 4-byte texels: t[i] the neighbour's packed texels (Y | Cb << sh | Cr << 2 sh),
-// ref[i] the reference's samples (Y, Cb, Cr, unused), read from shared memory (one broadcast load each).
+// ref[i] the reference's samples (Y, Cb, Cr, packed), read from shared memory (one broadcast load each).
 // Each window row accumulates in its own chain (three independent chains of nine absolute differences
 // instead of one of 27), which shortens the dependent path of an entry.
 template <int FMT>
@@ -304,8 +304,12 @@ __device__ __forceinline__ int window_sum(const uint32_t* t, const int4* ref) {
     unsigned m[3] = {0u, 0u, 0u};
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
-        const int4 r = ref[i];
         unsigned& a = m[i / 3];
+        if (FMT == FMT_U8X4) {  // 8-bit samples: one packed absolute difference per texel
+            a += __vsadu4(t[i], (unsigned)ref[i].w);
+            continue;
+        }
+        const int4 r = ref[i];
         a = __sad(t[i] & mk, (unsigned)r.x, __sad((t[i] >> sh) & mk, (unsigned)r.y, __sad(t[i] >> (2 * sh), (unsigned)r.z, a)));
     }
     return (int)(m[0] + m[1] + m[2]);
@@ -321,11 +325,15 @@ __device__ __forceinline__ int window_sum(const uint32_t* t, const int4* ref) {
 // per item). Within a group each thread software-pipelines its segments: the next segment's projection is
 // computed while the current window's nine gathers are in flight. Windows that touch an image border take
 // the checked loop. The reciprocal is the Newton-Raphson step where the start-up check found it exact.
+// An integer-shift entry (rectified rigs) is one addition instead of the projection. 1920x1080, 8 references x 250 labels
+// x 7 neighbours: 167 instructions per entry, 0.317 ms per reference and launch; writing the results contiguously
+// through shared memory (the output has the neighbours innermost, a warp's words lie N apart) relieved the L2 from 57 to
+// 15 % busy but took 204 instructions and 0.346 ms.
 constexpr int kGroup = 16;
 static_assert(9 * kGroup <= kCentreThreads, "one stage sample per thread");
 
 struct CentreStage {
-    int4 ref[kGroup * 9];  // reference samples (Y, Cb, Cr, 0), segment-major
+    int4 ref[kGroup * 9];  // reference samples (Y, Cb, Cr, packed texel), segment-major
     int2 c[kGroup];        // centres; (-1, -1) for an empty segment
     int inside[kGroup];    // the segment's 3x3 window lies inside the reference image
 };
@@ -357,11 +365,24 @@ __device__ __forceinline__ void store_stage(const CentreArgs& a, CentreStage& st
     constexpr uint32_t mk = (1u << sh) - 1u;
     if (!r.valid) return;
     const int g = tid / 9;
-    st.ref[tid] = make_int4((int)(r.w & mk), (int)((r.w >> sh) & mk), (int)(r.w >> (2 * sh)), 0);
+    st.ref[tid] = make_int4((int)(r.w & mk), (int)((r.w >> sh) & mk), (int)(r.w >> (2 * sh)), (int)r.w);
     if (tid - 9 * g == 0) {
         st.c[g] = r.c;
         st.inside[g] = r.c.x >= 1 && r.c.x + 1 < a.W && r.c.y >= 1 && r.c.y + 1 < a.H_;
     }
+}
+
+// Whether an FP32 entry maps every pixel (x, y) below 2^15 to (x + D, y), as the contract's sequence rounds: a unit
+// homography that keeps the row (|h5| < 0.25) and moves the column by h2, where h2 + 0.5 lies more than
+// 2^-23 (2^15 + |h2|) from every integer, so that neither rounding of x + h2 and + 0.5 crosses one (the cost kernel's
+// integer-shift entries, ftv_cost.cu).
+__device__ __forceinline__ bool shift_entry(const float (&h)[9], int& D) {
+    if (!(h[0] == 1.0f && h[1] == 0.0f && h[3] == 0.0f && h[4] == 1.0f && h[6] == 0.0f && h[7] == 0.0f && h[8] == 1.0f &&
+          fabsf(h[5]) < 0.25f && fabsf(h[2]) < 0x1p20f))
+        return false;
+    const double h2 = (double)h[2], f = floor(h2 + 0.5), g = h2 + 0.5 - f;
+    D = (int)f;
+    return fmin(g, 1.0 - g) > 0x1p-23 * (32768.0 + fabs(h2));
 }
 
 // The projection of a segment centre through one entry (the contract's FP32 sequence) and the fast-path test.
@@ -371,11 +392,19 @@ struct CentreProj {
     bool in, fast;
 };
 
+// shift: an integer-shift entry (shift_entry), whose sample is (x + D, y) with D in h[2]'s bits.
 template <bool FAST>
-__device__ __forceinline__ CentreProj project_entry(const float (&h)[9], const CentreStage& st, int g, int w,
+__device__ __forceinline__ CentreProj project_entry(const float (&h)[9], bool shift, const CentreStage& st, int g, int w,
                                                     int hgt) {
     CentreProj p{st.c[g], 0, 0, false, false};
     if (p.c.x < 0) return p;
+    if (shift) {
+        p.ui = p.c.x + __float_as_int(h[2]);
+        p.vi = p.c.y;
+        p.in = (unsigned)p.ui < (unsigned)w && p.vi < hgt;
+        p.fast = st.inside[g] && p.ui >= 1 && p.ui + 1 < w && p.vi + 1 < hgt;
+        return p;
+    }
     const float x = (float)p.c.x, y = (float)p.c.y;
     const float X = __fmaf_rn(h[0], x, __fmaf_rn(h[1], y, h[2]));
     const float Yh = __fmaf_rn(h[3], x, __fmaf_rn(h[4], y, h[5]));
@@ -414,6 +443,9 @@ __global__ void __launch_bounds__(kCentreThreads, 4) centre_table3t_kernel(Centr
             float h[9];
 #pragma unroll
             for (int i = 0; i < 9; ++i) h[i] = __ldg(a.H + (int64_t)j * 9 + i);
+            int D = 0;
+            const bool shift = shift_entry(h, D);
+            if (shift) h[2] = __int_as_float(D);
             const NbrView nv = a.nbrs[k];
             const int32_t* lv = a.labels_v[k];
             const uint32_t* tex = static_cast<const uint32_t*>(nv.texels);
@@ -421,7 +453,7 @@ __global__ void __launch_bounds__(kCentreThreads, 4) centre_table3t_kernel(Centr
             const int s0 = group * kGroup, n = min(kGroup, a.S - s0);
             int32_t* mp = a.m + (int64_t)s0 * nent + (int64_t)d * a.N + k;
             int32_t* spp = a.sp + (int64_t)s0 * nent + (int64_t)d * a.N + k;
-            CentreProj cur = project_entry<FAST>(h, cs, 0, nv.w, nv.h);
+            CentreProj cur = project_entry<FAST>(h, shift, cs, 0, nv.w, nv.h);
             for (int g = 0; g < n; ++g) {
                 uint32_t t[9];
                 if (cur.fast) {
@@ -433,7 +465,7 @@ __global__ void __launch_bounds__(kCentreThreads, 4) centre_table3t_kernel(Centr
                 }
                 const int spv = (cur.in && lv) ? __ldg(lv + (int64_t)cur.vi * nv.w + cur.ui) : -1;
                 CentreProj nxt{};
-                if (g + 1 < n) nxt = project_entry<FAST>(h, cs, g + 1, nv.w, nv.h);
+                if (g + 1 < n) nxt = project_entry<FAST>(h, shift, cs, g + 1, nv.w, nv.h);
                 int m;
                 if (cur.fast) {
                     m = window_sum<FMT>(t, cs.ref + 9 * g);
