@@ -358,75 +358,83 @@ __device__ __forceinline__ bool shift_fp64(const double* __restrict__ hg, int& D
 // instead of 2^-24 of the image coordinates. The bound delta covers, at every pixel of the box:
 //   the FP32 rounding of the coefficients and of the two fused multiply-adds (3 * 2^-24 of the magnitude
 //   M = |a0| rx + |a1| ry + |a2|), the FP64 rounding of the coefficients (2^-50 of the global magnitudes),
-//   the quotient of those errors ((e_X + |u'| e_W) / W), the rounded reciprocal, product and + 0.5
-//   (2^-23 |u'| + 2^-24 (|u'| + 1)), and the FP64 projection's own error against exact arithmetic
+//   the quotient of those errors ((e_X + |u'| e_W) / W), the rounded reciprocal and product (2^-23 |u'|; the
+//   remainder from the nearest integer is exact), and the FP64 projection's own error against exact arithmetic
 //   (3 * 2^-53 (A_X + |u| A_W) / W + 2 * 2^-53 (|u| + 1)),
-// doubled. Where u' computed in FP32 lies farther than delta from every half-integer, the integer nearest to
+// and a sixteenth more. The bounds are formed in FP32: the few roundings of one (at most 2^-18 of it) lie within that
+// sixteenth, or are added where a comparison stands without it (up). A_X is taken from the local coefficients
+// (|H0| <= |a0| + |U0 c0|, |H2| <= |X0| + |H0 x0| + |H1 y0|), W0 from its FP32 rounding; magnitudes that FP32
+// cannot hold end in kSlow. FP64 does at most 2 multiply-adds a cycle and SM here, and the bounds were most of its
+// work: 975x545, 7 views, 100 labels 2.14 -> 1.98 ms, and 1.90 with the margin above in place of a doubling (near
+// evaluations 0.0225 -> 0.011 % of all). Where u' computed in FP32 lies farther than delta from every half-integer, the integer nearest to
 // it, plus U0, is the FP64 projection's column floor(u + 0.5) (both see the same side of the same
-// half-integer); otherwise the evaluation is redone in FP64. Returns kGeneral (that test applies), kRect (the same, rectified: below),
-// kOut (the FP64 projection puts no
-// pixel of the box in view: behind the camera, or wholly beyond one image edge by more than the bound) or
-// kSlow (no bound: W may come near zero in the box, or delta is large; every evaluation in FP64).
+// half-integer); otherwise the evaluation is redone in FP64. Returns kGeneral (that test applies), kRect (the
+// same, rectified: below), kOut (the FP64 projection puts no pixel of the box in view: behind the camera, or wholly
+// beyond one image edge by more than the bound) or kSlow (no bound: W may come near zero in the box, or delta is large; every evaluation in FP64).
 __device__ uint32_t stage_precise(const double* __restrict__ hg, int x0, int y0, int rx, int ry, int wv, int hv,
                                   float* h, PEntry& P) {
     double H[9];
 #pragma unroll
     for (int f = 0; f < 9; ++f) H[f] = __ldg(&hg[f]);
-    const double u = 0x1p-53;
-    const double dx0 = (double)x0, dy0 = (double)y0, drx = (double)rx, dry = (double)ry;
-    const double ax = fabs(dx0) + drx, ay = fabs(dy0) + dry;
-    const double AX = fabs(H[0]) * ax + fabs(H[1]) * ay + fabs(H[2]);
-    const double AY = fabs(H[3]) * ax + fabs(H[4]) * ay + fabs(H[5]);
-    const double AW = fabs(H[6]) * ax + fabs(H[7]) * ay + fabs(H[8]);
+    const double dx0 = (double)x0, dy0 = (double)y0;
     const double X0 = fma(H[0], dx0, fma(H[1], dy0, H[2]));
     const double Y0 = fma(H[3], dx0, fma(H[4], dy0, H[5]));
     const double W0 = fma(H[6], dx0, fma(H[7], dy0, H[8]));
-    const double gW = fabs(H[6]) * drx + fabs(H[7]) * dry + 0x1p-48 * AW;
-    if (W0 + gW < 0.0) return kOut;  // W < 0 at every pixel of the box
-    const double Wlo = W0 - gW;      // the exact W is at least this at every pixel of the box
-    if (!(Wlo > 0x1p-60)) return kSlow;
-    const double U0 = rint(fmin(fmax((double)__fdiv_rn((float)X0, (float)W0), -0x1p24), 0x1p24));
-    const double V0 = rint(fmin(fmax((double)__fdiv_rn((float)Y0, (float)W0), -0x1p24), 0x1p24));
-    h[0] = __double2float_rn(fma(-U0, H[6], H[0]));
-    h[1] = __double2float_rn(fma(-U0, H[7], H[1]));
-    h[2] = __double2float_rn(fma(-U0, W0, X0));
-    h[3] = __double2float_rn(fma(-V0, H[6], H[3]));
-    h[4] = __double2float_rn(fma(-V0, H[7], H[4]));
-    h[5] = __double2float_rn(fma(-V0, W0, Y0));
+    const float X0f = __double2float_rn(X0), Y0f = __double2float_rn(Y0);
     h[6] = __double2float_rn(H[6]);
     h[7] = __double2float_rn(H[7]);
     h[8] = __double2float_rn(W0);
-    const double Ma = fabs((double)h[0]) * drx + fabs((double)h[1]) * dry + fabs((double)h[2]);
-    const double Mb = fabs((double)h[3]) * drx + fabs((double)h[4]) * dry + fabs((double)h[5]);
-    const double Mc = fabs((double)h[6]) * drx + fabs((double)h[7]) * dry + fabs((double)h[8]);
-    const double eX = 0x1.82p-23 * Ma + 0x1p-50 * (Ma + AX + fabs(U0) * AW) + 0x1p-130;
-    const double eY = 0x1.82p-23 * Mb + 0x1p-50 * (Mb + AY + fabs(V0) * AW) + 0x1p-130;
-    const double eW = 0x1.82p-23 * Mc + 0x1p-50 * (Mc + AW) + 0x1p-130;
-    if (!(Wlo > 2.0 * eW)) return kSlow;
-    const double Wl = Wlo - eW;  // lower bound of the FP32 W and of the FP64 projection's W
-    const double Ub = (Ma * (1.0 + 0x1p-20) + 2.0 * eX) / Wl;
-    const double Vb = (Mb * (1.0 + 0x1p-20) + 2.0 * eY) / Wl;
-    const double qu = (eX + Ub * eW) / Wl, qv = (eY + Vb * eW) / Wl;
-    const double du = 2.0 * (qu + 0x1.01p-23 * Ub + 0x1.01p-24 * (Ub + 1.0) +
-                             3.0 * u * (AX + (fabs(U0) + Ub) * AW) / Wl + 2.01 * u * (fabs(U0) + Ub + 1.0)) + 0x1p-30;
-    const double dv = 2.0 * (qv + 0x1.01p-23 * Vb + 0x1.01p-24 * (Vb + 1.0) +
-                             3.0 * u * (AY + (fabs(V0) + Vb) * AW) / Wl + 2.01 * u * (fabs(V0) + Vb + 1.0)) + 0x1p-30;
+    const float up = 1.0f + 0x1p-18f;  // above the roundings of any one bound below
+    const float frx = (float)rx, fry = (float)ry, ax = fabsf((float)x0) + frx, ay = fabsf((float)y0) + fry;
+    const float c0 = fabsf(h[6]), c1 = fabsf(h[7]), c2 = fabsf(h[8]);
+    const float AW = up * (2.0f * (c0 * ax + c1 * ay) + c2) + 0x1p-120f;
+    const float Rc = c0 * frx + c1 * fry;
+    const float gW = up * Rc + 0x1p-48f * AW + 0x1.1p-24f * c2 + 0x1p-120f;
+    if (h[8] + gW < 0.0f) return kOut;             // W < 0 at every pixel of the box
+    const float Wlo = (h[8] - gW) * (2.0f - up);   // the exact W is at least this at every pixel of the box
+    if (!(Wlo > 0x1p-60f && Wlo < 0x1p100f)) return kSlow;
+    const float U0 = rintf(fminf(fmaxf(__fdiv_rn(X0f, h[8]), -0x1p24f), 0x1p24f));
+    const float V0 = rintf(fminf(fmaxf(__fdiv_rn(Y0f, h[8]), -0x1p24f), 0x1p24f));
+    const double dU = (double)U0, dV = (double)V0;
+    h[0] = __double2float_rn(fma(-dU, H[6], H[0]));
+    h[1] = __double2float_rn(fma(-dU, H[7], H[1]));
+    h[2] = __double2float_rn(fma(-dU, W0, X0));
+    h[3] = __double2float_rn(fma(-dV, H[6], H[3]));
+    h[4] = __double2float_rn(fma(-dV, H[7], H[4]));
+    h[5] = __double2float_rn(fma(-dV, W0, Y0));
+    const float Ma = up * (fabsf(h[0]) * frx + fabsf(h[1]) * fry + fabsf(h[2])) + 0x1p-120f;
+    const float Mb = up * (fabsf(h[3]) * frx + fabsf(h[4]) * fry + fabsf(h[5])) + 0x1p-120f;
+    const float Mc = up * (Rc + c2) + 0x1p-120f;
+    const float aU = fabsf(U0), aV = fabsf(V0);
+    const float AX = up * (2.0f * ((fabsf(h[0]) + aU * c0) * ax + (fabsf(h[1]) + aU * c1) * ay) + fabsf(X0f)) + 0x1p-100f;
+    const float AY = up * (2.0f * ((fabsf(h[3]) + aV * c0) * ax + (fabsf(h[4]) + aV * c1) * ay) + fabsf(Y0f)) + 0x1p-100f;
+    const float eX = 0x1.82p-23f * Ma + 0x1p-50f * (Ma + AX + aU * AW);
+    const float eY = 0x1.82p-23f * Mb + 0x1p-50f * (Mb + AY + aV * AW);
+    const float eW = 0x1.82p-23f * Mc + 0x1p-50f * (Mc + AW);
+    if (!(Wlo > 2.0f * eW)) return kSlow;
+    const float rW = up * __frcp_rn(Wlo - eW);  // 1 / a lower bound of the FP32 W and of the FP64 projection's W
+    const float Ub = up * (Ma + 2.0f * eX) * rW, Vb = up * (Mb + 2.0f * eY) * rW;
+    const float du = 1.0625f * ((eX + Ub * eW + 0x1.8p-52f * (AX + (aU + Ub) * AW)) * rW + 0x1.01p-23f * Ub +
+                             0x1.02p-52f * (aU + Ub + 1.0f)) + 0x1p-30f;
+    const float dv = 1.0625f * ((eY + Vb * eW + 0x1.8p-52f * (AY + (aV + Vb) * AW)) * rW + 0x1.01p-23f * Vb +
+                             0x1.02p-52f * (aV + Vb + 1.0f)) + 0x1p-30f;
     // every pixel of the box has its column (row) beyond one edge by more than the bound
-    if (U0 + Ub + 0.5 + du < 0.0 || U0 - Ub + 0.5 - du >= (double)wv || V0 + Vb + 0.5 + dv < 0.0 ||
-        V0 - Vb + 0.5 - dv >= (double)hv)
+    const float lu = up * (Ub + du), lv = up * (Vb + dv);
+    if (U0 < -0.501f - lu || (float)((int)U0 - wv) > lu - 0.499f || V0 < -0.501f - lv ||
+        (float)((int)V0 - hv) > lv - 0.499f)
         return kOut;
-    if (!(du < 0.25 && dv < 0.25 && Ub < 0x1p21 && Vb < 0x1p21)) return kSlow;
+    if (!(du < 0.25f && dv < 0.25f && Ub < 0x1p21f && Vb < 0x1p21f)) return kSlow;
     P.u0 = (int)U0 - kRoundBits;  // the kernel adds it to the bits of t + kRound
     P.v0 = (int)V0 - kRoundBits;
     // near a tie when |t - nearest integer| >= thr
-    P.thr_u = __double2float_rd(0.5 - du - 0x1p-22);
-    P.thr_v = __double2float_rd(0.5 - dv - 0x1p-22);
+    P.thr_u = __fsub_rd(0.5f, __fadd_ru(du, 0x1p-22f));
+    P.thr_v = __fsub_rd(0.5f, __fadd_ru(dv, 0x1p-22f));
     // Rectified local frame (linear rigs with parallel axes): with a0 = b1 = c2 = 1 and a1 = b0 = c0 = c1 = 0
     // the general evaluation computes exactly t_u = x' + a2 (rounded) and W = r = 1, so the
     // bound above holds for that shorter sequence; and when |b2| + delta_v < 0.5 every pixel's row decision
     // is floor(y' + b2 + 0.5 +- delta_v) = y', i.e. the row is y' + V0 = y + (V0 - y0) with no test.
     if (h[0] == 1.0f && h[1] == 0.0f && h[3] == 0.0f && h[4] == 1.0f && h[6] == 0.0f && h[7] == 0.0f &&
-        h[8] == 1.0f && fabs((double)h[5]) + dv < 0.49) {
+        h[8] == 1.0f && fabsf(h[5]) + dv < 0.49f) {
         P.v0 = (int)V0 - y0;
         return kRect;
     }
@@ -513,9 +521,6 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cost_kernel(const RefJob
         Ref ref[kPPT];
         int run[kPPT], iy[kPPT];  // run[j]: first the pixel's segment, then its index among the warp's runs
         int rowx[kPPT];  // y * W + x (integer-shift entries)
-        // The float row: kept in registers except in the mixed kernel, which needs registers for rowx and,
-        // on the rigs it serves, rarely takes the general or affine paths that read it (exact conversion).
-        auto row_f = [&](int j) { return KIND == kKindMixed ? (float)iy[j] : py[j]; };
 #pragma unroll
         for (int j = 0; j < kPPT; ++j) {
             const int w = w0 + warp * kWarpPix + j * 32 + lane;
@@ -617,6 +622,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cost_kernel(const RefJob
         }
         for (int i = tid; i < N; i += kThreads) sBase[i] = nbrs[i].texels;
         if (tid <= min(nk, kSegAcc)) sWoffs[tid] = Jp->woffs[k0 + tid];
+        // The float row: kept in registers except in the mixed kernel, which needs registers for rowx and,
+        // on the rigs it serves, rarely takes the general or affine paths that read it (exact conversion).
+        auto row_f = [&](int j) { return KIND == kKindMixed ? (float)iy[j] : py[j]; };
         // The runs of equal segments among the warp's pixels (records are in list order). Ballots, not a loop until
         // every pixel is numbered: after a loop whose length depends on the data the compiler keeps the label loop's
         // counters and addresses in vector instead of uniform registers (3840x2160 15-view rig: 473 against 437 ms).
