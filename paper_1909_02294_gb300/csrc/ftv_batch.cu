@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "ftv_internal.h"
+#include "ftv_strip.cuh"
 
 using namespace ftv;
 
@@ -98,6 +99,8 @@ BatchLayout layout(int max_views, int max_units) {
     return L;
 }
 
+constexpr int kRowThreads = 128;  // CTAs of the row kernels
+
 __device__ __forceinline__ int find_base(const int32_t* base_field_of, int stride_bytes, int n, int v) {
     // largest i in [0, n) with base(i) <= v, where base(i) is an int at byte offset i * stride
     int lo = 0, hi = n - 1;
@@ -113,33 +116,39 @@ __device__ __forceinline__ int find_base(const int32_t* base_field_of, int strid
 
 // --------------------------------------------------------------------------------------------- pack
 
-__device__ __forceinline__ uint32_t load_plane(const void* plane, int64_t pitch, int sb, int x, int y) {
-    const char* row = static_cast<const char*>(plane) + (int64_t)y * pitch;
-    return sb == 1 ? (uint32_t)reinterpret_cast<const uint8_t*>(row)[x] : (uint32_t)reinterpret_cast<const uint16_t*>(row)[x];
+// Four adjacent pixels per thread, rows flattened over the tasks. Memory-bound: the row's loads of a thread and the
+// rows of the CTAs resident on an SM are what is in flight. Single pixels took 36 us for twelve 960x540 views, strips
+// 26.
+template <int SB, int FMT>
+__device__ __forceinline__ void pack_row(const PackTask& T, int y, bool vec) {
+    for (int x = threadIdx.x * 4; x < T.W; x += blockDim.x * 4) {
+        const int n = min(4, T.W - x);
+        uint32_t s[3][4];
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            load4<SB>(static_cast<const char*>(T.planes[c]) + (int64_t)y * T.pitch[c] + (int64_t)x * SB, n, vec, s[c]);
+        if (clamp4(s, T.maxv)) atomicOr(T.status, ST_BAD_SAMPLE);
+        const int64_t i = (int64_t)y * T.W + x;
+        store4<FMT>(T.out, i, n, vec, s);
+        if (T.cost_out) store4<FMT_U16S>(T.cost_out, i, n, vec, s);
+    }
 }
 
-__global__ void pack_multi_kernel(const Header* __restrict__ hdr, const PackTask* __restrict__ tasks) {
+__global__ void __launch_bounds__(kRowThreads) pack_multi_kernel(const Header* __restrict__ hdr,
+                                                                 const PackTask* __restrict__ tasks) {
     const int rows = hdr->pack_rows, n = hdr->n_pack;
     for (int g = blockIdx.x; g < rows; g += gridDim.x) {
-        const int t = find_base(&tasks[0].row_base, sizeof(PackTask), n, g);
-        const PackTask& T = tasks[t];
+        const PackTask& T = tasks[find_base(&tasks[0].row_base, sizeof(PackTask), n, g)];
         const int y = g - T.row_base;
-        for (int x = threadIdx.x; x < T.W; x += blockDim.x) {
-            uint32_t a = load_plane(T.planes[0], T.pitch[0], T.sb, x, y);
-            uint32_t b = load_plane(T.planes[1], T.pitch[1], T.sb, x, y);
-            uint32_t c = load_plane(T.planes[2], T.pitch[2], T.sb, x, y);
-            if (a > T.maxv || b > T.maxv || c > T.maxv) {
-                atomicOr(T.status, ST_BAD_SAMPLE);
-                a = min(a, T.maxv);
-                b = min(b, T.maxv);
-                c = min(c, T.maxv);
-            }
-            const int64_t i = (int64_t)y * T.W + x;
-            if (T.fmt == FMT_U8X4) static_cast<uint32_t*>(T.out)[i] = a | (b << 8) | (c << 16);
-            else if (T.fmt == FMT_P10) static_cast<uint32_t*>(T.out)[i] = a | (b << 10) | (c << 20);
-            else static_cast<uint2*>(T.out)[i] = make_uint2(a | (b << 16), c);
-            if (T.cost_out) static_cast<uint2*>(T.cost_out)[i] = make_uint2(a | (b << 16), c | ((a + b + c) << 16));
-        }
+        // whole strips only, every load and store aligned to its size
+        uintptr_t a = (reinterpret_cast<uintptr_t>(T.out) | reinterpret_cast<uintptr_t>(T.cost_out)) & 15;
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            a |= (reinterpret_cast<uintptr_t>(T.planes[c]) | (uintptr_t)T.pitch[c]) & (uintptr_t)(4 * T.sb - 1);
+        const bool vec = a == 0 && T.W % 4 == 0;
+        if (T.sb == 1) pack_row<1, FMT_U8X4>(T, y, vec);
+        else if (T.fmt == FMT_P10) pack_row<2, FMT_P10>(T, y, vec);
+        else pack_row<2, FMT_U16X4>(T, y, vec);
     }
 }
 
@@ -388,17 +397,7 @@ __global__ void wta_multi_kernel(const Header* __restrict__ hdr, const WtaUnit* 
         } else if (m == FTV_MASK_REUSE_I) {
             label = T.i_label[s];
         } else {
-            unsigned long long best = ~0ull;
-            const int32_t* row = T.cost + (int64_t)s * T.L;
-            for (int d = lane; d < T.L; d += 32) {
-                const unsigned long long k = ((unsigned long long)((uint32_t)row[d] ^ 0x80000000u) << 32) | (unsigned)d;
-                best = k < best ? k : best;
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                const unsigned long long t = __shfl_xor_sync(kFull, best, o);
-                best = t < best ? t : best;
-            }
-            label = (uint16_t)(best & 0xffffu);
+            label = (uint16_t)least_label(T.cost + (int64_t)s * T.L, T.L, lane);
         }
         if (lane == 0) {
             T.prev_label[s] = label;
@@ -408,20 +407,17 @@ __global__ void wta_multi_kernel(const Header* __restrict__ hdr, const WtaUnit* 
     }
 }
 
-__global__ void depth_multi_kernel(const Header* __restrict__ hdr, const WtaUnit* __restrict__ units) {
+// Four adjacent pixels per thread, rows flattened over the units (single pixels: 36 us for twelve 960x540 maps; strips
+// 13).
+__global__ void __launch_bounds__(kRowThreads) depth_multi_kernel(const Header* __restrict__ hdr,
+                                                                  const WtaUnit* __restrict__ units) {
     const int rows = hdr->depth_rows, n = hdr->n_units;
     for (int g = blockIdx.x; g < rows; g += gridDim.x) {
-        const int u = find_base(&units[0].depth_base, sizeof(WtaUnit), n, g);
-        const WtaUnit& T = units[u];
-        const int y = g - T.depth_base;
-        for (int x = threadIdx.x; x < T.W; x += blockDim.x) {
-            const int64_t p = (int64_t)y * T.W + x;
-            const int s = T.labels[p];
-            float z = 0.0f;
-            if ((unsigned)s < (unsigned)T.S && T.prev_label[s] < T.L) z = T.label_z[T.prev_label[s]];
-            else atomicOr(T.status, ST_BAD_LABEL);
-            T.depth[p] = z;
-        }
+        const WtaUnit& T = units[find_base(&units[0].depth_base, sizeof(WtaUnit), n, g)];
+        const int64_t row = (int64_t)(g - T.depth_base) * T.W;
+        const bool vec = ((reinterpret_cast<uintptr_t>(T.labels) | reinterpret_cast<uintptr_t>(T.depth)) & 15) == 0 && T.W % 4 == 0;
+        for (int x = threadIdx.x * 4; x < T.W; x += blockDim.x * 4)
+            depth4(T.labels, row + x, min(4, T.W - x), vec, T.S, T.prev_label, T.label_z, T.L, T.depth, T.status);
     }
 }
 
@@ -1134,7 +1130,7 @@ static cudaError_t enqueue(ftv_batch* b, cudaStream_t s) {
     cudaError_t e = cudaMemcpyAsync(b->d_desc, b->h_stage, b->lay.total, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_job_status, 0, sizeof(uint32_t) * b->max_jobs, s);
     if (e != cudaSuccess) return e;
-    pack_multi_kernel<<<g, 256, 0, s>>>(hdr, pack);
+    pack_multi_kernel<<<b->n_sm * 16, kRowThreads, 0, s>>>(hdr, pack);
     temporal_zero_multi_kernel<<<g, 256, 0, s>>>(hdr, temp);
     temporal_accumulate_multi_kernel<<<b->n_sm * b->temp_per_sm, 256, 0, s>>>(hdr, temp);
     temporal_decide_multi_kernel<<<g, kTChunk, 0, s>>>(hdr, temp);
@@ -1149,8 +1145,8 @@ static cudaError_t enqueue(ftv_batch* b, cudaStream_t s) {
         e = launch_cost(jobs, b->d_plan, b->cost_fmt, b->combine, b->fast_rcp, b->penalty_floor, b->kind, k, b->chunks,
                         b->cost_grid, s);
     if (e != cudaSuccess) return e;
-    wta_multi_kernel<<<g, 256, 0, s>>>(hdr, wta);
-    depth_multi_kernel<<<g, 256, 0, s>>>(hdr, wta);
+    wta_multi_kernel<<<b->n_sm * 8, 256, 0, s>>>(hdr, wta);
+    depth_multi_kernel<<<b->n_sm * 16, kRowThreads, 0, s>>>(hdr, wta);
     b->launches += 9 + b->chunks;
     e = cudaGetLastError();
     // every job's status word back to pinned host memory, read by ftv_batch_wait / ftv_batch_poll once the

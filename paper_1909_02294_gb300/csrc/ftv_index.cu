@@ -13,6 +13,7 @@
 #include <algorithm>
 
 #include "ftv_internal.h"
+#include "ftv_strip.cuh"
 
 namespace ftv {
 namespace {
@@ -25,27 +26,6 @@ template <int CAP>
 struct PackArgs {
     PackView v[CAP];
 };
-
-template <int SB>
-__device__ __forceinline__ void load4(const char* p, int n, bool vec, uint32_t* out) {
-    if (vec) {  // four samples in one load
-        if (SB == 1) {
-            const uint32_t t = __ldg(reinterpret_cast<const uint32_t*>(p));
-#pragma unroll
-            for (int k = 0; k < 4; ++k) out[k] = (t >> (8 * k)) & 0xff;
-        } else {
-            const uint2 t = __ldg(reinterpret_cast<const uint2*>(p));
-            out[0] = t.x & 0xffff;
-            out[1] = t.x >> 16;
-            out[2] = t.y & 0xffff;
-            out[3] = t.y >> 16;
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            out[k] = k >= n ? 0u : SB == 1 ? reinterpret_cast<const uint8_t*>(p)[k] : reinterpret_cast<const uint16_t*>(p)[k];
-    }
-}
 
 // Four adjacent pixels of a row per thread; blockIdx.y is the row, blockIdx.z the view. Samples above max_value
 // are reported and clamped so that they cannot spill into a neighbouring packed field. Memory-bound; a thread's
@@ -63,42 +43,8 @@ __global__ void __launch_bounds__(128) pack_kernel(const __grid_constant__ PackA
 #pragma unroll
     for (int c = 0; c < 3; ++c)
         load4<SB>(static_cast<const char*>(V.planes[c]) + (int64_t)y * V.pitch[c] + (int64_t)x * SB, n, vec, s[c]);
-    bool bad = false;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        bad = bad || s[0][k] > max_value || s[1][k] > max_value || s[2][k] > max_value;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) s[c][k] = min(s[c][k], max_value);
-    }
-    if (bad) atomicOr(status, ST_BAD_SAMPLE);
-    const int64_t i = (int64_t)y * V.W + x;
-    if (FMT == FMT_U8X4 || FMT == FMT_P10) {
-        constexpr int sh = FMT == FMT_U8X4 ? 8 : 10;
-        uint32_t t[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) t[k] = s[0][k] | (s[1][k] << sh) | (s[2][k] << (2 * sh));
-        uint32_t* out = static_cast<uint32_t*>(V.out) + i;
-        if (vec) *reinterpret_cast<uint4*>(out) = make_uint4(t[0], t[1], t[2], t[3]);
-        else
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (k < n) out[k] = t[k];
-    } else {
-        uint2 t[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            t[k] = make_uint2(s[0][k] | (s[1][k] << 16),
-                              FMT == FMT_U16S ? s[2][k] | ((s[0][k] + s[1][k] + s[2][k]) << 16) : s[2][k]);
-        uint2* out = static_cast<uint2*>(V.out) + i;
-        if (vec) {
-            reinterpret_cast<uint4*>(out)[0] = make_uint4(t[0].x, t[0].y, t[1].x, t[1].y);
-            reinterpret_cast<uint4*>(out)[1] = make_uint4(t[2].x, t[2].y, t[3].x, t[3].y);
-        } else {
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (k < n) out[k] = t[k];
-        }
-    }
+    if (clamp4(s, max_value)) atomicOr(status, ST_BAD_SAMPLE);
+    store4<FMT>(V.out, (int64_t)y * V.W + x, n, vec, s);
 }
 
 // ------------------------------------------------------------------------------------ segment index
@@ -436,7 +382,7 @@ constexpr int kLocCache = 1025;  // segments of a tile whose offsets are cached 
 // The records stay in list order. Ordering a tile's pixels by 16- or 32-pixel wide blocks, so that a gather meets
 // fewer rows, measured slower (1920x1080 rig 21.8 and 24.0 against 20.6 ms): a warp then meets more segments.
 __global__ void __launch_bounds__(kTileThreads) tile_kernel(const RefJob* __restrict__ jobs, const Plan* __restrict__ plan) {
-    __shared__ int sWoffs[kLocCache + 1];
+    __shared__ int sWoffs[kLocCache + 1], sFrom[kLocCache + 1];  // sFrom: list position - record position
     __shared__ int s_k0, s_k1, s_box[4];
     const int tid = threadIdx.x, lane = tid & 31;
     const int total = plan->total_tiles, n_jobs = plan->n_jobs;
@@ -453,8 +399,8 @@ __global__ void __launch_bounds__(kTileThreads) tile_kernel(const RefJob* __rest
         const int32_t* __restrict__ list = J.list;
         const int32_t* __restrict__ woffs = J.woffs;
         {  // this tile's share of the cost rows to clear
-            const int64_t words = (int64_t)n_work * L, b = words * tile / tiles, e = words * (tile + 1) / tiles;
             if (list == nullptr) {
+                const int64_t words = (int64_t)n_work * L, b = words * tile / tiles, e = words * (tile + 1) / tiles;
                 const bool vec = (reinterpret_cast<uintptr_t>(J.cost) & 15) == 0;
                 const int64_t vb = vec ? (b + 3) / 4 : 0, ve = vec ? e / 4 : 0;
                 if (vec && vb < ve) {
@@ -466,9 +412,12 @@ __global__ void __launch_bounds__(kTileThreads) tile_kernel(const RefJob* __rest
                     for (int64_t i = b + tid; i < e; i += kTileThreads) J.cost[i] = 0;
                 }
             } else {
-                for (int64_t i = b + tid; i < e; i += kTileThreads) {
-                    const int k = (int)(i / L), d = (int)(i - (int64_t)k * L), s = list[k];
-                    if ((unsigned)s < (unsigned)J.S) J.cost[(int64_t)s * L + d] = 0;
+                // whole rows, one per warp
+                const int kb = (int)((int64_t)n_work * tile / tiles), ke = (int)((int64_t)n_work * (tile + 1) / tiles);
+                for (int k = kb + (tid >> 5); k < ke; k += kTileThreads / 32) {
+                    const int s = list[k];
+                    if ((unsigned)s < (unsigned)J.S)
+                        for (int d = lane; d < L; d += 32) J.cost[(int64_t)s * L + d] = 0;
                 }
             }
         }
@@ -489,7 +438,14 @@ __global__ void __launch_bounds__(kTileThreads) tile_kernel(const RefJob* __rest
         const int k0 = s_k0, k1 = s_k1, nk = k1 - k0 + 1;
         const bool cached = nk + 1 <= kLocCache;
         if (cached)
-            for (int i = tid; i <= nk; i += kTileThreads) sWoffs[i] = woffs[k0 + i];
+            for (int i = tid; i <= nk; i += kTileThreads) {
+                const int at = woffs[k0 + i];
+                sWoffs[i] = at;
+                if (list != nullptr && i < nk) {
+                    const int l = list[k0 + i];  // an entry outside the segments owns no pixels: its offset is not read
+                    sFrom[i] = (unsigned)l < (unsigned)J.S ? J.offs[l] - at : 0;
+                }
+            }
         __syncthreads();
         int x0 = INT32_MAX, x1 = -1, y0 = INT32_MAX, y1 = -1;
 #pragma unroll
@@ -498,7 +454,7 @@ __global__ void __launch_bounds__(kTileThreads) tile_kernel(const RefJob* __rest
             if (w < w1) {
                 const int k = cached ? k0 + upper_index(sWoffs, 0, nk + 1, w) : upper_index(woffs, k0, k1 + 1, w);
                 int i = w;
-                if (list != nullptr) i = J.offs[list[k]] + (w - (cached ? sWoffs[k - k0] : woffs[k]));
+                if (list != nullptr) i = cached ? w + sFrom[k - k0] : J.offs[list[k]] + (w - woffs[k]);
                 const uint32_t xy = J.pix[i];
                 J.recs[w] = make_int2((int)xy, k);
                 const int x = xy & 0xffff, y = xy >> 16;

@@ -14,6 +14,7 @@
 #include <climits>
 
 #include "ftv_internal.h"
+#include "ftv_strip.cuh"
 
 namespace ftv {
 namespace {
@@ -365,39 +366,19 @@ __global__ void wta_kernel(const int32_t* __restrict__ cost, int S, int L, const
             if (lane == 0) out[s] = ifr_label[s];
             continue;
         }
-        // order key: signed cost mapped to unsigned in the high word, label in the low word
-        unsigned long long best = ~0ull;
-        const int32_t* row = cost + (int64_t)s * L;
-        for (int d = lane; d < L; d += 32) {
-            const unsigned long long k =
-                ((unsigned long long)((uint32_t)row[d] ^ 0x80000000u) << 32) | (unsigned long long)d;
-            best = k < best ? k : best;
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long t = __shfl_xor_sync(kFull, best, o);
-            best = t < best ? t : best;
-        }
-        if (lane == 0) out[s] = (uint16_t)(best & 0xffffu);
+        const int d = least_label(cost + (int64_t)s * L, L, lane);
+        if (lane == 0) out[s] = (uint16_t)d;
     }
 }
 
-__global__ void depth_map_kernel(const int32_t* __restrict__ labels, int W, int S,
-                                 const uint16_t* __restrict__ seg_label, const float* __restrict__ label_z, int L,
-                                 float* __restrict__ depth, uint32_t* status) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y;
+// Four adjacent pixels of a row per thread.
+__global__ void __launch_bounds__(128) depth_map_kernel(const int32_t* __restrict__ labels, int W, int S,
+                                                        const uint16_t* __restrict__ seg_label,
+                                                        const float* __restrict__ label_z, int L,
+                                                        float* __restrict__ depth, bool vec, uint32_t* status) {
+    const int x = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (x >= W) return;
-    const int64_t p = (int64_t)y * W + x;
-    const int s = labels[p];
-    float z = 0.0f;
-    if ((unsigned)s < (unsigned)S) {
-        const int d = seg_label[s];
-        if (d < L) z = label_z[d];
-        else atomicOr(status, ST_BAD_LABEL);
-    } else {
-        atomicOr(status, ST_BAD_LABEL);
-    }
-    depth[p] = z;
+    depth4(labels, (int64_t)blockIdx.y * W + x, min(4, W - x), vec, S, seg_label, label_z, L, depth, status);
 }
 
 }  // namespace
@@ -499,8 +480,9 @@ cudaError_t launch_wta(const int32_t* cost, int S, int L, const uint8_t* mask, c
 cudaError_t launch_depth_map(const int32_t* labels, int W, int H, int S, const uint16_t* seg_label,
                              const float* label_z, int L, float* depth, uint32_t* status, cudaStream_t s) {
     if (W <= 0 || H <= 0) return cudaSuccess;
-    const dim3 block(256), grid((W + 255) / 256, H);
-    depth_map_kernel<<<grid, block, 0, s>>>(labels, W, S, seg_label, label_z, L, depth, status);
+    const dim3 block(128), grid((W + 511) / 512, H);
+    const bool vec = ((reinterpret_cast<uintptr_t>(labels) | reinterpret_cast<uintptr_t>(depth)) & 15) == 0 && W % 4 == 0;
+    depth_map_kernel<<<grid, block, 0, s>>>(labels, W, S, seg_label, label_z, L, depth, vec, status);
     return cudaGetLastError();
 }
 
