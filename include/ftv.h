@@ -529,7 +529,7 @@ typedef struct ftv_segmenter_config {
 } ftv_segmenter_config;
 
 /* Create a segmenter for a fixed set of image sizes on the current device; allocates its device scratch
- * (about 100 bytes per pixel) and a pinned staging block. Synchronous. FTV_ERR_INVALID_ARG,
+ * (128 bytes per pixel) and a pinned staging block. Synchronous. FTV_ERR_INVALID_ARG,
  * FTV_ERR_OUT_OF_MEMORY. */
 FTV_API ftv_status ftv_segmenter_init(const ftv_segmenter_config* cfg, ftv_segmenter** out);
 
@@ -596,7 +596,8 @@ FTV_API ftv_status ftv_last_kernel_ms(ftv_ctx* ctx, float* ms);
  * Launch shape of the context's cost kernel (no paper counterpart: the GPU's work decomposition). A work
  * item is one tile of the kernel's compile-time pixel count times one block of consecutive labels;
  * label_block caps the labels per block (the labels are split into equal blocks of at most that many,
- * 1 <= label_block <= the stage's limit for the context's neighbour count), and ctas_per_sm sets the
+ * 1 <= label_block <= the stage's limit for the context's neighbour count; a launch whose tiles are too few
+ * to fill the device takes smaller blocks by itself), and ctas_per_sm sets the
  * persistent grid (1 up to the occupancy limit; 0 = the occupancy limit). Every shape gives the same
  * volume. Set between calls, not while a call of the context is being issued. The batch path
  * (ftv_batch_*) uses a context's label block and its own occupancy-sized grid.

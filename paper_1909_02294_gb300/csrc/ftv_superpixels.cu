@@ -51,6 +51,7 @@ constexpr int kCTile = 32;                       // component tiles
 constexpr int kLoopCap = 1 << 26;                // bound of every union-find walk (parents strictly decrease)
 // One CTA of 1024 threads per SM: a barrier costs by the CTAs that meet at it (about 10 us with 912 CTAs of 256).
 constexpr int kRegionThreads = 1024;  // 152 of 1024: about 1 us
+constexpr int kRun = 128;             // entries that a warp of regions_kernel appends to a list at a time
 constexpr unsigned long long kNone = ~0ull;
 
 enum : uint32_t { SP_LOOP_CAP = 1u, SP_ROUND_CAP = 2u, SP_BARRIER = 4u };
@@ -106,6 +107,7 @@ struct Scratch {
     int2* orph[2];                // [P] pick lists of (pixel, image), alternating between rounds
     int32_t* cnt;
     uint32_t* barrier;            // arrivals at the grid barriers of regions_kernel (cleared with cnt)
+    int32_t* work;                // [2 phases] items drawn from for_items (cleared with cnt)
     uint32_t* status;
     int32_t n_images, tiles, ctiles;  // images, and pixel tiles and component tiles of all of them
     int64_t pixels;
@@ -165,22 +167,24 @@ __device__ void unite(int32_t* par, int32_t a, int32_t b, uint32_t* status) {
     atomicOr(status, SP_LOOP_CAP);
 }
 
-// A warp's share of a list that grows in global memory: entries gather in 64 words of shared memory and leave 32 at a
-// time, coalesced, with one atomic (an append of the whole CTA waited at three barriers per call).
-template <class T>
+// A warp's share of a list that grows in global memory: entries gather in shared memory (RUN + 32 words of it) and leave
+// RUN at a time, coalesced, with one atomic (an append of the whole CTA waited at three barriers per call). All warps of
+// the chip meet at that atomic, so a long list takes long runs (15 fragmented images of
+// 3840x2160: 54.5 ms with runs of 32, 44.2 of 128).
+template <class T, int RUN>
 struct WarpList {
-    T* buf;  // the warp's 64 entries
+    T* buf;
     T* list;
     int32_t* counter;
     int n;
 
     __device__ __forceinline__ void flush() {
-        const int lane = threadIdx.x & 31, k = min(n, 32);
+        const int lane = threadIdx.x & 31, k = min(n, RUN);
         __syncwarp();
         int base = 0;
         if (lane == 0) base = atomicAdd(counter, k);
         base = __shfl_sync(kFull, base, 0);
-        if (lane < k) list[base + lane] = buf[lane];
+        for (int i = lane; i < k; i += 32) list[base + i] = buf[i];
         T rest{};
         if (lane < n - k) rest = buf[k + lane];
         __syncwarp();
@@ -194,7 +198,7 @@ struct WarpList {
         if (m == 0) return;
         if (keep) buf[n + __popc(m & ((1u << (threadIdx.x & 31)) - 1u))] = v;
         n += __popc(m);
-        if (n >= 32) flush();
+        if (n >= RUN) flush();
     }
     __device__ __forceinline__ void finish() {
         while (n > 0) flush();
@@ -554,7 +558,7 @@ __global__ void __launch_bounds__(kThreads) components_kernel(Scratch s) {
         if (l >= 0 && end) atomicAdd(&s_sum[0][r], (uint32_t)(lane - start + 1));
     }
     __syncthreads();
-    WarpList<int32_t> roots{s_buf[warp], s.uroots[1], &s.cnt[4 + 2 * s.rounds], 0};
+    WarpList<int32_t, 32> roots{s_buf[warp], s.uroots[1], &s.cnt[4 + 2 * s.rounds], 0};
 #pragma unroll
     for (int k = 0; k < kRows; ++k) {
         const int row = warp * kRows + k, y = y0 + row, i = row * kCTile + lane;
@@ -642,8 +646,8 @@ constexpr int kBarrierPolls = 1 << 23;
 __device__ bool grid_barrier(const Scratch& s, uint32_t& phase) {
     __shared__ int s_ok;
     __syncthreads();
+    ++phase;
     if (threadIdx.x == 0) {
-        ++phase;
         __threadfence();
         atomicAdd(s.barrier, 1u);
         const uint32_t target = phase * gridDim.x;
@@ -658,12 +662,45 @@ __device__ bool grid_barrier(const Scratch& s, uint32_t& phase) {
     return s_ok != 0;
 }
 
+// Calls f(t) for this warp's share of the turns 0 .. n - 1; all lanes make every call. The warps take turns. Where that
+// would be more than kTurns each, they draw runs of kTurns turns from a counter instead: with fixed turns the SMs drift
+// apart (a third of a phase on 15 images of 3840x2160 full of fragments), wait at the barrier, and the lists and groups
+// in use at a time no longer fit the L2 (that call 76 ms with fixed turns, 54 with runs of 4 or 8, 57 of 2,
+// 68 of 32).
+constexpr uint32_t kTurns = 8;
+
+template <class F>
+__device__ __forceinline__ void for_turns(uint32_t n, int32_t* counter, F f) {
+    const uint32_t warps = gridDim.x * (kRegionThreads / 32), w = blockIdx.x * (kRegionThreads / 32) + (threadIdx.x >> 5);
+    const bool draw = n > warps * kTurns;
+    uint32_t t = draw ? w * kTurns : w, left = kTurns;
+    while (t < n) {
+        f((int)t);
+        if (!draw) {
+            t += warps;
+        } else if (--left > 0) {
+            ++t;
+        } else {
+            uint32_t c = 0;
+            if ((threadIdx.x & 31) == 0) c = warps + (uint32_t)atomicAdd(counter, 1);
+            t = __shfl_sync(kFull, c, 0) * kTurns;
+            left = kTurns;
+        }
+    }
+}
+
+// The same for n items (n < 2^31), 32 to a turn: f(base), items base .. base + 31, base < n.
+template <class F>
+__device__ __forceinline__ void for_items(int64_t n, int32_t* counter, F f) {
+    for_turns((uint32_t)((n + 31) / 32), counter, [&](int t) { f(t * 32); });
+}
+
 // Calls f(image index, image, x, y0) for this warp's share of all images' 32 x 4 pixel tiles (column x of the lane, rows
 // y0 .. y0 + 3; positions past the image's edges included); all lanes make every call.
 template <class F>
-__device__ __forceinline__ void for_tiles(const Scratch& s, F f) {
-    const int warps = kRegionThreads / 32, lane = threadIdx.x & 31;
-    for (int t = blockIdx.x * warps + (threadIdx.x >> 5); t < s.tiles; t += gridDim.x * warps) {
+__device__ __forceinline__ void for_tiles(const Scratch& s, int32_t* counter, F f) {
+    const int lane = threadIdx.x & 31;
+    for_turns((uint32_t)s.tiles, counter, [&](int t) {
         int lo = 0, hi = s.n_images - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
@@ -673,7 +710,7 @@ __device__ __forceinline__ void for_tiles(const Scratch& s, F f) {
         const SegImage& im = s.img[lo];
         const int tw = (im.W + kTileW - 1) / kTileW, q = t - im.tile_base;
         f(lo, im, (q % tw) * kTileW + lane, (q / tw) * kTileH);
-    }
+    });
 }
 
 // From the tile components to the labels, in one cooperative launch whose phases are separated by grid barriers: links
@@ -692,11 +729,11 @@ __device__ __forceinline__ void for_tiles(const Scratch& s, F f) {
 // such an image (25 phases of 2 to 8 us, 1 us of them the barrier), 1.12 ms for eight of 1920x1080, a quarter of it the
 // first pick (a third of these scenes' pixels lie outside their label's main component).
 __global__ void __launch_bounds__(kRegionThreads, 1) regions_kernel(Scratch s) {
-    __shared__ int2 s_buf[kRegionThreads / 32][64];
-    __shared__ int32_t s_buf2[kRegionThreads / 32][64];
+    __shared__ int2 s_buf[kRegionThreads / 32][kRun + 32];  // one list at a time
     uint32_t phase = 0;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, stride = gridDim.x * kRegionThreads;
-    auto int_list = [&](int32_t* list, int32_t* counter) { return WarpList<int32_t>{s_buf2[warp], list, counter, 0}; };
+    auto work = [&](int k) { return s.work + 2 * phase + k; };  // the phase's counters for for_items
+    auto int_list = [&](int32_t* list, int32_t* counter) { return WarpList<int32_t, kRun>{reinterpret_cast<int32_t*>(s_buf[warp]), list, counter, 0}; };
 
     // links across the component tiles' borders: a tile's top row in three directions, its left column in two and its
     // right column in one, each a warp's task (a link waits on a chain of loads)
@@ -727,7 +764,7 @@ __global__ void __launch_bounds__(kRegionThreads, 1) regions_kernel(Scratch s) {
     {
         const int n = __ldcg(&s.cnt[4 + 2 * s.rounds]);
         auto comps = int_list(s.comps, &s.cnt[0]);
-        for (int base = blockIdx.x * kRegionThreads + warp * 32; base < n; base += stride) {
+        for_items(n, work(0), [&](int base) {
             const int i = base + lane;
             bool root = false;
             int32_t c = 0;
@@ -743,25 +780,27 @@ __global__ void __launch_bounds__(kRegionThreads, 1) regions_kernel(Scratch s) {
                 }
             }
             comps.append(root, c);
-        }
+        });
         comps.finish();
     }
     if (!grid_barrier(s, phase)) return;
     // every component takes its index in the list and offers itself as its label's main component (the largest, the
     // earliest named on ties)
     const int n_comps = __ldcg(&s.cnt[0]);
-    for (int i = blockIdx.x * kRegionThreads + tid; i < n_comps; i += stride) {
+    for_items(n_comps, work(0), [&](int base) {
+        const int i = base + lane;
+        if (i >= n_comps) return;
         const int32_t c = s.comps[i];
         const unsigned long long key = ((__ldcg(&s.csum[c].x) >> 40) << 32) | (unsigned long long)(~(uint32_t)c);
         atomicMax(&s.mainkey[s.lab[c]], key);
         s.par[c] = -1 - i;
-    }
+    });
     if (!grid_barrier(s, phase)) return;
     // the groups, and every pixel's component index (a pixel's parent is its tile component's root, whose parent is
     // the component's name; four pixels per thread in flight)
     {
         auto orphans = int_list(s.uroots[0], &s.cnt[1]);
-        for (int base = blockIdx.x * kRegionThreads + warp * 32; base < n_comps; base += stride) {
+        for_items(n_comps, work(0), [&](int base) {
             const int i = base + lane;
             bool is_main = false;
             if (i < n_comps) {
@@ -779,13 +818,14 @@ __global__ void __launch_bounds__(kRegionThreads, 1) regions_kernel(Scratch s) {
                 s.dirty[i] = 0;
             }
             orphans.append(i < n_comps && !is_main, i);
-        }
+        });
         orphans.finish();
     }
-    for (int64_t p0 = blockIdx.x * kRegionThreads + tid; p0 < s.pixels; p0 += 4 * (int64_t)stride) {
+    for_items((s.pixels + 3) / 4, work(1), [&](int base) {
+        const int64_t p0 = 4 * (int64_t)base + lane;
         int32_t r[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) r[k] = p0 + (int64_t)k * stride < s.pixels ? s.par[p0 + (int64_t)k * stride] : -1;
+        for (int k = 0; k < 4; ++k) r[k] = p0 + 32 * k < s.pixels ? s.par[p0 + 32 * k] : -1;
 #pragma unroll
         for (int step = 0; step < 2; ++step)
 #pragma unroll
@@ -793,18 +833,18 @@ __global__ void __launch_bounds__(kRegionThreads, 1) regions_kernel(Scratch s) {
                 if (r[k] >= 0) r[k] = s.par[r[k]];
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            if (p0 + (int64_t)k * stride < s.pixels) s.comp[p0 + (int64_t)k * stride] = -1 - r[k];
-    }
+            if (p0 + 32 * k < s.pixels) s.comp[p0 + 32 * k] = -1 - r[k];
+    });
     if (!grid_barrier(s, phase)) return;
     for (int r = 0; r < s.rounds; ++r) {
         const int n_roots = __ldcg(&s.cnt[1 + r]);
         if (n_roots == 0) break;
-        WarpList<int2> next{s_buf[warp], s.orph[(r + 1) & 1], &s.cnt[2 + s.rounds + r + 1], 0};
+        WarpList<int2, kRun> next{s_buf[warp], s.orph[(r + 1) & 1], &s.cnt[2 + s.rounds + r + 1], 0};
         if (r == 0) {
             // Every group is one component: no walks, and a pixel all of whose neighbours lie in its own component,
             // the common case, is done after loads that its warp shares: a lane holds four rows of a column and the
             // rows above and below, and takes its neighbours' columns by shuffles.
-            for_tiles(s, [&](int k, const SegImage& im, int x, int y0) {
+            for_tiles(s, work(0), [&](int k, const SegImage& im, int x, int y0) {
                 const int W = im.W, H = im.H;
                 const int32_t* comp = s.comp + im.pix_base;
                 int32_t c[6], edge[6];  // rows y0 - 1 .. y0 + 4; edge: the column beyond the warp's, lanes 0 and 31
@@ -850,7 +890,7 @@ __global__ void __launch_bounds__(kRegionThreads, 1) regions_kernel(Scratch s) {
         } else {
             const int n = __ldcg(&s.cnt[2 + s.rounds + r]);
             const int2* in = s.orph[r & 1];
-            for (int base = blockIdx.x * kRegionThreads + warp * 32; base < n; base += stride) {
+            for_items(n, work(0), [&](int base) {
                 const int i = base + lane;
                 bool keep = false;
                 int2 o = make_int2(0, 0);
@@ -861,19 +901,20 @@ __global__ void __launch_bounds__(kRegionThreads, 1) regions_kernel(Scratch s) {
                     keep = s.glab[a] < 0 && pick_pixel(s, s.img[o.y], o.x, pc, a);
                 }
                 next.append(keep, o);
-            }
+            });
         }
         next.finish();
         if (!grid_barrier(s, phase)) return;
         const int32_t* u = s.uroots[r & 1];
-        for (int i = blockIdx.x * kRegionThreads + tid; i < n_roots; i += stride) {
-            const int32_t c = u[i];
+        for_items(n_roots, work(0), [&](int base) {
+            if (base + lane >= n_roots) return;
+            const int32_t c = u[base + lane];
             const unsigned long long b = s.best[c];
             if (b != kNone) unite_groups(s, c, s.comp[(uint32_t)b]);
-        }
+        });
         if (!grid_barrier(s, phase)) return;
         auto dirty = int_list(s.dirty_list, &s.cnt[6 + 2 * s.rounds + r]);
-        for (int base = blockIdx.x * kRegionThreads + warp * 32; base < n_roots; base += stride) {
+        for_items(n_roots, work(0), [&](int base) {
             const int i = base + lane;
             bool first = false;
             int32_t t = 0;
@@ -892,11 +933,11 @@ __global__ void __launch_bounds__(kRegionThreads, 1) regions_kernel(Scratch s) {
                 }
             }
             dirty.append(first, t);
-        }
+        });
         dirty.finish();
         if (!grid_barrier(s, phase)) return;
         auto left = int_list(s.uroots[(r + 1) & 1], &s.cnt[2 + r]);
-        for (int base = blockIdx.x * kRegionThreads + warp * 32; base < n_roots; base += stride) {
+        for_items(n_roots, work(0), [&](int base) {
             const int i = base + lane;
             bool keep = false;
             int32_t c = 0;
@@ -911,7 +952,7 @@ __global__ void __launch_bounds__(kRegionThreads, 1) regions_kernel(Scratch s) {
                 }
             }
             left.append(keep, c);
-        }
+        });
         left.finish();
         const int n_dirty = __ldcg(&s.cnt[6 + 2 * s.rounds + r]);
         for (int i = blockIdx.x * kRegionThreads + tid; i < n_dirty; i += stride) {
@@ -923,12 +964,14 @@ __global__ void __launch_bounds__(kRegionThreads, 1) regions_kernel(Scratch s) {
     }
     if (blockIdx.x == 0 && tid == 0 && __ldcg(&s.cnt[1 + s.rounds]) != 0) atomicOr(s.status, SP_ROUND_CAP);
     // every component takes its group's label (an anchored root keeps its own; it is not written here)
-    for (int i = blockIdx.x * kRegionThreads + tid; i < n_comps; i += stride) {
+    for_items(n_comps, work(0), [&](int base) {
+        const int i = base + lane;
+        if (i >= n_comps) return;
         const int32_t t = find_root(s.gpar, i, s.status);
         if (t != i) s.glab[i] = s.glab[t];
-    }
+    });
     if (!grid_barrier(s, phase)) return;
-    for_tiles(s, [&](int, const SegImage& im, int x, int y0) {
+    for_tiles(s, work(0), [&](int, const SegImage& im, int x, int y0) {
         if (x >= im.W) return;
         const int W = im.W, H = im.H, base = im.pix_base + y0 * W + x;
         int32_t g[4];
@@ -968,6 +1011,10 @@ struct ftv_segmenter {
 };
 
 namespace {
+
+// Counter words of a segmenter: the lists' and the barrier's, then two for each phase of regions_kernel (four barriers
+// before the rounds, four in a round, one after).
+size_t counters(int rounds) { return (size_t)(3 * rounds + 8) + 2 * (size_t)(4 * rounds + 6); }
 
 template <class T>
 bool dalloc(ftv_segmenter* g, T** p, size_t n) {
@@ -1079,7 +1126,7 @@ extern "C" ftv_status ftv_segmenter_init(const ftv_segmenter_config* cfg, ftv_se
     ok = ok && dalloc(g, &s.best, P) && dalloc(g, &s.orph[0], P) && dalloc(g, &s.orph[1], P);
     ok = ok && dalloc(g, &s.uroots[0], P) && dalloc(g, &s.uroots[1], P) && dalloc(g, &s.dirty, P) &&
          dalloc(g, &s.dirty_list, P);
-    ok = ok && dalloc(g, &s.cnt, 3 * g->rounds + 8) && dalloc(g, &s.status, 1);
+    ok = ok && dalloc(g, &s.cnt, counters(g->rounds)) && dalloc(g, &s.status, 1);
     ok = ok && cudaMemset(s.status, 0, sizeof(uint32_t)) == cudaSuccess;
     if (!ok) {
         release(g);
@@ -1088,6 +1135,7 @@ extern "C" ftv_status ftv_segmenter_init(const ftv_segmenter_config* cfg, ftv_se
     }
     s.img = g->d_img;
     s.barrier = reinterpret_cast<uint32_t*>(s.cnt + 2 * g->rounds + 5);
+    s.work = s.cnt + 3 * g->rounds + 8;
     s.n_images = g->n_images;
     s.tiles = (int32_t)tiles;
     s.ctiles = (int32_t)ctiles;
@@ -1187,7 +1235,7 @@ extern "C" ftv_status ftv_superpixels(ftv_segmenter* g, const void* const* d_pla
     Scratch& s = g->sc;
     cudaError_t e = cudaMemcpyAsync(g->d_img, g->h_img, sizeof(SegImage) * g->n_images, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaEventRecord(g->staged, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(s.cnt, 0, sizeof(int32_t) * (3 * g->rounds + 8), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(s.cnt, 0, sizeof(int32_t) * counters(g->rounds), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(s.sums[0], 0, sizeof(Sums) * (size_t)g->K, st);
     if (e != cudaSuccess) {
         if (prev >= 0 && prev != g->device) cudaSetDevice(prev);

@@ -38,3 +38,17 @@ def test_tilings_equal_the_oracle(sizes, bits, step, compactness, iters):
         for v, o in zip(views, out):
             assert np.array_equal(o.cpu().numpy(), oracle.superpixels(v, sb, bits, step, compactness, iters))
     sg.close()
+
+
+def test_an_image_of_noise_large_enough_to_draw_turns():
+    """5.3 million pixels of noise: nearly every pixel is its own component, the lists and tile loops of the merge are long
+    enough for the drawn turns."""
+    w, h = 2636, 2011
+    rng = np.random.default_rng(6)
+    view = synth.View(*(rng.integers(0, 256, (h, w)).astype(np.uint8) for _ in range(3)))
+    sg = ftv.Segmenter([(w, h)], 1, 8, 12, 0, 1)
+    out = [torch.full((h, w), -3, dtype=torch.int32, device="cuda")]
+    ftv.ftv_superpixels(sg, [tuple(dev(a) for a in (view.Y, view.U, view.V))], out)
+    assert ftv.ftv_segmenter_check(sg) == 0
+    assert np.array_equal(out[0].cpu().numpy(), oracle.superpixels(view, 1, 8, 12, 0, 1))
+    sg.close()
