@@ -27,7 +27,7 @@
 // regions_kernel, one cooperative launch that links the tiles, sums the components, picks every label's main component,
 // runs the merge rounds (round 0 over every pixel, later rounds over the pixels of unanchored groups that still
 // touched another group, a list that shrinks every round) and writes the labels.
-// 8 images of 1920x1080, 10 passes: 4.28 -> 2.66 ms; one of 480x270: 0.55 -> 0.27 ms, 113 launches -> 12.
+// 8 images of 1920x1080, 10 passes: 4.28 -> 2.47 ms; one of 480x270: 0.55 -> 0.26 ms, 113 launches -> 12.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
