@@ -153,7 +153,8 @@ __device__ void scan_counts(const int32_t* __restrict__ in, int n, int32_t* out,
         *mx = max(*mx, c[k]);
     }
     int all;
-    int p = block_exclusive_scan(sum, &all) + s_before;  // its barriers order the additions to s_before
+    int p = block_exclusive_scan(sum, &all);
+    p += s_before;  // a statement of its own: the scan's barriers come between the additions to s_before and this read
 #pragma unroll
     for (int k = 0; k < kScanPer; ++k) {
         sm[at(threadIdx.x * kScanPer + k)] = p;
