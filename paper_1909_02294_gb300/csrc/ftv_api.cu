@@ -317,6 +317,7 @@ ftv_status ftv_depth_init(const ftv_config* cfg, ftv_ctx** out) {
     c->fast_rcp = fast_reciprocal_exact();
     c->penalty_floor = (int64_t)c->penalty >= max_sample_cost(c);
     c->cost_blocks_per_sm = cost_blocks_per_sm(c->cost_fmt, c->combine, c->fast_rcp);
+    ok = ok && finish_setup() == cudaSuccess;
     if (!ok) {
         free_ctx(c);
         return FTV_ERR_CUDA;

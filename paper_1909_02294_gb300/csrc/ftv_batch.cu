@@ -681,6 +681,7 @@ ftv_status ftv_stream_init(ftv_ctx* ctx, const int32_t* const* d_labels, const i
             ok = cudaMemcpyAsync(R.d_labels, d_labels[i], sizeof(int32_t) * (size_t)r.W * r.H, cudaMemcpyDeviceToDevice,
                                  s) == cudaSuccess;
     }
+    ok = ok && finish_setup() == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         free_stream_state(ctx);
@@ -894,6 +895,7 @@ ftv_status ftv_batch_create(int32_t max_jobs, int32_t max_units, int32_t max_vie
     ok = ok && cudaMemset(b->d_job_status, 0, sizeof(uint32_t) * max_jobs) == cudaSuccess;
     ok = ok && cudaMallocHost(reinterpret_cast<void**>(&b->h_job_status), sizeof(uint32_t) * max_jobs) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming) == cudaSuccess;
+    ok = ok && finish_setup() == cudaSuccess;
     if (ok) {
         std::memset(b->h_stage, 0, b->lay.total);
         std::memset(b->h_job_status, 0, sizeof(uint32_t) * max_jobs);

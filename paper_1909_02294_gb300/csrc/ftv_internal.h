@@ -190,6 +190,10 @@ struct ftv_ctx {
 
 namespace ftv {
 
+// Waits for the clears and uploads that setting up an object queued on the legacy default stream: a non-blocking stream
+// is not ordered after it, and its first launch reads them (the plan's ticket has to be zero).
+inline cudaError_t finish_setup() { return cudaStreamSynchronize(cudaStreamLegacy); }
+
 // ftv_api.cu
 struct IndexRef;
 IndexRef index_ref(const ftv_ctx* c, int ref, const int32_t* labels, int n_segments);

@@ -1128,6 +1128,7 @@ extern "C" ftv_status ftv_segmenter_init(const ftv_segmenter_config* cfg, ftv_se
          dalloc(g, &s.dirty_list, P);
     ok = ok && dalloc(g, &s.cnt, counters(g->rounds)) && dalloc(g, &s.status, 1);
     ok = ok && cudaMemset(s.status, 0, sizeof(uint32_t)) == cudaSuccess;
+    ok = ok && ftv::finish_setup() == cudaSuccess;
     if (!ok) {
         release(g);
         cudaGetLastError();
