@@ -1177,7 +1177,9 @@ extern "C" ftv_status ftv_segmenter_init(const ftv_segmenter_config* cfg, ftv_se
     s.PY = (g->S + s.G - 1) / s.G;
     s.packed = g->bd <= 10;
     // shared memory of an assignment tile: the cells it can see (kAGroups consecutive groups, from a multiple of
-    // kAGroups, touch at most ceil((kAGroups - 1) / G) + 1 cell rows), 52 bytes each
+    // kAGroups, touch at most ceil((kAGroups - 1) / G) + 1 cell rows), 52 bytes each. At most 66 x 6 cells (step 1), 20.6
+    // KB: below what every launch may ask for, so that no limit is set. A limit would belong to the kernel, and the
+    // next segmenter's would replace it.
     {
         // One group per thread while the tiles of kAGroups would not give every SM a few warps: 480x270, 10 passes,
         // 72 against 125 us; 8 x 1920x1080, 1300 against 1010 us.
@@ -1188,12 +1190,6 @@ extern "C" ftv_status ftv_segmenter_init(const ftv_segmenter_config* cfg, ftv_se
         const int ncx = (kATileW - 1 + g->S - 1) / g->S + 3, ncy = (g->groups - 1 + s.G - 1) / s.G + 3;
         s.max_cells = ncx * ncy;
         g->assign_smem = (size_t)s.max_cells * (2 * sizeof(int4) + 5 * sizeof(uint32_t));
-        const cudaError_t e = cudaFuncSetAttribute(assign_function(g->dist_mode, g->sb, g->groups),
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->assign_smem);
-        if (e != cudaSuccess) {
-            release(g);
-            return FTV_ERR_CUDA;
-        }
     }
     *out = g;
     return FTV_OK;
