@@ -46,7 +46,7 @@ typedef enum ftv_status {
     FTV_ERR_OUT_OF_MEMORY = 2, /* device allocation failed */
     FTV_ERR_CUDA = 3,          /* a CUDA runtime call failed */
     FTV_ERR_OVERFLOW = 4,      /* a segment is large enough that its int32 cost sum could overflow */
-    FTV_ERR_TIMEOUT = 5,       /* reserved: a bounded device wait gave up */
+    FTV_ERR_TIMEOUT = 5,       /* a bounded device-side wait gave up */
     FTV_ERR_BUSY = 6,          /* batch admission refused: over the HBM budget or out of slots */
     FTV_ERR_STATE = 7,         /* call out of order (e.g. no segment index built yet) */
     FTV_ERR_CHECKED = 8        /* checked builds (FTV_CHECKED) only: a cost-kernel gather index fell outside
@@ -547,6 +547,12 @@ FTV_API ftv_status ftv_superpixels(ftv_segmenter* sg, const void* const* d_plane
 /* Wait for `stream`, then return and clear the segmenter's device status word (FTV_OK if clean,
  * FTV_ERR_TIMEOUT if a bounded loop gave up). */
 FTV_API ftv_status ftv_segmenter_check(ftv_segmenter* sg, ftv_stream stream);
+
+/* Bound of the waits inside this segmenter's later ftv_superpixels calls: the blocks of its last kernel wait for one
+ * another between phases, and one that has polled `polls` times without the others arriving gives up, on which the
+ * kernel ends early, the label maps are left incomplete and ftv_segmenter_check answers FTV_ERR_TIMEOUT. 0 restores
+ * the default (2^23 polls, seconds). FTV_ERR_INVALID_ARG for a negative value. */
+FTV_API ftv_status ftv_segmenter_set_poll_limit(ftv_segmenter* sg, int32_t polls);
 
 /* Kernel launches this segmenter has enqueued since creation. */
 FTV_API int64_t ftv_segmenter_launch_count(const ftv_segmenter* sg);

@@ -109,6 +109,7 @@ struct Scratch {
     uint32_t* barrier;            // arrivals at the grid barriers of regions_kernel (cleared with cnt)
     int32_t* work;                // [2 phases] items drawn from for_items (cleared with cnt)
     uint32_t* status;
+    int32_t polls;                // bound of the grid barriers' waits
     int32_t n_images, tiles, ctiles;  // images, and pixel tiles and component tiles of all of them
     int64_t pixels;
     int32_t S, sb, rounds, max_cells;
@@ -638,10 +639,10 @@ __device__ void unite_groups(Scratch& s, int32_t a, int32_t b) {
 }
 
 // A barrier of the whole grid (a cooperative launch: every CTA is resident). Arrivals count up; `phase` is the number
-// of barriers passed. Waits a bounded number of polls (seconds), then reports SP_BARRIER and returns false, on which
-// every CTA leaves the kernel.
-constexpr int kBarrierPolls = 1 << 23;
-
+// of barriers passed. Waits at most s.polls polls, then reports SP_BARRIER and returns false, on which the CTA leaves
+// the kernel. The others may still pass this barrier, but not the next one, where its arrival is missing: no CTA ever
+// works on a phase before every CTA has finished the one before it.
+constexpr int kBarrierPolls = 1 << 23;  // seconds
 
 __device__ bool grid_barrier(const Scratch& s, uint32_t& phase) {
     __shared__ int s_ok;
@@ -652,9 +653,9 @@ __device__ bool grid_barrier(const Scratch& s, uint32_t& phase) {
         atomicAdd(s.barrier, 1u);
         const uint32_t target = phase * gridDim.x;
         int polls = 0;
-        while (*reinterpret_cast<volatile uint32_t*>(s.barrier) < target && ++polls < kBarrierPolls) {
+        while (*reinterpret_cast<volatile uint32_t*>(s.barrier) < target && ++polls < s.polls) {
         }
-        s_ok = polls < kBarrierPolls;
+        s_ok = polls < s.polls;
         if (!s_ok) atomicOr(s.status, SP_BARRIER);
         __threadfence();
     }
@@ -1137,6 +1138,7 @@ extern "C" ftv_status ftv_segmenter_init(const ftv_segmenter_config* cfg, ftv_se
     s.img = g->d_img;
     s.barrier = reinterpret_cast<uint32_t*>(s.cnt + 2 * g->rounds + 5);
     s.work = s.cnt + 3 * g->rounds + 8;
+    s.polls = kBarrierPolls;
     s.n_images = g->n_images;
     s.tiles = (int32_t)tiles;
     s.ctiles = (int32_t)ctiles;
@@ -1275,6 +1277,12 @@ extern "C" ftv_status ftv_segmenter_check(ftv_segmenter* g, ftv_stream stream) {
     if (cudaMemcpy(&st, g->sc.status, sizeof(st), cudaMemcpyDeviceToHost) != cudaSuccess) return FTV_ERR_CUDA;
     if (st && cudaMemset(g->sc.status, 0, sizeof(st)) != cudaSuccess) return FTV_ERR_CUDA;
     return st ? FTV_ERR_TIMEOUT : FTV_OK;
+}
+
+extern "C" ftv_status ftv_segmenter_set_poll_limit(ftv_segmenter* g, int32_t polls) {
+    if (!g || polls < 0) return FTV_ERR_INVALID_ARG;
+    g->sc.polls = polls > 0 ? polls : kBarrierPolls;
+    return FTV_OK;
 }
 
 extern "C" int64_t ftv_segmenter_launch_count(const ftv_segmenter* g) { return g ? g->launches : 0; }

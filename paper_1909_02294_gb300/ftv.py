@@ -117,6 +117,7 @@ def _load() -> ctypes.CDLL:
         "ftv_superpixels": [vp, vp, vp, vp, vp],
         "ftv_segmenter_check": [vp, vp],
         "ftv_segmenter_destroy": [vp],
+        "ftv_segmenter_set_poll_limit": [vp, i32],
         "ftv_segmenter_set_profiling": [vp, i32],
         "ftv_segmenter_kernel_ms": [vp, vp, vp],
     }
@@ -149,7 +150,7 @@ EXPORTED = ["ftv_depth_init", "ftv_depth_destroy", "ftv_compute_homographies", "
             "ftv_job_footprint", "ftv_batch_set_budget", "ftv_batch_submit", "ftv_batch_flush", "ftv_batch_poll",
             "ftv_segmenter_init", "ftv_segmenter_segments", "ftv_superpixels", "ftv_segmenter_check",
             "ftv_segmenter_launch_count", "ftv_segmenter_destroy", "ftv_segmenter_set_profiling",
-            "ftv_segmenter_kernel_ms"]
+            "ftv_segmenter_kernel_ms", "ftv_segmenter_set_poll_limit"]
 
 
 def _ok(code: int, where: str) -> None:
@@ -736,6 +737,11 @@ def ftv_superpixels(sg: Segmenter, planes, labels, stream=None) -> None:
 def ftv_segmenter_check(sg: Segmenter, stream=None) -> int:
     """Wait for the stream and return the segmenter's device status code (0 = clean)."""
     return int(lib.ftv_segmenter_check(sg.handle, _stream(stream)))
+
+
+def ftv_segmenter_set_poll_limit(sg: Segmenter, polls: int) -> None:
+    """Bound of the waits inside later ftv_superpixels calls (0: the default)."""
+    _ok(lib.ftv_segmenter_set_poll_limit(sg.handle, polls), "ftv_segmenter_set_poll_limit")
 
 
 def ftv_segmenter_launch_count(sg: Segmenter) -> int:
