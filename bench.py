@@ -144,14 +144,14 @@ def _traffic_for_current_kernel(workload_key: str, table: str = "cost_kernel_tra
     return None
 
 
-def algorithmic_bytes(wl, culled: int = 0) -> tuple[int, int]:
+def algorithmic_bytes(wl, skipped: int = 0) -> tuple[int, int]:
     """Per cost-volume launch: (evaluation bytes, compulsory bytes). One sampled evaluation reads one
     3-sample texel of the neighbour view (3 x sample_bytes); evaluations the kernel decided without
-    sampling (a whole tile out of a neighbour's view, ftv_culled_evaluations) read nothing. Compulsory
+    sampling (a whole tile out of a neighbour's view, ftv_skipped_evaluations) read nothing. Compulsory
     streams are every packed view read once, each reference pixel's index record and reference texel,
     and the int32 volume written once."""
     sb = wl.sample_bytes
-    evals = wl.evaluations() - culled
+    evals = wl.evaluations() - skipped
     comp = 0
     for v in range(wl.n_views):
         c = wl.cams[v]
@@ -171,10 +171,10 @@ OPS_PER_EVAL = 25
 OPS_PER_PIXEL_LABEL = 1
 
 
-def algorithmic_ops(wl, culled: int = 0) -> int:
-    """Per cost-volume launch; a culled evaluation (decided without sampling) is not charged."""
+def algorithmic_ops(wl, skipped: int = 0) -> int:
+    """Per cost-volume launch; an evaluation decided without sampling is not charged."""
     px_labels = sum(wl.cams[r].width * wl.cams[r].height * wl.n_labels for r in wl.ref_views)
-    return (wl.evaluations() - culled) * OPS_PER_EVAL + px_labels * OPS_PER_PIXEL_LABEL
+    return (wl.evaluations() - skipped) * OPS_PER_EVAL + px_labels * OPS_PER_PIXEL_LABEL
 
 
 def _oracle_table(wl, r, nb, fp64: bool):
@@ -752,7 +752,8 @@ def main():
             kernel_ms.append(ftv.ftv_last_kernel_ms(ctx))
         torch.cuda.synchronize()
     launches = ftv.ftv_launch_count(ctx) - launches0
-    culled = ftv.ftv_culled_evaluations(ctx)  # the same for every step (the last launch's count)
+    culled = ftv.ftv_culled_evaluations(ctx)  # of the last launch (every step's are alike)
+    skipped = ftv.ftv_skipped_evaluations(ctx)
     recomputed = ftv.ftv_fp64_recomputed(ctx)
     if world > 1:
         dist.barrier()
@@ -815,7 +816,7 @@ def main():
 
     if rank == 0:
         peak, peak_kind = _peaks()
-        ev_bytes, comp_bytes = algorithmic_bytes(wl, culled)
+        ev_bytes, comp_bytes = algorithmic_bytes(wl, skipped)
         kms = statistics.mean(kernel_ms)
         achieved = (ev_bytes + comp_bytes) / (kms / 1000.0) / 1e9
         traffic = _traffic_for_current_kernel(args.workload + ("_fp64" if fp64 else ""))
@@ -825,7 +826,7 @@ def main():
         n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
         sm_mhz = clk["sm_mhz"] if clk else 2070.0
         alu_peak = n_sm * 128 * sm_mhz * 1e6 / 1e12  # lane operations per second, Tops/s
-        alu_achieved = algorithmic_ops(wl, culled) / (kms / 1000.0) / 1e12
+        alu_achieved = algorithmic_ops(wl, skipped) / (kms / 1000.0) / 1e12
         line = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": 1000 * total_s / args.steps, "higher_is_better": True,
@@ -835,6 +836,7 @@ def main():
                        "depth_maps_per_s": whole_job_rate(world, R * args.steps, total_s),
                        "cost_kernel_ms": kms, "evaluations_per_step": evals,
                        "culled_evaluations_per_step": culled, "culled_fraction": culled / evals,
+                       "skipped_evaluations_per_step": skipped, "skipped_fraction": skipped / evals,
                        "precision": "FP64 projection" if fp64 else "FP32 contract",
                        "launch_shape": {"label_block": shape_now["label_block"],
                                         "ctas_per_sm": shape_now["ctas_per_sm"], "chosen_by": shape_rec["source"],
@@ -844,7 +846,7 @@ def main():
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind,
                          "algorithmic_bytes_per_launch": ev_bytes + comp_bytes,
-                         "definition": "one 3-sample texel (3 x sample bytes) per sampled evaluation (culled "
+                         "definition": "one 3-sample texel (3 x sample bytes) per sampled evaluation (skipped "
                                        "ones read nothing) + compulsory streams, over the cost kernel's "
                                        "event-timed duration",
                          "kernel": "cost_kernel<FMT_P10, MIN" + (", FP64 projection>" if fp64 else ">"),
@@ -859,7 +861,7 @@ def main():
             "alu_roofline": {"bound": "alu", "achieved": alu_achieved, "peak": alu_peak, "unit": "Tops/s",
                              "frac": alu_achieved / alu_peak,
                              "peak_kind": f"{n_sm} SMs x 128 lanes x {sm_mhz:.0f} MHz (median sampled SM clock)",
-                             "algorithmic_ops_per_launch": algorithmic_ops(wl, culled),
+                             "algorithmic_ops_per_launch": algorithmic_ops(wl, skipped),
                              "ops_per_evaluation": OPS_PER_EVAL},
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                     "steps": n_e2e, "overlap": "step k+1's uploads on a second stream during step k (two input sets)"},

@@ -574,14 +574,22 @@ FTV_API ftv_status ftv_segmenter_destroy(ftv_segmenter* sg);
 FTV_API ftv_status ftv_check(ftv_ctx* ctx, ftv_stream stream);
 
 /* Wait for `stream`, then report in *culled how many pixel x label x neighbour evaluations of the context's
- * most recent ftv_cost_volume call were decided without sampling. The cost kernel bounds each tile of
- * pixels by its box and tests every (neighbour, label) homography against the neighbour view at the
+ * most recent ftv_cost_volume call the corner test decided without sampling. The cost kernel bounds each tile of
+ * pixels by its box and tests every projective (neighbour, label) homography against the neighbour view at the
  * box's corners, with a margin that covers the FP32 contract's rounding at every pixel of the box; when
  * no pixel can land inside the view, every one of those samples costs the out-of-view penalty, which is
  * what the kernel then applies (under the minimum with a penalty of at least 3 (2^bit_depth - 1), the
- * default, that changes nothing). Results are identical with and without this; the count is for
- * accounting (a roofline that charges only the samples taken). */
+ * default, that changes nothing). Under the FP32 contract affine entries take no part in this test (a rectified
+ * rig's count is 0), under the FP64 projection whole-number shifts take none.
+ * ftv_skipped_evaluations counts every evaluation that was decided for a whole tile. */
 FTV_API ftv_status ftv_culled_evaluations(ftv_ctx* ctx, ftv_stream stream, int64_t* culled);
+
+/* Wait for `stream`, then report in *skipped how many evaluations of the context's most recent ftv_cost_volume call
+ * were decided for a whole tile of pixels at once, without a test or a sample per pixel: the culled ones, those of
+ * whole-number shifts (rectified rigs) that move every column of the tile out of the view, and those of affine
+ * entries whose Wz is not positive. Results are identical with and without this; the count is for accounting (a
+ * roofline that charges only the samples taken). */
+FTV_API ftv_status ftv_skipped_evaluations(ftv_ctx* ctx, ftv_stream stream, int64_t* skipped);
 
 /* Wait for `stream`, then report in *recomputed how many evaluations of the context's most recent
  * ftv_cost_volume call (FTV_PRECISION_FP64 contexts) were computed in double precision: those whose

@@ -627,6 +627,15 @@ ftv_status ftv_culled_evaluations(ftv_ctx* ctx, ftv_stream stream, int64_t* cull
     return FTV_OK;
 }
 
+ftv_status ftv_skipped_evaluations(ftv_ctx* ctx, ftv_stream stream, int64_t* skipped) {
+    if (!ctx || !skipped) return FTV_ERR_INVALID_ARG;
+    if (cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) return FTV_ERR_CUDA;
+    unsigned long long v = 0;
+    if (cudaMemcpy(&v, &ctx->d_plan->skipped, sizeof(v), cudaMemcpyDeviceToHost) != cudaSuccess) return FTV_ERR_CUDA;
+    *skipped = (int64_t)v;
+    return FTV_OK;
+}
+
 ftv_status ftv_check(ftv_ctx* ctx, ftv_stream stream) {
     if (!ctx) return FTV_ERR_INVALID_ARG;
     DeviceGuard g(ctx->device);

@@ -340,6 +340,7 @@ __device__ void plan_block(const RefJob& J, RefJob* out, int u, int n_jobs, int 
         for (int k = 0; k < kMaxChunks; ++k) plan->counter[k] = 0;
         plan->n_jobs = n_jobs;
         plan->culled = 0;
+        plan->skipped = 0;
         plan->recomputed = 0;
         plan->checked = 0;
         plan->ticket = 0;

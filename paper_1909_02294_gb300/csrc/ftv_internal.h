@@ -92,7 +92,8 @@ struct Plan {
     int32_t total_tiles;
     int32_t ticket;            // blocks of the plan kernel that have finished (zero between launches)
     int32_t n_jobs;            // units in the launch
-    unsigned long long culled; // evaluations decided without sampling: the tile is out of that view
+    unsigned long long culled; // evaluations decided by the corner test (box_class, stage_precise) for a whole tile
+    unsigned long long skipped;  // those and the other entries no pixel of the tile visits (integer shifts, Wz <= 0)
     unsigned long long recomputed;  // FP64-precision evaluations computed in double precision
     uint32_t checked;          // checked builds: ST_CHECKED when a gather index fell outside its view
     int32_t counter[kMaxChunks];  // next item of each chunk, relative to the chunk's first (persistent CTAs)

@@ -79,6 +79,7 @@ def _load() -> ctypes.CDLL:
         "ftv_wta_depth": [vp, i32, vp, i32, vp, vp, vp, vp, vp, vp, vp, vp, vp],
         "ftv_check": [vp, vp],
         "ftv_culled_evaluations": [vp, vp, vp],
+        "ftv_skipped_evaluations": [vp, vp, vp],
         "ftv_fp64_recomputed": [vp, vp, vp],
         "ftv_set_launch_shape": [vp, i32, i32],
         "ftv_get_launch_shape": [vp, vp, vp, vp, vp],
@@ -142,7 +143,7 @@ EXPORTED = ["ftv_depth_init", "ftv_depth_destroy", "ftv_compute_homographies", "
             "ftv_get_homographies_f64", "ftv_compute_homographies_f64", "ftv_fp64_recomputed", "ftv_set_launch_shape", "ftv_get_launch_shape",
             "ftv_autotune", "ftv_get_neighbours",
             "ftv_get_label_depths", "ftv_segment_index", "ftv_cost_volume", "ftv_temporal_mask", "ftv_temporal_mask_views",
-            "ftv_wta_depth", "ftv_check", "ftv_culled_evaluations", "ftv_launch_count", "ftv_status_str", "ftv_set_profiling",
+            "ftv_wta_depth", "ftv_check", "ftv_culled_evaluations", "ftv_skipped_evaluations", "ftv_launch_count", "ftv_status_str", "ftv_set_profiling",
             "ftv_last_kernel_ms", "ftv_temporal_mask_static", "ftv_stream_init", "ftv_stream_footprint",
             "ftv_stream_labels", "ftv_stream_mask", "ftv_stream_changed", "ftv_stream_state_bytes", "ftv_stream_state_save",
             "ftv_stream_state_load", "ftv_reciprocal_check", "ftv_centre_table", "ftv_adjacency", "ftv_batch_create", "ftv_batch_destroy", "ftv_batch_prepare", "ftv_batch_launch",
@@ -415,10 +416,18 @@ def ftv_check(ctx: Context, stream=None) -> int:
 
 
 def ftv_culled_evaluations(ctx: Context, stream=None) -> int:
-    """Evaluations of the most recent ftv_cost_volume call decided without sampling (whole tile out of
-    a neighbour's view); waits for the stream."""
+    """Evaluations of the most recent ftv_cost_volume call that the corner test decided without sampling (whole
+    tile out of a neighbour's view, projective entries); waits for the stream."""
     n = ctypes.c_int64()
     _ok(lib.ftv_culled_evaluations(ctx.handle, _stream(stream), ctypes.byref(n)), "ftv_culled_evaluations")
+    return int(n.value)
+
+
+def ftv_skipped_evaluations(ctx: Context, stream=None) -> int:
+    """Evaluations of the most recent ftv_cost_volume call decided for a whole tile at once: the culled ones and those
+    of affine entries that no pixel of the tile samples; waits for the stream."""
+    n = ctypes.c_int64()
+    _ok(lib.ftv_skipped_evaluations(ctx.handle, _stream(stream), ctypes.byref(n)), "ftv_skipped_evaluations")
     return int(n.value)
 
 
