@@ -617,7 +617,9 @@ bool any_affine_entry(const ftv_config* cfg) {
         for (int k = b; k < e; ++k) {
             const int v = cfg->nbr_offsets ? (cfg->nbr_views ? cfg->nbr_views[k] : r) : k;
             if (v == r || v < 0 || v >= cfg->n_views) continue;
-            for (int d = 0; d < cfg->n_labels; ++d) {
+            int begin, end;
+            affine_labels(cfg->cams[r], cfg->cams[v], cc, iz, &begin, &end);
+            for (int d = begin; d < end; ++d) {
                 double H[9];
                 if (plane_homography(cfg->cams[r], cfg->cams[v], cc, iz[d], H) != 0) continue;
                 if ((float)H[6] == 0.0f && (float)H[7] == 0.0f) return true;

@@ -7,6 +7,7 @@
 // homography H = K_v (R_vr + t_vr n^T / delta) K_r^-1 with R_vr = R_v R_r^T, t_vr = t_v - R_vr t_r.
 // The operation order below is fixed (and documented in ftv.h) so that the FP32 rounding of each
 // entry is reproducible by any implementation that follows the same order.
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -97,6 +98,43 @@ int plane_homography(const ftv_camera& cr, const ftv_camera& cv, const ftv_camer
     mul33(M, Kinv, T);
     mul33(cv.K, T, H);
     return 0;
+}
+
+// The labels [*begin, *end) among which an affine homography of a pair has to be, if it has one (third row (0, 0, .) in
+// FP32). The row's first two entries come from m = p + q w with p = (R_vr[6], R_vr[7]), q = t_vr[2] (n[0], n[1]) and w
+// the label's inverse plane distance: H[6] = m[0] / fx, H[7] = m[0] K_r^-1[1] + m[1] / fy. With the reference's own
+// planes q is zero, so every label has the first one's row. With the centre camera's, m has to cancel to below 2^-109
+// (FP32 holds 2^-149, focal lengths are below 2^30, the skew is below 2^10 of them), which an entry of p above 2^-80
+// does only where the plane distance is -q / p within 2^-28; the labels around it are returned. Looking at these labels
+// instead of all: 15 views, 400 labels 2470 us -> 17 (centre planes 5640 -> 10), 32 views, 1000 labels 28 ms -> 65 us (67 ms -> 54).
+void affine_labels(const ftv_camera& cr, const ftv_camera& cv, const ftv_camera* cc, const std::vector<double>& iz, int* begin,
+                   int* end) {
+    *begin = 0;
+    *end = 1;
+    if (cc == nullptr) return;
+    *end = (int)iz.size();
+    double R[3], n[3];
+    for (int j = 0; j < 3; ++j) {
+        R[j] = dot3(cv.R[6], cr.R[j * 3 + 0], cv.R[7], cr.R[j * 3 + 1], cv.R[8], cr.R[j * 3 + 2]);
+        n[j] = dot3(cr.R[j * 3 + 0], cc->R[6], cr.R[j * 3 + 1], cc->R[7], cr.R[j * 3 + 2], cc->R[8]);
+    }
+    const int k = std::fabs(R[0]) >= std::fabs(R[1]) ? 0 : 1;
+    if (!(std::fabs(R[k]) > 0x1p-80 && std::fabs(cr.K[0]) < 0x1p30 && std::fabs(cr.K[4]) < 0x1p30 &&
+          std::fabs(cr.K[1]) < 0x1p10 * std::fabs(cr.K[0])))
+        return;
+    const double t = cv.t[2] - dot3(R[0], cr.t[0], R[1], cr.t[1], R[2], cr.t[2]);
+    const double delta = -(t * n[k]) / R[k], c = dot3(n[0], cr.t[0], n[1], cr.t[1], n[2], cr.t[2]);
+    const double z = (delta - c) + cc->t[2];
+    const double err = 0x1p-20 * (std::fabs(delta) + std::fabs(n[0] * cr.t[0]) + std::fabs(n[1] * cr.t[1]) +
+                                  std::fabs(n[2] * cr.t[2]) + std::fabs(cc->t[2]));
+    if (!(std::fabs(z) + err < 0x1p100)) return;
+    if (z + err <= 0.0) {
+        *end = 0;
+        return;
+    }
+    const double lo = (1.0 - 0x1p-20) / (z + err);
+    *begin = (int)(std::lower_bound(iz.begin(), iz.end(), lo) - iz.begin());
+    if (z - err > 0.0) *end = (int)(std::upper_bound(iz.begin(), iz.end(), (1.0 + 0x1p-20) / (z - err)) - iz.begin());
 }
 
 }  // namespace ftv

@@ -213,6 +213,8 @@ void free_stream_state(ftv_ctx* c);
 
 // Host geometry (ftv_geometry.cpp)
 bool label_inv_depths(int L, double z_near, double z_far, std::vector<double>& iz);
+void affine_labels(const ftv_camera& cr, const ftv_camera& cv, const ftv_camera* cc, const std::vector<double>& iz, int* begin,
+                   int* end);
 int plane_homography(const ftv_camera& cr, const ftv_camera& cv, const ftv_camera* cc, double iz, double H[9]);
 
 // Launchers (ftv_index.cu). Descriptors travel as kernel parameters (graph-capturable, no host staging buffer to
