@@ -122,6 +122,10 @@ typedef struct ftv_config {
 /*
  * Create a context: validates the configuration, forms every homography (below), allocates the
  * device scratch and uploads the table. Synchronous. On success *out receives the context.
+ * Device memory, as ftv_job_footprint counts it: packed views, 4 bytes per view pixel, or 8 for samples of more than 10
+ * bits and for 2-byte samples of up to 14 bits of a rig with neighbours but no affine homography; per reference pixel
+ * 4 bytes of segment index and 8 of the cost kernel's records (16 more per 1024 pixels); the homography tables; and
+ * 136 bytes per segment of max_segments and 84 more for each reference.
  *
  * Candidate inverse depths (Sec. IV-A): a = 1/z_far, b = 1/z_near, step = (b - a)/(L - 1),
  * iz_d = a + d * step (FP64). Plane homography of Eq. 4's transform T[.] from reference r into view v

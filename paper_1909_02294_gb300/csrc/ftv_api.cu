@@ -245,7 +245,7 @@ ftv_status ftv_depth_init(const ftv_config* cfg, ftv_ctx** out) {
     // Classify the entries the way the cost kernel's staging does: projective-only when no entry has
     // h6 = h7 = 0, so that no entry takes an affine or rectified path.
     {
-        bool any_affine = false;
+        bool any_affine = max_n == 0;
         for (const auto& r : c->refs)
             for (size_t e = 0; e < r.h_H.size(); e += 9) any_affine = any_affine || (r.h_H[e + 6] == 0.0f && r.h_H[e + 7] == 0.0f);
         c->kind = any_affine ? kKindMixed : kKindProjective;

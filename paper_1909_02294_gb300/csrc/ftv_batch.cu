@@ -605,18 +605,20 @@ int64_t job_bytes(const ftv_ctx* c) {
            stream_bytes_of(packed, refs, c->L) + input;
 }
 
-// Whether any homography of cfg is affine (as FP32), which decides the cost kernel's texel format.
+// Whether any homography of cfg is affine (as FP32), or there is none, which decides the cost kernel's texel format.
 bool any_affine_entry(const ftv_config* cfg) {
     std::vector<double> iz;
     if (!label_inv_depths(cfg->n_labels, cfg->z_near, cfg->z_far, iz)) return false;
     const bool centre = cfg->plane_mode == FTV_PLANES_CENTRE && cfg->centre_view >= 0 && cfg->centre_view < cfg->n_views;
     const ftv_camera* cc = centre ? &cfg->cams[cfg->centre_view] : nullptr;
+    bool none = true;
     for (int i = 0; i < cfg->n_refs; ++i) {
         const int r = cfg->ref_views[i];
         const int b = cfg->nbr_offsets ? cfg->nbr_offsets[i] : 0, e = cfg->nbr_offsets ? cfg->nbr_offsets[i + 1] : cfg->n_views;
         for (int k = b; k < e; ++k) {
             const int v = cfg->nbr_offsets ? (cfg->nbr_views ? cfg->nbr_views[k] : r) : k;
             if (v == r || v < 0 || v >= cfg->n_views) continue;
+            none = false;
             int begin, end;
             affine_labels(cfg->cams[r], cfg->cams[v], cc, iz, &begin, &end);
             for (int d = begin; d < end; ++d) {
@@ -626,7 +628,7 @@ bool any_affine_entry(const ftv_config* cfg) {
             }
         }
     }
-    return false;
+    return none;
 }
 
 }  // namespace

@@ -202,7 +202,8 @@ NbrView nbr_view(const ftv_ctx* c, int v, void* base, size_t offset, size_t texe
 // Texel format of the cost kernel's views. Projective rigs take FMT_U16S where the samples allow it: its cost is
 // four instructions instead of seven, and the projection leaves the L1 room for 8-byte texels (3840x2160 15-view
 // rig: 435 against 479 ms per volume with FMT_P10). Rigs with affine entries keep 4-byte texels: there the gathers
-// are most of the work (1920x1080 8-view rig: 20.0 against 21.2 ms).
+// are most of the work (1920x1080 8-view rig: 20.0 against 21.2 ms); so does a context without neighbours, which
+// gathers nothing (any_affine is then true).
 inline int cost_format(bool any_affine, int sample_bytes, int bit_depth, int fmt) {
     return !any_affine && sample_bytes == 2 && bit_depth <= 14 ? FMT_U16S : fmt;
 }

@@ -69,3 +69,9 @@ def _check(ftv, cams, centre, lists=None):
     pad = lambda b: (b + 255) & ~255
     wide = 0 if affine else len(cams) * (pad(W * H * 8) - pad(W * H * 4))
     assert _bytes(ftv, cams, lists, mode, centre or 0) == base + wide
+
+
+def test_context_without_neighbours_takes_the_smaller_texels(ftv):
+    arc = synth.arc_rig(3, 3.0, 8.0, 64.0, W, H, seed=1)
+    lin = synth.linear_rig(3, 0.1, 64.0, W, H)
+    assert _bytes(ftv, arc, [[], [], []]) == _bytes(ftv, lin, [[], [], []])
