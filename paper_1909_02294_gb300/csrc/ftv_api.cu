@@ -46,17 +46,14 @@ void free_ctx(ftv_ctx* c) {
         cudaFree(r.d_H);
         cudaFree(r.d_H64);
         cudaFree(r.d_nbrs);
-        cudaFree(r.d_offs);
-        cudaFree(r.d_recs);
-        cudaFree(r.d_tiles);
-        cudaFree(r.d_cursor);
         cudaFree(r.d_pix);
         cudaFree(r.d_centre);
         cudaFree(r.d_nbr_labels);
     }
     cudaFree(c->d_packed);
     cudaFree(c->d_status);
-    cudaFree(c->d_woffs_all);
+    cudaFree(c->d_index);
+    cudaFree(c->d_records);
     cudaFree(c->d_jobs);
     cudaFree(c->d_plan);
     cudaFree(c->d_tstats);
@@ -272,22 +269,29 @@ ftv_status ftv_depth_init(const ftv_config* cfg, ftv_ctx** out) {
     ok = ok && dalloc(&c->d_status, 1) == cudaSuccess;
     ok = ok && dalloc(&c->d_jobs, kMaxUnits) == cudaSuccess;
     ok = ok && dalloc(&c->d_plan, 1) == cudaSuccess && cudaMemset(c->d_plan, 0, sizeof(Plan)) == cudaSuccess;
-    ok = ok && dalloc(&c->d_woffs_all, (size_t)c->n_refs * ((size_t)c->max_segments + 1)) == cudaSuccess;
+    const size_t per_ref = (size_t)c->max_segments + 1;
+    ok = ok && dalloc(&c->d_index, 3 * (size_t)c->n_refs * per_ref) == cudaSuccess;
     ok = ok && dalloc(&c->d_tstats, (size_t)std::max(1, c->n_refs) * c->max_segments * 8) == cudaSuccess;
     c->tstats_zero.assign(c->n_refs, 0);
     ok = ok && dalloc(&c->d_label_z, (size_t)c->L) == cudaSuccess;
     ok = ok && dalloc(&c->d_adj_deg, (size_t)c->max_segments) == cudaSuccess;
     ok = ok && dalloc(&c->d_adj_slots, (size_t)c->max_segments * 32) == cudaSuccess;
     ok = ok && dalloc(&c->d_adj_offs, (size_t)c->max_segments) == cudaSuccess;
+    int64_t tiles = 0, at = 0;
+    for (const auto& r : c->refs) tiles += tiles_of((int64_t)r.W * r.H);
+    static_assert(kTile * sizeof(int2) % sizeof(int4) == 0, "a tile's records in units of int4");
+    ok = ok && dalloc(&c->d_records, (size_t)tiles * (1 + kTile * sizeof(int2) / sizeof(int4))) == cudaSuccess;
     for (auto& r : c->refs) {
+        if (!ok) break;
         ok = ok && dalloc(&r.d_H, r.h_H.size()) == cudaSuccess;
         if (c->precision == FTV_PRECISION_FP64) ok = ok && dalloc(&r.d_H64, r.h_H64.size()) == cudaSuccess;
         ok = ok && dalloc(&r.d_nbrs, (size_t)r.n_nbrs * 2) == cudaSuccess;
-        ok = ok && dalloc(&r.d_offs, (size_t)c->max_segments + 1) == cudaSuccess;
-        ok = ok && dalloc(&r.d_cursor, (size_t)c->max_segments) == cudaSuccess;
-        ok = ok && dalloc(&r.d_recs, (size_t)tiles_of((int64_t)r.W * r.H) * kTile) == cudaSuccess;
-        ok = ok && dalloc(&r.d_tiles, (size_t)tiles_of((int64_t)r.W * r.H)) == cudaSuccess;
-        r.d_woffs = c->d_woffs_all ? c->d_woffs_all + (&r - c->refs.data()) * ((size_t)c->max_segments + 1) : nullptr;
+        r.d_tiles = c->d_records + at;
+        r.d_recs = reinterpret_cast<int2*>(c->d_records + tiles) + at * kTile;
+        at += tiles_of((int64_t)r.W * r.H);
+        r.d_woffs = c->d_index + (&r - c->refs.data()) * per_ref;
+        r.d_offs = r.d_woffs + c->n_refs * per_ref;
+        r.d_cursor = r.d_offs + c->n_refs * per_ref;
         ok = ok && dalloc(&r.d_pix, (size_t)r.W * r.H) == cudaSuccess;
         ok = ok && dalloc(&r.d_centre, (size_t)c->max_segments) == cudaSuccess;
         ok = ok && dalloc(&r.d_nbr_labels, (size_t)std::max(1, r.n_nbrs)) == cudaSuccess;

@@ -571,7 +571,7 @@ int64_t context_bytes_of(size_t packed, const std::vector<RefDims>& refs, int64_
     b += std::max<int64_t>(1, (int64_t)refs.size()) * MS * 8 * 8 + L * 4 + MS * 4 + MS * 32 * 4 + MS * 4;
     for (const RefDims& r : refs) {
         b += r.N * L * 9 * 4 + (fp64 ? r.N * L * 9 * 8 : 0) + 2 * r.N * (int64_t)sizeof(NbrView);
-        b += 2 * (MS + 1) * 4 + MS * 4 + r.W * r.H * 4 + MS * 8 + std::max<int64_t>(1, r.N) * 8;
+        b += 3 * (MS + 1) * 4 + r.W * r.H * 4 + MS * 8 + std::max<int64_t>(1, r.N) * 8;
         b += tiles_of(r.W * r.H) * (int64_t)(kTile * sizeof(int2) + sizeof(int4));
     }
     return b;

@@ -107,11 +107,11 @@ struct RefState {
     float* d_H = nullptr;      // [N][L][9]
     double* d_H64 = nullptr;   // [N][L][9] unrounded table (FP64-precision contexts only)
     NbrView* d_nbrs = nullptr; // [2][N]: views packed in cost_fmt, then in fmt (both in the context's d_packed)
-    int32_t* d_offs = nullptr;   // [max_segments + 1]
-    int32_t* d_cursor = nullptr; // [max_segments]
-    int2* d_recs = nullptr;      // [tiles * kTile] tile records
-    int4* d_tiles = nullptr;     // [tiles]
-    int32_t* d_woffs = nullptr;  // [max_segments + 1], in the context's d_woffs_all; also the index's counts
+    int32_t* d_offs = nullptr;   // [max_segments + 1], d_cursor and d_woffs likewise: in the context's d_index
+    int32_t* d_cursor = nullptr;
+    int32_t* d_woffs = nullptr;  // also the index's counts
+    int2* d_recs = nullptr;      // [tiles * kTile] tile records, and
+    int4* d_tiles = nullptr;     // [tiles]: in the context's d_records
     uint32_t* d_pix = nullptr;   // [W * H]
     int32_t S_indexed = -1;      // segment count of the cached index (-1: none)
     int2* d_centre = nullptr;    // [max_segments] segment centres (centre table)
@@ -173,7 +173,9 @@ struct ftv_ctx {
     std::vector<size_t> cost_offset_bytes;    // byte offset of each view packed in cost_fmt
     size_t cost_texel_bytes = 4;
     uint32_t* d_status = nullptr;
-    int32_t* d_woffs_all = nullptr;           // [n_refs][max_segments + 1]
+    // One allocation for what every reference has (each one costs a creation about 10 us):
+    int32_t* d_index = nullptr;               // [3][n_refs][max_segments + 1]: counts, offsets, cursors
+    int4* d_records = nullptr;                // every reference's d_tiles, then every one's d_recs
     ftv::RefJob* d_jobs = nullptr;            // [n_refs]
     ftv::Plan* d_plan = nullptr;
     int64_t* d_tstats = nullptr;              // per reference: temporal sums, 8 planes of max_segments (adjacency scratch)
