@@ -286,7 +286,7 @@ __device__ __forceinline__ int centre_field(const Scratch& s, const SegImage& im
 // strict comparison ignores.
 // Bound by instruction issue (about seven per candidate and pixel): 101 us per pass over eight 1920x1080 images, where
 // four horizontal pixels per thread, each with its own candidates, took 280 instructions per pixel and 184 us.
-template <int DM, int SB, int AG>
+template <int DM, int SB, int AG, int ROWS>
 __global__ void __launch_bounds__(kATileW) assign_kernel(Scratch s, int pass, int accumulate, int last) {
     extern __shared__ __align__(16) unsigned char smem[];
     const SegImage& im = s.img[blockIdx.z];
@@ -355,10 +355,10 @@ __global__ void __launch_bounds__(kATileW) assign_kernel(Scratch s, int pass, in
         for (int g = 0; g < AG && cj < gh; ++g) {
             const int ya = cj * S + gi * PY, rows = min(min(PY, S - gi * PY), H - ya);
             if (rows > 0) {
-                int v0[kPY], v1[kPY], v2[kPY], be[kPY];
-                typename Dist<DM>::T bd[kPY];
+                int v0[ROWS], v1[ROWS], v2[ROWS], be[ROWS];
+                typename Dist<DM>::T bd[ROWS];
 #pragma unroll
-                for (int r = 0; r < kPY; ++r) {
+                for (int r = 0; r < ROWS; ++r) {
                     const bool in = r < rows;
                     v0[r] = in ? load(0, ya + r) : 0;
                     v1[r] = in ? load(1, ya + r) : 0;
@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(kATileW) assign_kernel(Scratch s, int pass, in
                     int t = 0;
                     if (DM == DIST_DOT32) t = a.x + (x - x0) * a.y + (ya - y0) * a.z;
 #pragma unroll
-                    for (int r = 0; r < kPY; ++r) {
+                    for (int r = 0; r < ROWS; ++r) {
                         typename Dist<DM>::T D;
                         if (DM == DIST_DOT32) {
                             D = (typename Dist<DM>::T)(t + v0[r] * a.w + v1[r] * b.x + v2[r] * b.y);
@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(kATileW) assign_kernel(Scratch s, int pass, in
                 }
                 if (last) {
 #pragma unroll
-                    for (int r = 0; r < kPY; ++r)
+                    for (int r = 0; r < ROWS; ++r)
                         if (r < rows) {
                             const int bj = be[r] / ncx;
                             const int64_t gp = (int64_t)im.pix_base + (int64_t)(ya + r) * W + x;
@@ -401,14 +401,14 @@ __global__ void __launch_bounds__(kATileW) assign_kernel(Scratch s, int pass, in
                 if (accumulate) {
                     uint32_t n = 0, q0 = 0, q1 = 0, q2 = 0, qy = 0;
 #pragma unroll
-                    for (int r = 0; r < kPY; ++r) {
+                    for (int r = 0; r < ROWS; ++r) {
                         if (r < rows) {
                             n += 1;
                             q0 += v0[r];
                             q1 += v1[r];
                             q2 += v2[r];
                             qy += ya + r - y0;
-                            if (r + 1 >= rows || be[r + 1 < kPY ? r + 1 : r] != be[r]) {
+                            if (r + 1 >= rows || be[r + 1 < ROWS ? r + 1 : r] != be[r]) {
                                 // a tile has at most 64 x 20 pixels, so that n < 2^11, the relative y sum < 2^15 and the
                                 // relative x sum < 2^17; at 10 bits a colour sum is below 2^21
                                 const int e = be[r];
@@ -1035,20 +1035,23 @@ void release(ftv_segmenter* g) {
     delete g;
 }
 
-template <int D>
-const void* assign_function_of(int sb, int groups) {
-    if (groups == 1)
-        return sb == 1 ? reinterpret_cast<const void*>(assign_kernel<D, 1, 1>) : reinterpret_cast<const void*>(assign_kernel<D, 2, 1>);
-    return sb == 1 ? reinterpret_cast<const void*>(assign_kernel<D, 1, kAGroups>)
-                   : reinterpret_cast<const void*>(assign_kernel<D, 2, kAGroups>);
+// The rows of a group are compiled in: with five for all, steps of one and two pixels leave most of a thread's
+// comparisons unused (8 images of 1920x1080, 12 bits, 10 passes: step 1 17.9 -> 13.7 ms, step 2 7.9 -> 5.3). Images small enough
+// for one group per thread wait on the chain of passes instead and keep the one form.
+template <int D, int SB>
+const void* assign_function_of(int groups, int rows) {
+    if (groups == 1) return reinterpret_cast<const void*>(assign_kernel<D, SB, 1, kPY>);
+    if (rows == 1) return reinterpret_cast<const void*>(assign_kernel<D, SB, kAGroups, 1>);
+    if (rows == 2) return reinterpret_cast<const void*>(assign_kernel<D, SB, kAGroups, 2>);
+    return reinterpret_cast<const void*>(assign_kernel<D, SB, kAGroups, kPY>);
 }
 
-const void* assign_function(int dist_mode, int sb, int groups) {
+const void* assign_function(int dist_mode, int sb, int groups, int rows) {
     switch (dist_mode) {
-        case DIST_DOT32: return assign_function_of<DIST_DOT32>(sb, groups);
-        case DIST_NARROW: return assign_function_of<DIST_NARROW>(sb, groups);
-        case DIST_WIDE: return assign_function_of<DIST_WIDE>(sb, groups);
-        default: return assign_function_of<DIST_WIDE_COLOUR>(sb, groups);
+        case DIST_DOT32: return sb == 1 ? assign_function_of<DIST_DOT32, 1>(groups, rows) : assign_function_of<DIST_DOT32, 2>(groups, rows);
+        case DIST_NARROW: return sb == 1 ? assign_function_of<DIST_NARROW, 1>(groups, rows) : assign_function_of<DIST_NARROW, 2>(groups, rows);
+        case DIST_WIDE: return sb == 1 ? assign_function_of<DIST_WIDE, 1>(groups, rows) : assign_function_of<DIST_WIDE, 2>(groups, rows);
+        default: return sb == 1 ? assign_function_of<DIST_WIDE_COLOUR, 1>(groups, rows) : assign_function_of<DIST_WIDE_COLOUR, 2>(groups, rows);
     }
 }
 
@@ -1251,7 +1254,7 @@ extern "C" ftv_status ftv_superpixels(ftv_segmenter* g, const void* const* d_pla
         if (prof) cudaEventRecord(g->ev[2 + 2 * it], st);
         int pass = it, add = acc, end = last;
         void* args[] = {&s, &pass, &add, &end};
-        e = cudaLaunchKernel(assign_function(g->dist_mode, g->sb, g->groups), agrid, dim3(kATileW), args, g->assign_smem, st);
+        e = cudaLaunchKernel(assign_function(g->dist_mode, g->sb, g->groups, s.PY), agrid, dim3(kATileW), args, g->assign_smem, st);
         if (prof) cudaEventRecord(g->ev[3 + 2 * it], st);
         ++n;
     }
