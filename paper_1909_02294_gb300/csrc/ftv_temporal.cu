@@ -40,9 +40,14 @@ __device__ __forceinline__ void add64(int64_t* dst, int v) {
 // B pixels differ in label adds them one by one. At the end each non-empty bin is added to the segment's 64-bit sums,
 // once per tile. All sums are exact integers, so the order of the additions does not change the result. Tile bins are
 // 32-bit: a tile has 1024 pixels of differences below 2^16.
+// Segments of fewer than three pixels on average take the columns of a strip 32 apart (STEP): nearly every pixel is a run
+// of its own then and goes to global memory, where a warp's additions of four columns each touch four times the
+// sectors. Four 960x540 references of one-pixel segments: adjacent columns 129 us, 32 apart 105; of 2 x 2 pixel ones 98
+// and 106 (L2 flushed).
 // Single columns took 61 instructions per pixel and 127 us for eight 1920x1080 references; the strips take 72, of which
 // the bytes need 54. Two rows per thread and six CTAs per SM: the loads of a strip are all in flight at once, so that
-// more rows cost warps (four rows 107 us; four CTAs 80, eight 76).
+// more rows cost warps (four rows 107 us; four CTAs 80, eight 76; all measured on three planes with an I frame. Luma
+// alone gains little: eight 1920x1080 references with an I frame and a flushed L2 135 -> 131 us).
 constexpr int kAccCols = 128;      // pixels per tile row
 constexpr int kStrips = kAccCols / 4;
 constexpr int kAccRows = 2;        // rows per thread
@@ -56,8 +61,8 @@ struct TemporalRefs {
     TemporalRef r[kMaxTemporalRefs];
 };
 
-// Four adjacent samples of a row, packed in 16-bit lanes; n of them lie in the view (the rest repeat the last).
-template <int SB, bool VEC>
+// Four samples of a row, STEP columns apart, packed in 16-bit lanes; n of them lie in the view (the rest repeat the last).
+template <int SB, bool VEC, int STEP>
 __device__ __forceinline__ uint2 load_strip(const char* p, int n) {
     if constexpr (VEC && SB == 2) {
         return __ldg(reinterpret_cast<const uint2*>(p));
@@ -67,7 +72,7 @@ __device__ __forceinline__ uint2 load_strip(const char* p, int n) {
     } else {
         uint32_t v[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = (uint32_t)load_sample<SB>(p + (int64_t)min(k, n - 1) * SB);
+        for (int k = 0; k < 4; ++k) v[k] = (uint32_t)load_sample<SB>(p + (int64_t)min(k, n - 1) * (STEP * SB));
         return make_uint2(v[0] | (v[1] << 16), v[2] | (v[3] << 16));
     }
 }
@@ -80,7 +85,7 @@ __device__ __forceinline__ int strip_dot(const uint2& v, uint32_t weights, int c
     return d;
 }
 
-template <int SB, int NCH, bool HAS_I, bool VEC>
+template <int SB, int NCH, bool HAS_I, bool VEC, int STEP>
 __global__ void __launch_bounds__(kAccThreads, 6) temporal_accumulate_kernel(const __grid_constant__ TemporalRefs p,
                                                                           uint32_t* status) {
     constexpr int Q = 1 + NCH * (HAS_I ? 2 : 1);  // per segment: n, dP[NCH], dI[NCH]
@@ -91,12 +96,12 @@ __global__ void __launch_bounds__(kAccThreads, 6) temporal_accumulate_kernel(con
     if ((int)blockIdx.x * kAccCols >= W || (int)blockIdx.y * kAccRowsTile >= H) return;  // past this view
     int64_t* __restrict__ stats = f.stats;
     const int tid = threadIdx.x;
-    const int x = blockIdx.x * kAccCols + tid % kStrips * 4;
+    const int x = blockIdx.x * kAccCols + tid % kStrips * (STEP == 1 ? 4 : 1);  // columns x, x + STEP, ..
     const int y0 = blockIdx.y * kAccRowsTile + (tid / kStrips) * kAccRows;
     // Positions past the view's edge are clamped into it, so the loads need no branch, and those pixels are then
     // dropped through their label.
     // A vector load's strip is clamped as a whole: W is then a multiple of four.
-    const int xc = VEC ? min(x, W - 4) : min(x, W - 1), nx = min(4, W - xc), yc0 = min(y0, H - 1);
+    const int xc = VEC ? min(x, W - 4) : min(x, W - 1), nx = min(4, (W - xc + STEP - 1) / STEP), yc0 = min(y0, H - 1);
     int lab[kAccRows][4];
     uint2 a[kAccRows][NCH], b[kAccRows][NCH], e[kAccRows][HAS_I ? NCH : 1];
 #pragma unroll
@@ -111,13 +116,13 @@ __global__ void __launch_bounds__(kAccThreads, 6) temporal_accumulate_kernel(con
             lab[r][3] = t.w;
         } else {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) lab[r][k] = __ldg(pl + min(k, nx - 1));
+            for (int k = 0; k < 4; ++k) lab[r][k] = __ldg(pl + min(k, nx - 1) * STEP);
         }
 #pragma unroll
         for (int c = 0; c < NCH; ++c) {
-            a[r][c] = load_strip<SB, VEC>(static_cast<const char*>(f.cur[c]) + y * f.pc[c] + (int64_t)xc * SB, nx);
-            b[r][c] = load_strip<SB, VEC>(static_cast<const char*>(f.prev[c]) + y * f.pp[c] + (int64_t)xc * SB, nx);
-            if (HAS_I) e[r][c] = load_strip<SB, VEC>(static_cast<const char*>(f.ifr[c]) + y * f.pi[c] + (int64_t)xc * SB, nx);
+            a[r][c] = load_strip<SB, VEC, STEP>(static_cast<const char*>(f.cur[c]) + y * f.pc[c] + (int64_t)xc * SB, nx);
+            b[r][c] = load_strip<SB, VEC, STEP>(static_cast<const char*>(f.prev[c]) + y * f.pp[c] + (int64_t)xc * SB, nx);
+            if (HAS_I) e[r][c] = load_strip<SB, VEC, STEP>(static_cast<const char*>(f.ifr[c]) + y * f.pi[c] + (int64_t)xc * SB, nx);
         }
     }
     int lmin = INT_MAX, lmax = -1;
@@ -126,7 +131,7 @@ __global__ void __launch_bounds__(kAccThreads, 6) temporal_accumulate_kernel(con
     for (int r = 0; r < kAccRows; ++r)
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const bool in = x + k < W && y0 + r < H;
+            const bool in = x + k * STEP < W && y0 + r < H;
             if (in && (unsigned)lab[r][k] < (unsigned)S) {
                 lmin = min(lmin, lab[r][k]);
                 lmax = max(lmax, lab[r][k]);
@@ -389,7 +394,7 @@ cudaError_t launch_temporal_refs(const TemporalRef* refs, int n, int sample_byte
     if (n > kMaxTemporalRefs) return cudaErrorInvalidValue;
     TemporalRefs p{};
     int tx = 0, ty = 0, chunks = 1;
-    bool any_s = false, vec = true;
+    bool any_s = false, vec = true, fine = false;
     for (int k = 0; k < n; ++k) {
         p.r[k] = refs[k];
         tx = std::max(tx, (refs[k].W + kAccCols - 1) / kAccCols);
@@ -403,6 +408,7 @@ cudaError_t launch_temporal_refs(const TemporalRef* refs, int n, int sample_byte
             at |= u & (uintptr_t)(4 * sample_bytes - 1);
         }
         vec = vec && at == 0;
+        fine = fine || (int64_t)refs[k].S * 3 > (int64_t)refs[k].W * refs[k].H;
         chunks = std::max(chunks, (refs[k].S + kChunk - 1) / kChunk);
         any_s = any_s || refs[k].S > 0;
     }
@@ -410,8 +416,9 @@ cudaError_t launch_temporal_refs(const TemporalRef* refs, int n, int sample_byte
     if (tx > 0 && ty > 0) {
         const dim3 block(kAccThreads), grid(tx, ty, n);
 #define FTV_T(SB, NCH, HI) \
-    if (vec) temporal_accumulate_kernel<SB, NCH, HI, true><<<grid, block, 0, s>>>(p, status); \
-    else temporal_accumulate_kernel<SB, NCH, HI, false><<<grid, block, 0, s>>>(p, status)
+    if (fine) temporal_accumulate_kernel<SB, NCH, HI, false, kStrips><<<grid, block, 0, s>>>(p, status); \
+    else if (vec) temporal_accumulate_kernel<SB, NCH, HI, true, 1><<<grid, block, 0, s>>>(p, status); \
+    else temporal_accumulate_kernel<SB, NCH, HI, false, 1><<<grid, block, 0, s>>>(p, status)
         if (sample_bytes == 1) {
             if (nch == 1) { if (has_i) { FTV_T(1, 1, true); } else { FTV_T(1, 1, false); } }
             else { if (has_i) { FTV_T(1, 3, true); } else { FTV_T(1, 3, false); } }
