@@ -203,7 +203,8 @@ IndexRef index_ref(const ftv_ctx* c, int ref, const int32_t* labels, int n_segme
 NbrView nbr_view(const ftv_ctx* c, int v, void* base, size_t offset, size_t texel_bytes);
 // Texel format of the cost kernel's views. Projective rigs take FMT_U16S where the samples allow it: its cost is
 // four instructions instead of seven, and the projection leaves the L1 room for 8-byte texels (3840x2160 15-view
-// rig: 435 against 479 ms per volume with FMT_P10). Rigs with affine entries keep 4-byte texels: there the gathers
+// rig: 435 against 479 ms per volume with FMT_P10; with 2 neighbours, 1920x1080 and 250 labels 7.19 against 7.62, 960x540
+// alike, and 320x240 views 137 against 131 us, with 5 neighbours 319 against 295). Rigs with affine entries keep 4-byte texels: there the gathers
 // are most of the work (1920x1080 8-view rig: 20.0 against 21.2 ms); so does a context without neighbours, which
 // gathers nothing (any_affine is then true).
 inline int cost_format(bool any_affine, int sample_bytes, int bit_depth, int fmt) {
