@@ -1162,8 +1162,8 @@ extern "C" ftv_status ftv_segmenter_init(const ftv_segmenter_config* cfg, ftv_se
     // Distance arithmetic. |x - X| < 3S in pixels for every candidate (a candidate's pixels, hence its
     // mean, lie within one cell of the candidate's cell), so in 1/16 units dsp < 2 (48 S)^2, and
     // dcol <= 3 (16 (2^bd - 1))^2 for samples within the bit depth. In the DOT32 form positions are
-    // relative to the tile, |position| <= 16 (127 + 3S) = R, and every partial sum is bounded by
-    // wc' 3 vmax^2 + ws' 6 R^2.
+    // relative to the tile (64 columns, at most 20 rows and the one that the row term steps past them),
+    // |position| <= 16 (63 + 3S) = R, and every partial sum is bounded by wc' 3 vmax^2 + ws' 6 R^2.
     {
         const unsigned long long gcd = std::gcd(g->wc, g->ws);
         const unsigned long long wcn = g->wc / gcd, wsn = g->ws / gcd;
