@@ -59,12 +59,13 @@ def test_samples_next_to_a_boundary_are_left_to_fp64(monkeypatch, box, outside):
     tables = [[float(v) for v in table[0, d]] for d in range(table.shape[1])]
     counts = [rounding._check(h, W, H, *box) for h in tables]
     x0, y0 = (2 * box[0] + box[2] - 1) >> 1, (2 * box[1] + box[3] - 1) >> 1
-    modes = {stage32(h, x0, y0, box[2], box[3], W, H)[0] for h in tables}
+    rx, ry = max(x0 - box[0], box[0] + box[2] - 1 - x0), max(y0 - box[1], box[1] + box[3] - 1 - y0)
+    modes = {stage32(h, x0, y0, rx, ry, W, H)[0] for h in tables}
     if outside:
         assert modes == {"out"} and all(a == box[2] * box[3] for a, _ in counts)
     else:
-        assert modes - {"slow", "out"}  # the decision check is reached
-        assert sum(near for _, near in counts) > 0
+        assert modes == {"rect"}  # the decision check is reached
+        assert all(near == box[2] * box[3] for _, near in counts)
 
 
 @pytest.mark.parametrize("scale", [2.0 ** 140, 2.0 ** -140])
