@@ -22,17 +22,16 @@ constexpr unsigned kFull = 0xffffffffu;
 
 // ------------------------------------------------------------------------------------------ packing
 
-template <int CAP>
 struct PackArgs {
-    PackView v[CAP];
+    PackView v[FTV_MAX_VIEWS];
 };
 
 // Four adjacent pixels of a row per thread; blockIdx.y is the row, blockIdx.z the view. Samples above max_value
 // are reported and clamped so that they cannot spill into a neighbouring packed field. Memory-bound; a thread's
 // four samples of a plane come in one load and leave as one 16-byte store (or two) where the pointers, the
 // pitches and the width allow (every pixel of such a view then has 4-aligned company).
-template <int SB, int FMT, int CAP>
-__global__ void __launch_bounds__(128) pack_kernel(const __grid_constant__ PackArgs<CAP> args, uint32_t max_value,
+template <int SB, int FMT>
+__global__ void __launch_bounds__(128) pack_kernel(const __grid_constant__ PackArgs args, uint32_t max_value,
                                                    uint32_t* status) {
     const PackView& V = args.v[blockIdx.z];
     const int x = (blockIdx.x * blockDim.x + threadIdx.x) * 4, y = blockIdx.y;
@@ -49,9 +48,8 @@ __global__ void __launch_bounds__(128) pack_kernel(const __grid_constant__ PackA
 
 // ------------------------------------------------------------------------------------ segment index
 
-template <int CAP>
 struct IndexArgs {
-    IndexRef r[CAP];
+    IndexRef r[FTV_MAX_VIEWS];
 };
 
 // Four adjacent labels of a row (-1 past its end), in one load where the map allows.
@@ -74,8 +72,7 @@ __device__ __forceinline__ void load_labels(const IndexRef& R, int x, int y, int
 // those whose pixels all continue it, and the first one that continues it only in part.
 // Runs joined within a thread only took one addition per four pixels of a large segment, all at a few addresses: three
 // 961x541 maps of 8 segments each 223 us, this 12; of 60 px segments 8, of 10 px ones 5.
-template <int CAP>
-__global__ void __launch_bounds__(128) histogram_kernel(const __grid_constant__ IndexArgs<CAP> args, uint32_t* status) {
+__global__ void __launch_bounds__(128) histogram_kernel(const __grid_constant__ IndexArgs args, uint32_t* status) {
     const IndexRef& R = args.r[blockIdx.z];
     const int x = (blockIdx.x * blockDim.x + threadIdx.x) * 4, y = blockIdx.y, lane = threadIdx.x & 31;
     if (y >= R.H || x - 4 * lane >= R.W) return;  // uniform over the warp
@@ -108,34 +105,6 @@ __global__ void __launch_bounds__(128) histogram_kernel(const __grid_constant__ 
             mine = true;
         }
     }
-}
-
-// Block-wide exclusive scan of one int per thread (blockDim.x == 1024). Returns the exclusive prefix;
-// *total receives the block sum.
-__device__ int block_exclusive_scan(int v, int* total) {
-    __shared__ int warp_sums[32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = v;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += t;
-    }
-    if (lane == 31) warp_sums[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        const int nw = blockDim.x >> 5;
-        int s = lane < nw ? warp_sums[lane] : 0;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(kFull, s, o);
-            if (lane >= o) s += t;
-        }
-        warp_sums[lane] = s;  // inclusive prefix of warp sums
-    }
-    __syncthreads();
-    const int base = warp > 0 ? warp_sums[warp - 1] : 0;
-    *total = warp_sums[(blockDim.x >> 5) - 1];
-    __syncthreads();
-    return base + incl - v;
 }
 
 // Exclusive prefix of n counts by blocks of 1024, each of kScanChunk counts (eight consecutive ones per thread, read and
@@ -190,8 +159,7 @@ __device__ void scan_counts(const int32_t* __restrict__ in, int n, int32_t* out,
 
 // Counts -> offsets[S + 1]; cursor[s] = offsets[s] for the scatter. Also checks that no segment is large enough for its
 // int32 cost sum to overflow.
-template <int CAP>
-__global__ void __launch_bounds__(1024) offsets_kernel(const __grid_constant__ IndexArgs<CAP> args, uint32_t* status) {
+__global__ void __launch_bounds__(1024) offsets_kernel(const __grid_constant__ IndexArgs args, uint32_t* status) {
     const IndexRef& R = args.r[blockIdx.y];
     int mx = 0;
     scan_counts(R.counts, R.S, R.offs, R.cursor, R.offs + R.S, &mx);
@@ -208,8 +176,7 @@ __global__ void __launch_bounds__(1024) prefix_kernel(const int32_t* counts, int
 // its left-to-right order (the cost kernel's gathers follow this order: one atomic per run of a thread's four pixels
 // made it 3 % slower on the 1920x1080 rig). kScatterRows rows per warp, their atomics in flight together.
 constexpr int kScatterRows = 4;
-template <int CAP>
-__global__ void __launch_bounds__(256) scatter_kernel(const __grid_constant__ IndexArgs<CAP> args) {
+__global__ void __launch_bounds__(256) scatter_kernel(const __grid_constant__ IndexArgs args) {
     const IndexRef& R = args.r[blockIdx.z];
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y0 = blockIdx.y * kScatterRows;
     if (y0 >= R.H) return;
@@ -502,10 +469,9 @@ __global__ void __launch_bounds__(kTileThreads) tile_kernel(const RefJob* __rest
 
 cudaError_t launch_pack(const PackView* views, int n, int sample_bytes, int bit_depth, int fmt, uint32_t* status,
                         cudaStream_t s, int64_t* launches) {
-    constexpr int kCap = FTV_MAX_VIEWS;
     if (n <= 0) return cudaSuccess;
-    if (n > kCap) return cudaErrorInvalidValue;
-    PackArgs<kCap> args;
+    if (n > FTV_MAX_VIEWS) return cudaErrorInvalidValue;
+    PackArgs args;
     int W = 0, H = 0;
     for (int k = 0; k < n; ++k) {
         PackView v = views[k];
@@ -520,19 +486,18 @@ cudaError_t launch_pack(const PackView* views, int n, int sample_bytes, int bit_
     if (W <= 0 || H <= 0) return cudaSuccess;
     const dim3 block(128), grid((W + 511) / 512, H, n);
     const uint32_t maxv = (1u << bit_depth) - 1u;
-    if (sample_bytes == 1) pack_kernel<1, FMT_U8X4, kCap><<<grid, block, 0, s>>>(args, maxv, status);
-    else if (fmt == FMT_P10) pack_kernel<2, FMT_P10, kCap><<<grid, block, 0, s>>>(args, maxv, status);
-    else if (fmt == FMT_U16S) pack_kernel<2, FMT_U16S, kCap><<<grid, block, 0, s>>>(args, maxv, status);
-    else pack_kernel<2, FMT_U16X4, kCap><<<grid, block, 0, s>>>(args, maxv, status);
+    if (sample_bytes == 1) pack_kernel<1, FMT_U8X4><<<grid, block, 0, s>>>(args, maxv, status);
+    else if (fmt == FMT_P10) pack_kernel<2, FMT_P10><<<grid, block, 0, s>>>(args, maxv, status);
+    else if (fmt == FMT_U16S) pack_kernel<2, FMT_U16S><<<grid, block, 0, s>>>(args, maxv, status);
+    else pack_kernel<2, FMT_U16X4><<<grid, block, 0, s>>>(args, maxv, status);
     *launches += 1;
     return cudaGetLastError();
 }
 
 cudaError_t launch_segment_index(const IndexRef* refs, int n, uint32_t* status, cudaStream_t s, int64_t* launches) {
-    constexpr int kCap = FTV_MAX_VIEWS;
     if (n <= 0) return cudaSuccess;
-    if (n > kCap) return cudaErrorInvalidValue;
-    IndexArgs<kCap> args;
+    if (n > FTV_MAX_VIEWS) return cudaErrorInvalidValue;
+    IndexArgs args;
     int W = 1, H = 1, S = 1;
     for (int k = 0; k < n; ++k) {
         args.r[k] = refs[k];
@@ -550,9 +515,9 @@ cudaError_t launch_segment_index(const IndexRef* refs, int n, uint32_t* status, 
         }
     }
     const dim3 block(128), grid((W + 511) / 512, H, n);
-    histogram_kernel<kCap><<<grid, block, 0, s>>>(args, status);
-    offsets_kernel<kCap><<<dim3((S + kScanChunk - 1) / kScanChunk, n), 1024, 0, s>>>(args, status);
-    scatter_kernel<kCap><<<dim3((W + 255) / 256, (H + kScatterRows - 1) / kScatterRows, n), 256, 0, s>>>(args);
+    histogram_kernel<<<grid, block, 0, s>>>(args, status);
+    offsets_kernel<<<dim3((S + kScanChunk - 1) / kScanChunk, n), 1024, 0, s>>>(args, status);
+    scatter_kernel<<<dim3((W + 255) / 256, (H + kScatterRows - 1) / kScatterRows, n), 256, 0, s>>>(args);
     *launches += 3;
     return cudaGetLastError();
 }

@@ -1,5 +1,5 @@
 // Device code shared by the kernels of one context and of a batch: strips of four adjacent pixels of a row (packing,
-// depth maps) and the least-cost label of a segment.
+// depth maps), the least-cost label of a segment and the block-wide scan.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -128,6 +128,34 @@ __device__ __forceinline__ int least_label(const int32_t* row, int L, int lane) 
     }
     const int least = __reduce_min_sync(0xffffffffu, v);
     return __reduce_min_sync(0xffffffffu, v == least ? at : INT_MAX);
+}
+
+// Block-wide exclusive scan of one int per thread (whole warps). Returns the exclusive prefix;
+// *total receives the block sum.
+__device__ inline int block_exclusive_scan(int v, int* total) {
+    __shared__ int warp_sums[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int incl = v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) warp_sums[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+        const int nw = blockDim.x >> 5;
+        int s = lane < nw ? warp_sums[lane] : 0;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += t;
+        }
+        warp_sums[lane] = s;  // inclusive prefix of warp sums
+    }
+    __syncthreads();
+    const int base = warp > 0 ? warp_sums[warp - 1] : 0;
+    *total = warp_sums[(blockDim.x >> 5) - 1];
+    __syncthreads();
+    return base + incl - v;
 }
 
 }  // namespace ftv

@@ -67,12 +67,12 @@ struct SegImage {
     int32_t pad;
 };
 
-struct alignas(32) Centre {
-    int x, y, c0, c1, c2, p0, p1, p2;
+struct alignas(32) Centre {  // one 32-byte sector each
+    int x, y, c0, c1, c2;
 };
 
 struct alignas(32) Sums {
-    uint32_t n, x, y, c0, c1, c2, p0, p1;
+    uint32_t n, x, y, c0, c1, c2;
 };
 
 struct alignas(32) GSum {
@@ -81,8 +81,7 @@ struct alignas(32) GSum {
 
 // counters: [4 + 2 rounds] tile components, [6 + 2 rounds + r] anchored groups that gained members in round r, [0]
 // components, [1 + r] unanchored groups at the start of round r (r = 0..rounds), which
-// is also the length of the round's list uroots, [2 + rounds + r] length of round r's pick list,
-// [3 + 2 rounds] unused
+// is also the length of the round's list uroots, [2 + rounds + r] length of round r's pick list (r = 0..rounds)
 struct Scratch {
     const SegImage* img;
     Centre* cen[2];               // [K] cluster means before an assignment pass, alternating between passes
@@ -231,15 +230,7 @@ struct Dist<DIST_DOT32> {
 template <int DM>
 __device__ __forceinline__ typename Dist<DM>::T distance(const int4 a, const int4 b, int vx, int vy, int w0, int w1,
                                                          int w2, const Scratch& s) {
-    if (DM == DIST_DOT32) {
-        int d = a.x;
-        d += vx * a.y;
-        d += vy * a.z;
-        d += w0 * a.w;
-        d += w1 * b.x;
-        d += w2 * b.y;
-        return d;
-    }
+    static_assert(DM != DIST_DOT32, "assign_kernel steps that form from row to row");
     const int dx = vx - a.x, dy = vy - a.y;
     const uint32_t dsp = (uint32_t)dx * (uint32_t)dx + (uint32_t)dy * (uint32_t)dy;
     const int d0 = w0 - a.z, d1 = w1 - a.w, d2 = w2 - b.x;
@@ -310,7 +301,7 @@ __global__ void __launch_bounds__(kATileW) assign_kernel(Scratch s, int pass, in
     __syncthreads();
     for (int e = tid; e < ncells; e += kATileW) {
         const int j = cy0 + e / ncx, i = cx0 + e % ncx;
-        const Centre c{(int)acc[e], (int)acc[MC + e], (int)acc[2 * MC + e], (int)acc[3 * MC + e], (int)acc[4 * MC + e], 0, 0, 0};
+        const Centre c{(int)acc[e], (int)acc[MC + e], (int)acc[2 * MC + e], (int)acc[3 * MC + e], (int)acc[4 * MC + e]};
         // the cell's own tile: its first group's rows, its first column
         if (j * G >= g0 && j * G < g0 + AG && i * S >= x0 && i * S < x0 + kATileW) {
             const int k = im.seg_base + j * im.gw + i;
@@ -377,7 +368,7 @@ __global__ void __launch_bounds__(kATileW) assign_kernel(Scratch s, int pass, in
 #pragma unroll
                     for (int r = 0; r < ROWS; ++r) {
                         typename Dist<DM>::T D;
-                        if (DM == DIST_DOT32) {
+                        if constexpr (DM == DIST_DOT32) {
                             D = (typename Dist<DM>::T)(t + v0[r] * a.w + v1[r] * b.x + v2[r] * b.y);
                             t += a.z;
                         } else {

@@ -252,32 +252,6 @@ __global__ void __launch_bounds__(kAccThreads, 6) temporal_accumulate_kernel(con
     }
 }
 
-__device__ int block_exclusive_scan(int v, int* total) {
-    __shared__ int warp_sums[32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = v;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += t;
-    }
-    if (lane == 31) warp_sums[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        const int nw = blockDim.x >> 5;
-        int s = lane < nw ? warp_sums[lane] : 0;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(kFull, s, o);
-            if (lane >= o) s += t;
-        }
-        warp_sums[lane] = s;
-    }
-    __syncthreads();
-    const int base = warp > 0 ? warp_sums[warp - 1] : 0;
-    *total = warp_sums[(blockDim.x >> 5) - 1];
-    __syncthreads();
-    return base + incl - v;
-}
-
 __device__ __forceinline__ int64_t abs64(int64_t v) { return v < 0 ? -v : v; }
 
 // The masks and the ordered list of changed segments, in two passes over blocks of kChunk segments.
