@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cost_kernel(const RefJob
     __shared__ const void* sBase[FTV_MAX_NBRS];
     __shared__ int sAcc[kSegAcc * kMaxLB];
     __shared__ int sWoffs[kSegAcc + 1];  // listed-pixel offsets of the tile's first segments
-    __shared__ int s_item, s_culled, s_skipped;
+    __shared__ int s_item, s_culled;
     __shared__ PEntry sP[precise_kind(KIND) ? kHEntries : 1];
     // per label the neighbours to visit, grouped by class (kOut entries are left out): the first group is kIn
     // (projective) or kShiftIn, whose texel offsets are listed in sShift instead
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cost_kernel(const RefJob
     const int n_jobs = *reinterpret_cast<volatile int*>(&plan->n_jobs);
     for (int i = tid; i < kSegAcc * kMaxLB; i += kThreads) sAcc[i] = 0;
 
-    if (tid == 0) s_culled = s_skipped = 0;
+    if (tid == 0) s_culled = 0;
     for (;;) {
         __syncthreads();
         if (tid == 0)
@@ -667,17 +667,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cost_kernel(const RefJob
             else if (g3) pos = c1 + c2 + __popc(m3 & lt);
             if (pos >= 0) sOrd[l * N + pos] = (uint8_t)lane;
             if (kShifts && g1) sShift[l * N + pos] = __float_as_int(E->h[0]) + __float_as_int(E->h[8]);
-            if (lane == 0) {
-                const int c3 = __popc(m3), out = N - c1 - c2 - c3;
-                sCnt[l] = c1 | (c2 << 8) | (c3 << 16);
-                if (out > 0) atomicAdd(&s_skipped, out);
-            }
+            if (lane == 0) sCnt[l] = c1 | (c2 << 8) | (__popc(m3) << 16);
         }
         __syncthreads();
-        if (tid == 0) {
-            if (s_skipped > 0) atomicAdd(&plan->skipped, (unsigned long long)s_skipped * (unsigned)(w1 - w0));
-            s_skipped = 0;
-        }
 
         for (int l = 0; l < LBa; ++l) {
             int m[kPPT];
@@ -916,6 +908,15 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cost_kernel(const RefJob
         }
         __syncthreads();
 
+        if (warp == kThreads / 32 - 1) {  // the entries that no pixel visited (the last warp has the fewest row slices)
+            int out = 0;
+            for (int l = lane; l < LBa; l += 32) {
+                const int cnt = sCnt[l];
+                out += N - (cnt & 0xff) - ((cnt >> 8) & 0xff) - (cnt >> 16);
+            }
+            out = __reduce_add_sync(kFull, out);
+            if (lane == 0 && out > 0) atomicAdd(&plan->skipped, (unsigned long long)out * (unsigned)(w1 - w0));
+        }
         // write the row slices of this tile's first segments
         const int nacc = nk > 0xffff ? 0 : min(nk, kSegAcc);
         for (int i = tid; i < nacc * LBa; i += kThreads) {
