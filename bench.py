@@ -144,22 +144,35 @@ def _traffic_for_current_kernel(workload_key: str, table: str = "cost_kernel_tra
     return None
 
 
-def algorithmic_bytes(wl, skipped: int = 0) -> tuple[int, int]:
+def texel_format(wl, ctx) -> tuple[str, int]:
+    """The cost kernel's texel format of a context of this workload, and its bytes: 8-byte texels for samples above 10
+    bits, and for 2-byte samples of a rig without affine homographies (its distance is cheaper)."""
+    import paper_1909_02294_gb300 as ftv
+    if wl.sample_bytes == 1:
+        return "FMT_U8X4", 4
+    tables = [ftv.ftv_get_homographies(ctx, i) for i in range(len(wl.ref_views))]
+    affine = any(bool(np.any((t[..., 6] == 0) & (t[..., 7] == 0))) for t in tables) or not any(t.size for t in tables)
+    if not affine and wl.bit_depth <= 14:
+        return "FMT_U16S", 8
+    return ("FMT_P10", 4) if wl.bit_depth <= 10 else ("FMT_U16X4", 8)
+
+
+def algorithmic_bytes(wl, texel: int, skipped: int = 0) -> tuple[int, int]:
     """Per cost-volume launch: (evaluation bytes, compulsory bytes). One sampled evaluation reads one
     3-sample texel of the neighbour view (3 x sample_bytes); evaluations the kernel decided without
     sampling (a whole tile out of a neighbour's view, ftv_skipped_evaluations) read nothing. Compulsory
-    streams are every packed view read once, each reference pixel's index record and reference texel,
-    and the int32 volume written once."""
+    streams are every packed view read once (texel bytes per pixel), each reference pixel's record (8 bytes) and
+    reference texel, and the int32 volume written once."""
     sb = wl.sample_bytes
     evals = wl.evaluations() - skipped
     comp = 0
     for v in range(wl.n_views):
         c = wl.cams[v]
-        comp += c.width * c.height * 4
+        comp += c.width * c.height * texel
     for r in wl.ref_views:
         c = wl.cams[r]
         S = wl.labels(r)[1]
-        comp += c.width * c.height * 8 + S * wl.n_labels * 4
+        comp += c.width * c.height * (8 + texel) + S * wl.n_labels * 4
     return evals * 3 * sb, comp
 
 
@@ -816,7 +829,8 @@ def main():
 
     if rank == 0:
         peak, peak_kind = _peaks()
-        ev_bytes, comp_bytes = algorithmic_bytes(wl, skipped)
+        fmt, texel = texel_format(wl, ctx)
+        ev_bytes, comp_bytes = algorithmic_bytes(wl, texel, skipped)
         kms = statistics.mean(kernel_ms)
         achieved = (ev_bytes + comp_bytes) / (kms / 1000.0) / 1e9
         traffic = _traffic_for_current_kernel(args.workload + ("_fp64" if fp64 else ""))
@@ -849,7 +863,7 @@ def main():
                          "definition": "one 3-sample texel (3 x sample bytes) per sampled evaluation (skipped "
                                        "ones read nothing) + compulsory streams, over the cost kernel's "
                                        "event-timed duration",
-                         "kernel": "cost_kernel<FMT_P10, MIN" + (", FP64 projection>" if fp64 else ">"),
+                         "kernel": f"cost_kernel<{fmt}, MIN" + (", FP64 projection>" if fp64 else ">"),
                          "compulsory_bytes_per_launch": comp_bytes,
                          "compulsory_floor_ms": comp_bytes / (peak * 1e9) * 1e3,
                          "dram_fraction_of_algorithmic": (traffic / (ev_bytes + comp_bytes)) if traffic else None,
