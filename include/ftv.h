@@ -327,7 +327,7 @@ typedef struct ftv_frame_job {
 /* Make ctx a stream: copies the label maps d_labels[r] (int32 [H][W], n_segments[r] segments each, kept
  * for the stream's life), builds their segment indexes and allocates the resident state. t_p, t_i,
  * mode: the temporal test of ftv_temporal_mask. The first frame of a stream must be FTV_FRAME_I.
- * Asynchronous on `stream` apart from the allocations. */
+ * Asynchronous on `stream` apart from the allocations and uploads, which wait for the default stream. */
 FTV_API ftv_status ftv_stream_init(ftv_ctx* ctx, const int32_t* const* d_labels, const int32_t* n_segments,
                                    int32_t t_p, int32_t t_i, int32_t mode, ftv_stream stream);
 

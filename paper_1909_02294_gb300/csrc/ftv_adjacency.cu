@@ -10,7 +10,7 @@
 //
 // Kernels: one warp per segment walks the segment's pixels (segment index), collects the labels t > s of
 // their neighbours in a small shared hash, sorts them and sums the segment's colour; a scan turns the
-// per-segment counts into edge offsets; one thread per segment writes its edges and weights.
+// per-segment counts into edge offsets; four threads per segment write its edges and weights.
 #include <cuda_runtime.h>
 #include <stdint.h>
 

@@ -326,9 +326,9 @@ __device__ __forceinline__ int window_sum(const uint32_t* t, const int4* ref) {
 // computed while the current window's nine gathers are in flight. Windows that touch an image border take
 // the checked loop. The reciprocal is the Newton-Raphson step where the start-up check found it exact.
 // An integer-shift entry (rectified rigs) is one addition instead of the projection. 1920x1080, 8 references x 250 labels
-// x 7 neighbours: 167 instructions per entry, 0.317 ms per reference and launch; writing the results contiguously
-// through shared memory (the output has the neighbours innermost, a warp's words lie N apart) relieved the L2 from 57 to
-// 15 % busy but took 204 instructions and 0.346 ms.
+// x 7 neighbours: 163 instructions per entry, 0.32 ms per reference and launch (ALU pipe 58 %, L1 data stage 56 %, issue
+// 54 %, L2 33 %); writing the results contiguously through shared memory (the output has the neighbours innermost, a
+// warp's words lie N apart) relieved the L2 but took 204 instructions and 0.346 ms.
 constexpr int kGroup = 16;
 static_assert(9 * kGroup <= kCentreThreads, "one stage sample per thread");
 
